@@ -116,6 +116,14 @@ thread_local std::string g_create_error;
 
 }  // namespace
 
+// Tile and thread shape of a context's resident launches (k_resident).
+struct ResPlan {
+  bool on = false;
+  int t = 0, nth = 0, slots = 0;         // tile bits, threads that own amplitudes, slots per thread
+  int np = 0, ng = 0, npart = 0, nbuf = 0;  // as in ResParams
+  int ncode = 0;
+};
+
 struct aqc_ctx {
   int device = 0, prec = 0, n = 0;
   uint64_t N = 0;
@@ -156,6 +164,8 @@ struct aqc_ctx {
   int relabel = 1;    // choose the qubit -> index-bit order that keeps flips inside layouts
   std::vector<int> perm;  // perm[q] = index bit of qubit q in the library's vectors
   bool permuted = false;  // perm is not the identity
+  ResPlan res;        // resident launches (res.on: the state's size and products allow them)
+  int sms = 0;        // multiprocessors of the device
   SlabParams slab;    // slab-ordered last passes of a PEC step (slab.n_slabs == 0: off)
   bool in_batch = false;  // batch members use per-CTA tiles only
 
@@ -250,6 +260,11 @@ struct DeviceGuard {
   }
 };
 
+// Largest sizes of resident launches: 128 tiles of 2^13 complex64 or 2^12 complex128 amplitudes,
+// one beside two partner buffers in a multiprocessor's shared memory.  (complex128 n = 20 on 256
+// tiles measured 182 us per step, on the layout passes 177 us: both at the FP64 rate.)
+constexpr int kResMaxN[2] = {19, 20};  // by precision
+
 uint32_t layout_mask(const Layout& L) {
   uint32_t m = L.c >= 32 ? 0xffffffffu : ((1u << L.c) - 1u);
   if (L.w > 0) m |= ((1u << L.w) - 1u) << L.h;
@@ -313,13 +328,19 @@ int to_library_order(aqc_ctx* c, void* dst, const void* src) { return permute_ga
 // library order -> qubit order: dst[z] = src[perm(z)]
 int to_qubit_order(aqc_ctx* c, void* dst, const void* src) { return permute_gather(c, dst, src, c->perm); }
 
+// Sizes that resident launches take (the default tiles; a context that asks for tiles of its own
+// gets them, and so does a batch member, whose steps run on the batch's tiles).
+bool resident_size(const aqc_ctx* c) {
+  return c->tile_bits == 0 && !c->in_batch && c->n <= kResMaxN[c->prec];
+}
+
 // Order that minimises the products (weighted by how many share a flip mask) that no layout
 // holds: deterministic local search over transpositions, kept only if strictly better than the
 // identity.
 std::vector<int> choose_order(const aqc_ctx* c) {
   std::vector<int> id(c->n);
   for (int q = 0; q < c->n; q++) id[q] = q;
-  if (!c->relabel || c->layouts.size() < 2) return id;
+  if (!c->relabel || c->layouts.size() < 2 || resident_size(c)) return id;
   std::vector<std::pair<uint32_t, int>> masks;  // distinct multi-bit flip masks with counts
   for (const TermH& th : c->terms) {
     if (__builtin_popcount(th.x) < 2) continue;
@@ -422,6 +443,72 @@ void plan_slabs(aqc_ctx* c) {
   S.spin_limit = 1u << 22;
   S.queue = c->d_sync;
   S.done = c->d_sync + 1;
+}
+
+// Shape of the resident launches and the order of their products (res_idx, res_part).
+void plan_resident(aqc_ctx* c) {
+  DevTables* t = c->h_tab;
+  c->res = ResPlan();
+  if (!resident_size(c)) return;
+  ResPlan R;
+  const int H = c->prec == AQC_C128 ? 1 : 2;
+  // One tile while a step on one CTA takes less than an exchange between several; then at most
+  // 128 tiles (one per multiprocessor) of at least 2^8 complex64 / 2^7 complex128 amplitudes.
+  // Microseconds per step (linear / nonlinear path): complex64 n = 9 on one tile 1.8 / 2.2, on two
+  // 3.0 / 3.2; n = 10 on one 2.6 / 3.5, on four 2.7 / 2.9; n = 12 with tiles of 2^7 3.5 / 3.9, 2^8
+  // 3.2 / 3.8, 2^10 3.6 / 4.5; n = 16 with 2^9 4.6 / 5.4, 2^11 5.3 / 9.1.  complex128 n = 7 on one
+  // tile 3.0 / 4.3, on two 3.6 / 4.8; n = 8 on one 4.6 / 6.5, on two 3.9 / 5.1.
+  const bool c128 = c->prec == AQC_C128;
+  R.t = c->n <= (c128 ? 7 : 9) ? c->n : std::max(c128 ? 7 : 8, c->n - 7);
+  const int slots_all = std::max(1, (1 << R.t) / H);
+  R.nth = std::max(32, std::min(kResMaxThreads, slots_all));
+  R.slots = std::max(1, slots_all / R.nth);
+  // products by partner tile: the bits they flip above t, the own tile (no such bit) first
+  const int total = t->flip_begin[t->n_layouts + 1];
+  auto plain = [&](const DevFlip& f) { return f.zm == 0 && !f.has2; };
+  auto hop = [&](const DevFlip& f) {
+    return f.has2 && f.zm == 0 && f.zm2 == f.x && (f.ipow2 & 3) == 2 && f.group2 == f.group && f.coef2 == f.coef &&
+           __builtin_popcount(f.x) == 2;
+  };
+  std::vector<uint32_t> hi(1, 0u);
+  for (int i = 0; i < total; i++) hi.push_back(t->flips[i].x >> R.t);
+  std::sort(hi.begin(), hi.end());
+  hi.erase(std::unique(hi.begin(), hi.end()), hi.end());
+  for (int i = 0; i < total; i++) R.np += plain(t->flips[i]) ? 1 : 0;
+  R.ng = total - R.np;
+  R.npart = (int)hi.size() - 1;
+  int np = 0, ng = 0;
+  for (size_t d = 0; d < hi.size(); d++) {
+    ResPartner& pt = t->res_part[d];
+    pt.hi = (uint16_t)hi[d];
+    for (int pass = 0; pass < 3; pass++) {  // X strings with real coefficients, hops, the rest
+      for (int i = 0; i < total; i++) {
+        const DevFlip& f = t->flips[i];
+        if ((f.x >> R.t) != hi[d] || pass != (plain(f) ? 0 : (hop(f) ? 1 : 2))) continue;
+        t->res_idx[pass == 0 ? np++ : R.np + ng++] = (uint16_t)i;
+      }
+      if (pass == 1) pt.hop_end = (uint16_t)ng;
+    }
+    pt.plain_end = (uint16_t)np;
+    pt.gen_end = (uint16_t)ng;
+  }
+  if (t->table_class >= 0) {
+    const DevClass& cl = t->classes[t->table_class];
+    R.ncode = (cl.pen == AQC_PEN_SQUARED ? 4 : 1) * (cl.end - cl.begin);
+  }
+  // as many partner buffers as fit (two at least, so that one fills while the other is read);
+  // products whose tables leave no room stay on the layout passes
+  R.nbuf = R.npart ? R.npart + (R.slots >= 4 ? 4 : 0) : 0;
+  auto bytes = [&]() { return resident_smem_bytes(c->prec, R.t, R.nbuf, R.np, R.ng, t->n_z, R.nth, false); };
+  while (R.nbuf > 2 && bytes() > 222 * 1024) R.nbuf--;
+  R.on = bytes() <= 222 * 1024;
+  c->res = R;
+}
+
+// The launches run resident: no option that selects another pass order, no clause-by-clause
+// sequence (its coefficients change shape with s).
+bool resident_on(const aqc_ctx* c) {
+  return c->res.on && !c->slab.n_slabs && c->turn_req == 0 && c->step_class < 0;
 }
 
 int build_tables(aqc_ctx* c) {
@@ -642,6 +729,7 @@ int build_tables(aqc_ctx* c) {
       t->classes[k] = C;
     }
   }
+  plan_resident(c);
   c->step_m = c->step_class >= 0 ? classes[c->step_class].end - classes[c->step_class].begin : 0;
   c->table_class = t->table_class;
   CUDA_TRY(c, cudaMemcpyAsync(c->d_tab, t, sizeof(DevTables), cudaMemcpyHostToDevice, c->stream));
@@ -765,6 +853,89 @@ ApplyParams base_params(aqc_ctx* c) {
   return p;
 }
 
+// Fields of a resident launch that do not depend on what it runs.
+ResParams resident_params(aqc_ctx* c) {
+  ResParams p;
+  memset(&p, 0, sizeof(p));
+  const ResPlan& R = c->res;
+  p.tab = c->d_tab;
+  p.n = c->n;
+  p.t = R.t;
+  p.np = R.np;
+  p.ng = R.ng;
+  p.npart = R.npart;
+  p.nbuf = R.nbuf;
+  p.ncode = R.ncode;
+  p.dcode = c->table_class >= 0 ? c->d_dcode : nullptr;
+  p.h = c->h;
+  p.flags = c->d_sync + 1;
+  p.ticket = c->d_sync;
+  p.partials = c->d_partials;
+  p.slots = c->d_slots;
+  return p;
+}
+
+int launch_resident_on(aqc_ctx* c, const ResParams& p) {
+  const int limit = c->grid_limit > 0 ? std::min(c->grid_limit, c->sms) : c->sms;
+  CUDA_TRY(c, launch_resident(c->prec, p, c->res.slots, c->res.nth, limit, c->n_z, c->stream));
+  c->launches++;
+  return AQC_OK;
+}
+
+// One evaluation alone: out = H src, or (out null) <src|H|src> into the result slots.
+int resident_single(aqc_ctx* c, const double w[3], const void* src, void* out) {
+  ResParams p = resident_params(c);
+  p.single = out ? 6 : 7;
+  p.evals = 1;
+  for (int g = 0; g < 3; g++) p.w[g] = w[g];
+  p.src = src;
+  p.xout[0] = p.xout[1] = out;
+  return launch_resident_on(c, p);
+}
+
+// n_rk Runge-Kutta steps from the current step on and then, with hist, the derivative history
+// and the first predictor; or n_pec predictor-corrector steps.  The host counters are the
+// caller's.  The predictor ends in the exchange vector written last, which becomes V_P.
+int resident_steps(aqc_ctx* c, int n_rk, bool hist, int n_pec) {
+  ResParams p = resident_params(c);
+  p.n_rk = n_rk;
+  p.hist = hist ? 1 : 0;
+  p.n_pec = n_pec;
+  p.evals = 4 * n_rk + p.hist + n_pec;
+  p.step0 = (int)(c->step & 3);
+  if (c->step >= 4) p.step0 += 4;  // ring slots of the steps before (index mod 4), as f_k with k > 3
+  double* w = p.w;
+  for (int r = 0; r < n_rk; r++) {
+    const double t = c->seg_t0 + (double)(c->step + r) * c->h;
+    for (int stage = 1; stage <= 4; stage++, w += 3)
+      sched_weights(c, stage == 1 ? t : (stage == 4 ? t + c->h : t + 0.5 * c->h), w);
+  }
+  if (hist) {
+    sched_weights(c, c->seg_t0 + 3.0 * c->h, w);
+    w += 3;
+  }
+  if (c->cur_wdev) {
+    p.wdev = c->cur_wdev;
+    p.wstride = kGraphStepWeights;
+  } else {
+    for (int j = 0; j < n_pec; j++, w += 3) sched_weights(c, c->seg_t0 + (double)(c->step + j + 1) * c->h, w);
+  }
+  p.src = n_pec ? c->vec[V_P] : c->vec[V_Y];
+  p.xout[0] = c->vec[V_Q];
+  p.xout[1] = c->vec[V_P];
+  p.y = c->vec[V_Y];
+  p.yout = c->adaptive && n_pec ? c->vec[V_ACC] : c->vec[V_Y];
+  for (int k = 0; k < 4; k++) p.f[k] = c->vec[V_F0 + k];
+  p.acc = c->vec[V_ACC];
+  p.ylo = c->ycomp && n_pec ? c->vec_save : nullptr;
+  c->q_ready = -1;
+  int rc = launch_resident_on(c, p);
+  if (rc) return rc;
+  if (p.evals & 1) std::swap(c->vec[V_P], c->vec[V_Q]);
+  c->evals += p.evals;
+  return AQC_OK;
+}
+
 // One evaluation of H(t) src over all layouts.  The strided layouts run first as partial sums
 // (the first one also adds the products no layout holds); the contiguous layout 0 runs last
 // with the mode epilogue, so the kernel touching the most vectors has the smallest page
@@ -772,6 +943,8 @@ ApplyParams base_params(aqc_ctx* c) {
 // With top >= 0, only the partial passes of layouts top .. 1 run (the first of them adds the
 // products no layout holds); the caller finishes the evaluation.
 int evaluate(aqc_ctx* c, const double w[3], const void* src, ApplyParams fin, void* partial_out, int top = -1) {
+  if (top < 0 && resident_on(c) && (fin.mode == MODE_PARTIAL || fin.mode == MODE_ENERGY))
+    return resident_single(c, w, src, fin.mode == MODE_PARTIAL ? partial_out : nullptr);
   c->q_ready = -1;  // the passes below overwrite q
   const int nl = (int)c->layouts.size();
   const int hi = top >= 0 ? top : nl - 1, lo = top >= 0 ? 1 : 0;
@@ -869,6 +1042,15 @@ int start_history(aqc_ctx* c) {
   c->launches++;
   if (c->ycomp)  // the PEC steps' low part of y starts at zero
     CUDA_TRY(c, cudaMemsetAsync(c->vec_save, 0, (size_t)c->N * c->amp, c->stream));
+  c->hist_ready = true;
+  return AQC_OK;
+}
+
+// The start-up on resident launches: n_rk Runge-Kutta steps and, with hist, what start_history does.
+int resident_start(aqc_ctx* c, int n_rk, bool hist) {
+  int rc = resident_steps(c, n_rk, hist, 0);
+  if (rc || !hist) return rc;
+  if (c->ycomp) CUDA_TRY(c, cudaMemsetAsync(c->vec_save, 0, (size_t)c->N * c->amp, c->stream));
   c->hist_ready = true;
   return AQC_OK;
 }
@@ -998,6 +1180,7 @@ int pec_step_turn(aqc_ctx* c, const ApplyParams& fin0, const double w[3]) {
 }
 
 int pec_step(aqc_ctx* c) {
+  if (resident_on(c)) return resident_steps(c, 0, false, 1);
   const int64_t n = c->step;
   double w[3];
   sched_weights(c, c->seg_t0 + (double)(n + 1) * c->h, w);
@@ -1117,7 +1300,8 @@ int control_step(aqc_ctx* c) {
 
 int graph_k(const aqc_ctx* c) {
   if (c->adaptive || c->in_batch || c->slab.n_slabs || c->step_class >= 0) return 0;
-  if (c->graph_req < 0) return c->n <= 20 ? 16 : 0;  // launch-bound sizes
+  if (c->graph_req < 0)  // launch-bound sizes
+    return c->n > 20 ? 0 : (resident_on(c) ? kResMaxEvals : 16);
   return c->graph_req;
 }
 
@@ -1161,7 +1345,11 @@ int capture_steps(aqc_ctx* c, int K) {
   cudaError_t e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal);
   int rc = AQC_OK;
   if (e == cudaSuccess) {
-    for (int j = 0; j < K && rc == AQC_OK; j++) {
+    if (resident_on(c)) {  // one launch for the K steps (K is even: V_P and V_Q keep their places)
+      c->cur_wdev = c->d_wdev;
+      rc = resident_steps(c, 0, false, K);
+    }
+    for (int j = 0; j < K && rc == AQC_OK && !resident_on(c); j++) {
       c->cur_wdev = c->d_wdev + kGraphStepWeights * j;
       rc = pec_step(c);
       c->step++;
@@ -1480,6 +1668,7 @@ int aqc_create(aqc_ctx** out, int device, int precision, int n_qubits, void* wor
     delete c;
     return AQC_E_CUDA;
   }
+  if (cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) c->sms = 1;
   *out = c;
   return AQC_OK;
 }
@@ -1807,6 +1996,10 @@ int aqc_set_initial_state(aqc_ctx* ctx, int kind, uint64_t basis, const void* us
       FAIL(ctx, AQC_E_INVAL, "bad initial-state kind");
   }
   CUDA_TRY(ctx, cudaMemsetAsync(ctx->d_slots, 0, kSlotCount * sizeof(double), ctx->stream));
+  // the predictor and the partial sum hold nothing yet: their workspace places again, so that a
+  // graph captured for an earlier run of this context fits the next one
+  ctx->vec[V_P] = ctx->ws + ctx->wp.off_vec + (size_t)V_P * ctx->wp.vec_bytes;
+  ctx->vec[V_Q] = ctx->ws + ctx->wp.off_vec + (size_t)V_Q * ctx->wp.vec_bytes;
   ctx->step = 0;
   ctx->evals = 0;
   ctx->nsteps = 0;
@@ -1840,18 +2033,31 @@ int aqc_propagate(aqc_ctx* ctx, int64_t max_steps, aqc_stats* stats) {
     CUDA_TRY(ctx, cudaEventRecord(e0, ctx->stream));
   }
   while (!ctx->at_end && ctx->steps_done < target) {
-    if (ctx->step < 3) {
+    if (ctx->step < 3 && resident_on(ctx)) {
+      const int64_t m = std::min<int64_t>({3 - ctx->step, ctx->seg_m - ctx->step, target - ctx->steps_done});
+      const bool hist = ctx->step + m == 3 && ctx->seg_m > 3 && target - ctx->steps_done > m;
+      rc = resident_start(ctx, (int)m, hist);
+      for (int64_t i = 0; i < m && !rc; i++) count_step(ctx);
+    } else if (ctx->step < 3) {
       rc = rk4_step(ctx);
       if (!rc) count_step(ctx);
     } else {
       if (!ctx->hist_ready) {
-        rc = start_history(ctx);
+        rc = resident_on(ctx) ? resident_start(ctx, 0, true) : start_history(ctx);
         if (rc) break;
       }
       const int K = graph_k(ctx);
-      if (K > 0 && ctx->seg_m - ctx->step >= K && target - ctx->steps_done >= K) {
+      const int64_t left = std::min(ctx->seg_m - ctx->step, target - ctx->steps_done);
+      if (K > 0 && left >= K) {
         rc = pec_steps_graph(ctx, K);
         if (rc) break;
+        continue;
+      }
+      if (K > 0 && left > 1 && resident_on(ctx)) {  // fewer than a replay: one launch of their own
+        const int m = (int)std::min<int64_t>(left, kResMaxEvals);
+        rc = resident_steps(ctx, 0, false, m);
+        if (rc) break;
+        for (int i = 0; i < m; i++) count_step(ctx);
         continue;
       }
       rc = pec_step(ctx);

@@ -73,6 +73,15 @@ __host__ __device__ __forceinline__ uint32_t tile_z(const Layout& L, uint32_t j,
   return zb | (j & cm) | ((j >> L.c) << L.h);
 }
 
+// Products of a resident launch that read one partner tile (or the own one): ranges end at ...
+struct ResPartner {
+  uint16_t hi;         // the partner is the tile whose number is the own one XOR hi (0: the own tile)
+  uint16_t plain_end;  // X strings with real coefficients, in the launch's list of them
+  uint16_t hop_end;    // hops, in the list of the other products
+  uint16_t gen_end;    // the rest
+};
+constexpr int kResMaxTiles = 256;
+
 struct DevTables {
   int n_layouts;
   int n_remote;                     // flips no layout holds, gathered from global memory
@@ -95,6 +104,9 @@ struct DevTables {
   uint32_t clause_mask[kMaxClauses];
   DevZ z[kMaxZ];
   DevFlip flips[kMaxFlips];
+  uint16_t res_idx[kMaxFlips];      // order of the products in a resident launch: the X strings with
+                                    // real coefficients by partner tile, then the others
+  ResPartner res_part[kResMaxTiles];
 };
 
 enum Mode : int {
@@ -166,7 +178,7 @@ struct SlabParams {
   unsigned* queue;      // next work item (reset to 0 by the last CTA)
   unsigned* done;       // finished partial tiles per slab (reset to 0 by the last CTA)
 };
-constexpr int kMaxSlabs = 2048;
+constexpr int kMaxSlabs = 2048;  // also the room of the resident launches' flags (kResMaxTiles x kResFlagStride)
 
 // Partial-sum pass of a strided layout holding only X strings with real coefficients
 // (complex64, kernel k_partial_x): the source tile arrives by TMA through `tmap`.
@@ -185,6 +197,40 @@ struct XPartialParams {
   void* qout;
   uint32_t ntiles;
   double* slots;         // kSlotFault is set if a tile copy never completes
+};
+
+// A resident launch (kernel k_resident): a sequence of evaluations of one state whose tiles, one
+// per CTA, are all on the GPU at once.  n_rk Runge-Kutta steps, then (hist) the start of the
+// derivative history, or n_pec predictor-corrector steps; or one evaluation alone (single).
+constexpr int kResMaxThreads = 512;  // threads that own amplitudes (one more warp does scalar work)
+constexpr int kResMaxEvals = 64;
+constexpr int kResFlagStride = 8;   // 32 bytes between tile flags: polls of one do not slow another
+struct ResParams {
+  const DevTables* tab;
+  int n, t;              // tile = 2^t consecutive indices
+  int np, ng;            // X strings with real coefficients, other products
+  int npart, nbuf;       // partner tiles beside the own one, shared-memory buffers for them
+  int ncode;             // largest clause count in dcode
+  int evals;             // evaluations in the launch
+  int n_rk, hist, n_pec;
+  int single;            // 0, or one evaluation: 6 out = H src, 7 <src|H|src>
+  int step0;             // index of the first grid step within its segment
+  int wstride;           // doubles between the weights of consecutive evaluations in wdev
+  const double* wdev;    // nullable: weights from device memory
+  double w[3 * kResMaxEvals];
+  double h;
+  const uint8_t* dcode;  // nullable
+  const void* src;       // what the first evaluation acts on
+  void* xout[2];         // exchange vectors: evaluation e writes xout[e & 1]
+  void* y;
+  void* yout;            // where y_{n+1} goes (y, or a second vector under step-size control)
+  void* f[4];            // derivative ring
+  void* acc;             // Runge-Kutta accumulator (states whose owned vectors stay in memory)
+  void* ylo;             // nullable: low part of y (compensated corrector)
+  unsigned* flags;       // one per tile, kResFlagStride apart: evaluations published (zero between launches)
+  unsigned* ticket;
+  double* partials;      // (evals + 1) x grid
+  double* slots;
 };
 
 // vectors of a state (workspace order)
@@ -281,6 +327,10 @@ cudaError_t launch_fma64(int blocks, int iters, cudaStream_t s);
 // up sets slots[kSlotFault]
 cudaError_t launch_wait_flag(const unsigned* flag, int64_t polls, double* slots, cudaStream_t s);
 constexpr int kSlotWaitFlag = 6;  // a slot whose bits serve as the self-test's flag (never set)
+size_t resident_smem_bytes(int prec, int t, int nbuf, int np, int ng, int n_z, int nth, bool reg);
+// slots: 16-byte slots per thread and tile; max_grid: CTAs at most (fewer than tiles: a CTA walks
+// several tiles and the owned vectors stay in global memory)
+cudaError_t launch_resident(int prec, const ResParams& p, int slots, int nth, int max_grid, int n_z, cudaStream_t s);
 int64_t fma64_count(int blocks, int iters);
 int reduce_grid(uint64_t N);
 cudaError_t launch_batch(int prec, int threads, const BatchLaunch& b, int nitems, int smem, cudaStream_t s);

@@ -1,0 +1,918 @@
+// Resident evaluations: states small enough that every CTA of one launch holds its own tile.
+//
+// A launch runs a sequence of evaluations of H(t) (Runge-Kutta stages, the start of the
+// derivative history, predictor-corrector steps; Sec. I.B) without leaving the GPU.  The state is
+// cut into contiguous tiles of 2^t indices, one per CTA (several, when a caller limits the CTAs or
+// the tiles outnumber them).  A thread owns the same amplitudes through the launch: y, the
+// derivatives and the Runge-Kutta accumulator are read and written by that thread alone, in
+// registers while a thread owns at most two 16-byte slots, else in global memory (they stay in
+// L2).  Only the vector that H acts on next (the predictor, a stage input, or y) is seen by
+// other threads: the CTA's own tile of it stays in shared memory, and a copy goes to one of two
+// exchange vectors in global memory, from where the CTAs whose products flip bits above t fetch
+// it as whole tiles.
+//
+// Exchange: products are sorted by the bits they flip above t ("partner" tiles; all products of
+// one partner share one copy).  When a tile is done the CTA raises the tile's flag; one warp per
+// CTA waits for its partners' flags, one by one, and starts a bulk copy (cp.async.bulk, completion
+// on an mbarrier) of each partner tile as soon as it is up, while the other warps work on the
+// products inside the tile.  The partner relation is symmetric, so having a partner's data also
+// says that it no longer reads the exchange vector written next; no CTA waits for all others.
+//
+// Another warp does the scalar FP64 work beside them (coefficients of the next evaluation, the sum
+// of the last one's error partials): on this GPU an FP64 instruction of a warp holds its
+// multiprocessor's pipe for about 19 cycles, so reducing by shuffles in every warp would take
+// longer than a small state's step.
+//
+// Measured, microseconds per predictor-corrector step (before: one launch per layout pass, replayed
+// from a graph, each on as many CTAs as the state has 64 KiB tiles):
+//   complex64, nonlinear path: n = 12 31 -> 3.8, n = 16 43 -> 5.4, n = 18 46 -> 10.5, n = 20 50 -> 36
+//   complex128, linear path:   n = 10 20 -> 3.4, n = 16 about 55 -> 10.4, n = 19 88 -> 82
+// Below n = 14 a step is the exchange (about 1.5 us from the last store to the first partner read)
+// and one pass of dependent shared-memory reads; above it complex64 is bound by the
+// shared-memory reads of the partners (16 bytes per product and slot), complex128 by the FP64 pipe.
+#include <cuda_runtime.h>
+#include <math.h>
+#include <stdint.h>
+
+#include <type_traits>
+
+#include "aqc_internal.h"
+
+namespace aqc {
+
+namespace {
+
+template <typename R>
+struct RT;
+template <>
+struct RT<float> {
+  using C2 = float2;
+  static constexpr int H = 2;  // amplitudes per 16-byte slot
+};
+template <>
+struct RT<double> {
+  using C2 = double2;
+  static constexpr int H = 1;
+};
+
+template <typename R>
+struct RPlain {  // X string with a real coefficient: place of the partner, coefficient
+  uint32_t off;
+  R c;
+};
+struct RBase {  // the same before the group weight
+  double coef;
+  uint32_t off;
+  int group;
+};
+template <typename R>
+struct RGen {  // hop or general product: mask, phases, place, effective coefficients
+  uint32_t x, zm, zm2, off;
+  R cr, ci, cr2, ci2;
+};
+template <typename R>
+struct RScal {        // diagonal of one evaluation
+  R dt[256];          // identity prefactors plus the byte-table class's energy, by clause count
+  R cw[kMaxClasses];  // weights of the other clause classes
+};
+
+constexpr uint32_t kResPolls = 1u << 22;  // flag and mbarrier polls before a wait gives up
+constexpr int kService = 128;             // threads beside those that own amplitudes: four warps
+
+__host__ __device__ inline size_t up16(size_t v) { return (v + 15) & ~(size_t)15; }
+
+// shared memory: [own tile][nbuf partner tiles][clause bytes][weights][bases][plain x2][general x2]
+// [Z x2][scalars x2][reductions x2][lane sums][mbarriers]
+template <typename R>
+struct ResSmem {
+  size_t code, w, base, pl, gen, z, scal, red, lane, bar, total;
+  __host__ __device__ ResSmem(uint32_t tsize, int nbuf, int np, int ng, int nz, int nth, bool dred) {
+    code = up16((size_t)tsize * (1 + nbuf) * 2 * sizeof(R));
+    w = up16(code + tsize);
+    base = up16(w + 3 * kResMaxEvals * sizeof(double));
+    pl = up16(base + (size_t)np * sizeof(RBase));
+    gen = up16(pl + 2 * (size_t)np * sizeof(RPlain<R>));
+    z = up16(gen + 2 * (size_t)ng * sizeof(RGen<R>));
+    scal = up16(z + 2 * (size_t)nz * sizeof(R));
+    red = up16(scal + 2 * sizeof(RScal<R>));
+    lane = up16(red + 3 * (size_t)nth * (dred ? sizeof(double) : sizeof(R)));
+    bar = lane + 8 * (kResMaxEvals + 1) * sizeof(double);
+    total = bar + 2 * (size_t)(nbuf > 0 ? nbuf : 1) * sizeof(uint64_t);
+  }
+};
+
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+
+__device__ __forceinline__ unsigned flag_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void flag_release(unsigned* p, unsigned v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;\n" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void bar_init(uint32_t b, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(b), "r"(count) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(uint32_t b) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(b) : "memory");
+}
+__device__ __forceinline__ bool bar_try(uint32_t b, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(b), "r"(parity)
+      : "memory");
+  return ok != 0u;
+}
+// bounded wait; ends early when another warp of the CTA has given up
+__device__ __forceinline__ bool bar_wait(uint32_t b, uint32_t parity, const volatile int* abort) {
+  for (uint32_t i = 0; i < kResPolls; i++) {
+    if (bar_try(b, parity)) return true;
+    if (*abort) return false;
+  }
+  return false;
+}
+__device__ __forceinline__ void expect(uint32_t b, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(b), "r"(bytes) : "memory");
+}
+// the wait at the end of a launch that gave up: both phases of a barrier, short
+__device__ __forceinline__ bool bar_wait_short(uint32_t b, uint32_t parity) {
+  for (uint32_t i = 0; i < (1u << 14); i++)
+    if (bar_try(b, parity)) return true;
+  return false;
+}
+// bytes from global memory into shared memory (both 16-byte aligned), counted on b
+__device__ __forceinline__ void tile_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t b) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst), "l"(src),
+      "r"(bytes), "r"(b)
+      : "memory");
+}
+__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async;\n" ::: "memory"); }
+
+template <typename C2, int H>
+__device__ __forceinline__ void unpack(const float4& x, C2 (&v)[H]) {
+  const C2* xs = reinterpret_cast<const C2*>(&x);
+#pragma unroll
+  for (int q = 0; q < H; q++) v[q] = xs[q];
+}
+template <typename C2, int H>
+__device__ __forceinline__ float4 pack(const C2 (&v)[H]) {
+  float4 x;
+  C2* xs = reinterpret_cast<C2*>(&x);
+#pragma unroll
+  for (int q = 0; q < H; q++) xs[q] = v[q];
+  return x;
+}
+
+// hi + lo + inc as an exact two-sum renormalised into (hi, lo): the compensated corrector
+__device__ __forceinline__ float add_compensated(float hi, float& lo, float inc) {
+  const float s = __fadd_rn(hi, inc);
+  const float bp = __fsub_rn(s, hi);
+  const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bp)), __fsub_rn(inc, bp));
+  const float l = __fadd_rn(lo, e);
+  const float h = __fadd_rn(s, l);
+  lo = __fsub_rn(l, __fsub_rn(h, s));
+  return h;
+}
+__device__ __forceinline__ double add_compensated(double hi, double&, double inc) { return hi + inc; }
+
+// warp sum of v in lane order; the total in lane 0
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Kind of evaluation e of the launch: 1..4 Runge-Kutta stage, 5 start of the derivative history,
+// 0 predictor-corrector step; 6 H psi, 7 <psi|H|psi>.
+__device__ __forceinline__ int kind_of(const ResParams& P, int e) {
+  if (P.single) return P.single;
+  if (e < 4 * P.n_rk) return 1 + (e & 3);
+  return (P.hist && e == 4 * P.n_rk) ? 5 : 0;
+}
+
+// Coefficients of the off-diagonal products at weights w (one warp).
+template <typename R>
+__device__ __forceinline__ void coefficients(const ResParams& P, const double* w, const RBase* base, RPlain<R>* pl,
+                                             RGen<R>* gen) {
+  const DevTables* tab = P.tab;
+  const double w0 = w[0], w1 = w[1], w2 = w[2];
+  auto pick = [&](int g) { return g == 0 ? w0 : (g == 1 ? w1 : w2); };
+  const int lane = threadIdx.x & 31;
+  for (int k = lane; k < P.np; k += 32) {
+    const RBase d = base[k];
+    pl[k] = RPlain<R>{d.off, (R)(d.coef * pick(d.group))};
+  }
+  for (int k = lane; k < P.ng; k += 32) {
+    const DevFlip d = tab->flips[tab->res_idx[P.np + k]];
+    double v[4] = {0.0, 0.0, 0.0, 0.0};  // c i^ipow of the product and of its companion
+    auto phased = [](double c, int ipow, double* o) {
+      o[0] = (ipow & 1) ? 0.0 : ((ipow & 2) ? -c : c);
+      o[1] = (ipow & 1) ? ((ipow & 2) ? -c : c) : 0.0;
+    };
+    phased(d.coef * pick(d.group), d.ipow, v);
+    if (d.has2) phased(d.coef2 * pick(d.group2), d.ipow2, v + 2);
+    gen[k] = RGen<R>{d.x, d.zm, d.has2 ? d.zm2 : 0u, gen[k].off, (R)v[0], (R)v[1], (R)v[2], (R)v[3]};
+  }
+}
+
+// Coefficients of the diagonal at weights w (one warp).
+template <typename R>
+__device__ __forceinline__ void diagonal_of(const ResParams& P, const double* w, R* zc, RScal<R>* sc,
+                                            const double (&ident)[3], int nz, int ncls, double tscale, int tgroup) {
+  const DevTables* tab = P.tab;
+  const double w0 = w[0], w1 = w[1], w2 = w[2];
+  auto pick = [&](int g) { return g == 0 ? w0 : (g == 1 ? w1 : w2); };
+  const int lane = threadIdx.x & 31;
+  for (int k = lane; k < nz; k += 32) zc[k] = (R)(tab->z[k].coef * pick(tab->z[k].group));
+  const R dconst = (R)(ident[0] * w0 + ident[1] * w1 + ident[2] * w2);
+  if (P.dcode) {
+    const R wt = (R)(tscale * pick(tgroup));
+    for (int k = lane; k <= P.ncode; k += 32) sc->dt[k] = fma_(wt, (R)k, dconst);
+    if (ncls > 1)
+      for (int k = lane; k < ncls; k += 32) sc->cw[k] = (R)(tab->classes[k].scale * pick(tab->classes[k].group));
+  } else {
+    if (lane == 0) sc->dt[0] = dconst;
+    for (int k = lane; k < ncls; k += 32) sc->cw[k] = (R)(tab->classes[k].scale * pick(tab->classes[k].group));
+  }
+}
+
+__device__ __forceinline__ int count_clauses(const DevTables* __restrict__ tab, int pen, int b, int e, uint32_t z) {
+  int cnt = 0;
+  for (int k = b; k < e; k++) {
+    const int o = 1 - __popc(tab->clause_mask[k] & z);
+    cnt += pen == 0 ? (o != 0) : o * o;
+  }
+  return cnt;
+}
+
+// Diagonal parts beside the table lookup: other clause classes and Z strings (rare).
+template <typename R>
+__device__ __noinline__ R other_diagonal(const DevTables* tab, const RScal<R>& sc, const R* zc, int tcls, int code,
+                                         uint32_t z) {
+  R d = (R)0;
+  for (int cc = 0; cc < tab->n_classes; cc++) {
+    if (cc == tcls) continue;
+    const DevClass cl = tab->classes[cc];
+    const int cnt = (cl.derived && tcls >= 0) ? code - count_clauses(tab, cl.pen, cl.dbegin, cl.dend, z)
+                                              : count_clauses(tab, cl.pen, cl.begin, cl.end, z);
+    d = fma_(sc.cw[cc], (R)cnt, d);
+  }
+  for (int m = 0; m < tab->n_z; m++) d += (__popc(tab->z[m].zm & z) & 1) ? -zc[m] : zc[m];
+  return d;
+}
+
+// All threads of the CTA, from the loop of any role.
+__device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 0;\n" ::: "memory"); }
+
+// S slots per thread: a tile is S x (threads that own amplitudes) slots.  REG: the owned vectors
+// stay in registers for the launch and the CTA has one tile; otherwise a CTA walks its tiles and
+// the owned vectors come from global memory, a quarter tile at a time through the partner buffers
+// (S >= 4) or one slot ahead.  Per amplitude all variants run the same operations in the same
+// order.  PEC: predictor-corrector steps; otherwise the start-up and single evaluations.
+//
+// The warps take roles, each with its own loop over the evaluations: owners, the coefficients of
+// the next evaluation's products, those of its diagonal, the sums of the last one's error
+// partials, and the tile copies.
+template <typename R, int S, bool REG, bool PEC, bool COMP>
+__global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const __grid_constant__ ResParams P) {
+  using C2 = typename RT<R>::C2;
+  constexpr int H = RT<R>::H;
+  constexpr int A = S * H;  // amplitudes per thread and tile
+  constexpr bool kComp = COMP && sizeof(R) == 4;
+  constexpr bool kStream = PEC && !REG && !kComp && S >= 4;
+  constexpr int SC = S / 4 > 0 ? S / 4 : 1;  // slots per streamed quarter tile
+  using RED = typename std::conditional<REG, R, double>::type;
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ ResPartner s_part[kResMaxTiles];
+  __shared__ volatile int s_abort;
+  __shared__ double s_err[kResMaxEvals + 2];
+
+  const DevTables* tab = P.tab;
+  const int nth = (int)blockDim.x - kService, nwarps = nth >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const bool owner = tid < nth;
+  const int svc = (tid - nth) >> 5;  // service warp 0..3
+  const uint32_t tsize = 1u << P.t, tmask = tsize - 1u, tbytes = tsize * (uint32_t)sizeof(C2);
+  const uint32_t ntiles = 1u << (P.n - P.t), G = gridDim.x;
+  const int np = P.np, ng = P.ng, nz = tab->n_z, ncls = tab->n_classes;
+  const int nd = P.npart, nbuf = P.nbuf;  // partner tiles (beside the own one) and their buffers
+  const int nq = nd + (kStream && nbuf > 0 ? 4 : 0);  // ring entries per tile visit
+  const bool ring = nq > nbuf || (kStream && nbuf > 0);  // else every partner has a buffer of its own
+  const int tcls = P.dcode ? tab->table_class : -1;
+  const int E = P.evals;
+  const bool multi = ntiles > G;  // several tiles per CTA
+  const ResSmem<R> M(tsize, nbuf, np, ng, nz, nth, !REG);
+  C2* const xs = reinterpret_cast<C2*>(smem);
+  uint8_t* const s_code = smem + M.code;
+  double* const s_w = reinterpret_cast<double*>(smem + M.w);
+  RBase* const s_base = reinterpret_cast<RBase*>(smem + M.base);
+  RPlain<R>* const s_pl = reinterpret_cast<RPlain<R>*>(smem + M.pl);
+  RGen<R>* const s_gen = reinterpret_cast<RGen<R>*>(smem + M.gen);
+  R* const s_z = reinterpret_cast<R*>(smem + M.z);
+  RScal<R>* const s_sc = reinterpret_cast<RScal<R>*>(smem + M.scal);
+  RED* const s_red = reinterpret_cast<RED*>(smem + M.red);           // [parity][nth], then [nth] of the last
+  double* const s_lane = reinterpret_cast<double*>(smem + M.lane);  // [E + 1][8]
+  const uint32_t full0 = saddr(smem + M.bar), empty0 = full0 + 8u * (uint32_t)nbuf;
+
+  if (tid == 0) {
+    s_abort = 0;
+    for (int b = 0; b < nbuf; b++) {
+      bar_init(full0 + 8u * b, 1);
+      bar_init(empty0 + 8u * b, (uint32_t)nwarps);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
+  for (int k = tid; k <= nd; k += blockDim.x) s_part[k] = tab->res_part[k];
+  for (int k = tid; k < 3 * E; k += blockDim.x)
+    s_w[k] = P.wdev ? P.wdev[(size_t)P.wstride * (k / 3) + k % 3] : P.w[k];
+  __syncthreads();
+  // a product's place in shared memory: its flip inside the tile, and its partner's buffer when
+  // every partner has one (XOR with a slot's byte offset)
+  auto place = [&](uint32_t x) {
+    uint32_t p = 0;
+    if (!ring)
+      while (s_part[p].hi != (x >> P.t)) p++;
+    return (x & tmask) * (uint32_t)sizeof(C2) | p * tbytes;
+  };
+  for (int k = tid; k < np; k += blockDim.x) {
+    const DevFlip d = tab->flips[tab->res_idx[k]];
+    s_base[k] = RBase{d.coef, place(d.x), d.group};
+  }
+  for (int k = tid; k < ng; k += blockDim.x) s_gen[k].off = s_gen[ng + k].off = place(tab->flips[tab->res_idx[np + k]].x);
+  __syncthreads();
+
+  // copies of partner tiles (and of owned quarter tiles) for one visit of a tile; q0: ring entries
+  // so far, visit: tile visits so far
+  auto copy_in = [&](uint32_t tile, const C2* xin, int e, int latest, uint32_t q0) {
+    auto give_up = [&]() {
+      s_abort = 1;
+      P.slots[kSlotFault] = 1.0;
+    };
+    auto ready = [&](uint32_t other) {  // the partner has published this evaluation's source
+      if (e == 0) return true;
+      uint32_t polls = 0;
+      while (flag_acquire(P.flags + kResFlagStride * other) < (unsigned)e) {
+        if (++polls > kResPolls || s_abort) return false;
+        if (polls > 256u) __nanosleep(64);
+      }
+      return true;
+    };
+    if (!ring) {
+      if (lane == 0) expect(full0, (uint32_t)nd * tbytes);
+      __syncwarp();
+      for (int p = lane; p < nd; p += 32) {
+        const uint32_t other = tile ^ s_part[p + 1].hi;
+        if (!ready(other)) {
+          give_up();
+          break;
+        }
+        proxy_fence();  // the partner's stores, seen by its flag, before the asynchronous copy
+        tile_copy(saddr(xs + (size_t)(1 + p) * tsize), xin + ((size_t)other << P.t), tbytes, full0);
+      }
+    } else if (lane == 0) {
+      uint32_t b = q0 % (uint32_t)nbuf, use = q0 / (uint32_t)nbuf;
+      for (int p = 0; p < nq; p++) {
+        const uint32_t other = p < nd ? tile ^ s_part[p + 1].hi : tile;
+        if ((use > 0 && !bar_wait(empty0 + 8u * b, (use - 1u) & 1u, &s_abort)) || (p < nd && !ready(other))) {
+          give_up();
+          break;
+        }
+        proxy_fence();
+        const uint32_t dst = saddr(xs + (size_t)(1u + b) * tsize), bb = full0 + 8u * b;
+        expect(bb, tbytes);
+        if (p < nd) {
+          tile_copy(dst, xin + ((size_t)other << P.t), tbytes, bb);
+        } else {
+          const uint32_t part = tbytes / 4;
+          const size_t z = ((size_t)tile << P.t) + (size_t)(p - nd) * (tsize / 4);
+          const void* v[4] = {P.y, P.f[latest & 3], P.f[(latest - 1) & 3], P.f[(latest - 2) & 3]};
+#pragma unroll
+          for (int i = 0; i < 4; i++) tile_copy(dst + i * part, reinterpret_cast<const C2*>(v[i]) + z, part, bb);
+        }
+        if (++b == (uint32_t)nbuf) {
+          b = 0;
+          use++;
+        }
+      }
+    }
+    __syncwarp();
+  };
+  const C2* const src0 = reinterpret_cast<const C2*>(P.src);
+  C2* const XA = reinterpret_cast<C2*>(P.xout[0]);
+  C2* const XO = reinterpret_cast<C2*>(P.xout[1]);
+  // a[] holds f_latest; at a start-up f_k is known for k < step0, later for k <= step0
+  const int first_latest = P.single ? 0 : (P.n_rk > 0 || P.hist ? P.step0 - 1 : P.step0);
+  int latest = first_latest;
+  uint32_t q0 = 0, visit = 0;
+
+  if (owner) {
+    C2* const Y = reinterpret_cast<C2*>(P.y);
+    C2* const YO = reinterpret_cast<C2*>(P.yout);
+    C2* const ACC = reinterpret_cast<C2*>(P.acc);
+    C2* const YL = reinterpret_cast<C2*>(P.ylo);
+    auto F = [&](int k) { return reinterpret_cast<C2*>(P.f[k & 3]); };  // f_k's ring slot
+    const R h = (R)P.h;
+    const double e24 = P.h / 24.0;
+    const R h24 = (R)e24, h24lo = sizeof(R) == 8 ? (R)0 : (R)(e24 - (double)h24);
+    const R c9 = (R)9 * h24, c19 = (R)19 * h24, c5 = (R)5 * h24;
+    const R p55 = (R)55 * h24, p59 = (R)59 * h24, p37 = (R)37 * h24, p9 = (R)9 * h24;
+    const bool others = nz > 0 || ncls > (tcls >= 0 ? 1 : 0);
+    // y, f of the last three steps, Runge-Kutta accumulator and low part of y of one slot
+    struct Owned {
+      C2 y[H], a[H], b[H], c[H], rk[H], yl[H];
+    };
+    auto load = [&](const C2* v, C2 (&d)[H]) { unpack<C2, H>(*reinterpret_cast<const float4*>(v), d); };
+    auto store = [&](C2* v, const C2 (&d)[H]) { *reinterpret_cast<float4*>(v) = pack<C2, H>(d); };
+    const int j0 = tid * H, js = nth * H;  // tile position of the first slot, slot stride
+    const bool act = j0 < (int)tsize;      // tiles below one slot per thread: some idle
+    const uint32_t jb = (uint32_t)j0 * sizeof(C2), jsb = (uint32_t)js * sizeof(C2);
+    Owned o[REG ? S : 1];
+    if (REG && act && !P.single) {
+#pragma unroll
+      for (int s = 0; s < S; s++) {
+        const uint32_t z = (blockIdx.x << P.t) + (uint32_t)(j0 + s * js);
+        load(Y + z, o[s].y);
+        if (latest >= 0) load(F(latest) + z, o[s].a);
+        if (latest >= 1) load(F(latest - 1) + z, o[s].b);
+        if (latest >= 2) load(F(latest - 2) + z, o[s].c);
+        if (kComp) load(YL + z, o[s].yl);
+      }
+    }
+    const C2* xin = src0;
+    C2* xout = XA;
+    for (int e = 0; e < E; e++) {
+      const int kind = PEC ? 0 : kind_of(P, e), par = e & 1;
+      const bool last = e == E - 1;
+      const RPlain<R>* const pl = s_pl + par * np;
+      const RGen<R>* const gen = s_gen + par * ng;
+      const RScal<R>& sc = s_sc[par];
+      RED red0 = (RED)0, red1 = (RED)0;
+      for (uint32_t tile = blockIdx.x; tile < ntiles; tile += G, visit++) {
+        const uint32_t zb = tile << P.t;
+        if (e == 0 || multi) {  // the own tile and its clause bytes (then kept up to date in place)
+          if (multi) cta_sync();  // readers of the previous tile are done
+          for (uint32_t j = j0; j < tsize; j += js)
+            *reinterpret_cast<float4*>(xs + j) = __ldcg(reinterpret_cast<const float4*>(xin + zb + j));
+          if (tcls >= 0)
+            for (uint32_t j = j0; j < tsize; j += js)
+#pragma unroll
+              for (int q = 0; q < H; q++) s_code[j + q] = P.dcode[zb + j + q];
+          cta_sync();
+        }
+        R ar[A], ai[A];
+#pragma unroll
+        for (int g = 0; g < A; g++) ar[g] = ai[g] = (R)0;
+        // X strings with real coefficients [k, end) out of the tiles from `t` on; the two complex64
+        // amplitudes of a slot are read one by one, so a flip of index bit 0 needs no swap
+        auto plain = [&](const unsigned char* t, int k, int end) {
+          constexpr int U = S >= 4 ? 1 : 4 / S;  // products in flight
+          if constexpr (S >= 4) {  // many slots: one 16-byte load each, the swap chosen per product
+#pragma unroll 1
+            for (; k < end; k++) {
+              const RPlain<R> f = pl[k];
+              const uint32_t at = jb ^ (f.off & ~15u);
+              float4 v[S];
+#pragma unroll
+              for (int s = 0; s < S; s++) v[s] = *reinterpret_cast<const float4*>(t + (at ^ ((uint32_t)s * jsb)));
+              const bool sw = H == 2 && (f.off & 15u);
+#pragma unroll
+              for (int s = 0; s < S; s++) {
+                C2 u[H];
+                unpack<C2, H>(v[s], u);
+#pragma unroll
+                for (int q = 0; q < H; q++) {
+                  const C2 x = sw ? u[H - 1 - q] : u[q];
+                  ar[s * H + q] = fma_(f.c, x.x, ar[s * H + q]);
+                  ai[s * H + q] = fma_(f.c, x.y, ai[s * H + q]);
+                }
+              }
+            }
+            return;
+          }
+          auto one = [&](const RPlain<R>& f, int s, const C2 (&u)[H]) {
+#pragma unroll
+            for (int q = 0; q < H; q++) {
+              ar[s * H + q] = fma_(f.c, u[q].x, ar[s * H + q]);
+              ai[s * H + q] = fma_(f.c, u[q].y, ai[s * H + q]);
+            }
+          };
+          auto get = [&](uint32_t off, int s, C2 (&u)[H]) {
+            const uint32_t at = (jb ^ off) ^ ((uint32_t)s * jsb);
+#pragma unroll
+            for (int q = 0; q < H; q++) u[q] = *reinterpret_cast<const C2*>(t + (at ^ (uint32_t)(q * sizeof(C2))));
+          };
+          for (; k + U <= end; k += U) {
+            RPlain<R> f[U];
+            C2 u[U][S][H];
+#pragma unroll
+            for (int i = 0; i < U; i++) {
+              f[i] = pl[k + i];
+#pragma unroll
+              for (int s = 0; s < S; s++) get(f[i].off, s, u[i][s]);
+            }
+#pragma unroll
+            for (int i = 0; i < U; i++)
+#pragma unroll
+              for (int s = 0; s < S; s++) one(f[i], s, u[i][s]);
+          }
+          if (U > 1)
+            for (; k < end; k++) {
+              const RPlain<R> f = pl[k];
+#pragma unroll
+              for (int s = 0; s < S; s++) {
+                C2 u[H];
+                get(f.off, s, u);
+                one(f, s, u);
+              }
+            }
+        };
+        // hops [k, hops) and other products [.., end)
+        auto general = [&](const unsigned char* t, int k, int hops, int end) {
+#pragma unroll 1
+          for (; k < end; k++) {
+            const RGen<R> f = gen[k];
+#pragma unroll
+            for (int s = 0; s < S; s++) {
+              const uint32_t at = (jb ^ f.off) ^ ((uint32_t)s * jsb);
+#pragma unroll
+              for (int q = 0; q < H; q++) {
+                const C2 w = *reinterpret_cast<const C2*>(t + (at ^ (uint32_t)(q * sizeof(C2))));
+                const int g = s * H + q;
+                const uint32_t z = zb + (uint32_t)(j0 + s * js + q);
+                if (k < hops) {  // 2c where the two bits of z differ (cr - cr2 = 2c)
+                  const R cf = (__popc(f.x & z) & 1) ? f.cr - f.cr2 : (R)0;
+                  ar[g] = fma_(cf, w.x, ar[g]);
+                  ai[g] = fma_(cf, w.y, ai[g]);
+                } else {
+                  const uint32_t zsrc = z ^ f.x;
+                  const bool n1 = __popc(f.zm & zsrc) & 1, n2 = __popc(f.zm2 & zsrc) & 1;
+                  const R cr = (n1 ? -f.cr : f.cr) + (n2 ? -f.cr2 : f.cr2);
+                  const R ci = (n1 ? -f.ci : f.ci) + (n2 ? -f.ci2 : f.ci2);
+                  ar[g] = fma_(cr, w.x, fma_(-ci, w.y, ar[g]));
+                  ai[g] = fma_(cr, w.y, fma_(ci, w.x, ai[g]));
+                }
+              }
+            }
+          }
+        };
+        auto arrived = [&](uint32_t b, uint32_t parity) {
+          if (!bar_wait(full0 + 8u * b, parity, &s_abort)) {
+            if (!s_abort) P.slots[kSlotFault] = 1.0;
+            s_abort = 1;
+          }
+        };
+        const unsigned char* const t0p = smem;
+        int gb = s_part[0].gen_end;
+        if (act) {
+          plain(t0p, 0, s_part[0].plain_end);
+          if (gb > 0) general(t0p, 0, s_part[0].hop_end, gb);
+        }
+        if (nd > 0 && !ring) {  // every partner in one go: the places name the buffers
+          arrived(0, visit & 1u);
+          if (act) {
+            plain(t0p, s_part[0].plain_end, np);
+            for (int p = 1; p <= nd && gb < ng; p++) {
+              general(t0p, gb, s_part[p].hop_end, s_part[p].gen_end);
+              gb = s_part[p].gen_end;
+            }
+          }
+        }
+        uint32_t rb = ring ? q0 % (uint32_t)nbuf : 0u, ru = ring ? q0 / (uint32_t)nbuf : 0u;
+        auto release = [&]() {  // this warp is done with buffer rb; on to the next ring entry
+          __syncwarp();
+          if (lane == 0) bar_arrive(empty0 + 8u * rb);
+          if (++rb == (uint32_t)nbuf) {
+            rb = 0;
+            ru++;
+          }
+        };
+        if (ring) {
+          int pb = s_part[0].plain_end;
+          for (int p = 1; p <= nd; p++) {
+            const ResPartner pt = s_part[p];
+            arrived(rb, ru & 1u);
+            if (act) {
+              const unsigned char* t = smem + (size_t)(1u + rb) * tbytes;
+              plain(t, pb, pt.plain_end);
+              if (pt.gen_end > gb) general(t, gb, pt.hop_end, pt.gen_end);
+            }
+            pb = pt.plain_end;
+            gb = pt.gen_end;
+            release();
+          }
+        }
+        // every owner is past the products that read the own tile: it can be overwritten
+        asm volatile("bar.sync 1, %0;\n" ::"r"(nth) : "memory");
+        R t0 = (R)0, t1 = (R)0;
+        auto fetch_owned = [&](int s, Owned& w) {  // of one slot, from global memory
+          const uint32_t z = zb + (uint32_t)(j0 + s * js);
+          if (P.single) return;
+          load(Y + z, w.y);
+          if (kind == 0 || kind == 5) {
+            load(F(latest) + z, w.a);
+            load(F(latest - 1) + z, w.b);
+            load(F(latest - 2) + z, w.c);
+          }
+          if (kind >= 2 && kind <= 4) load(ACC + z, w.rk);
+          if (kComp && kind == 0) load(YL + z, w.yl);
+        };
+        const bool streamed = kStream && nq > nd;
+        Owned ow[kStream ? 1 : 2];
+        if (!REG && !kStream && act) fetch_owned(0, ow[0]);
+#pragma unroll
+        for (int s = 0; s < S; s++) {
+          Owned& w = REG ? o[REG ? s : 0] : ow[kStream ? 0 : (s & 1)];
+          if (streamed) {  // this slot's owned vectors from their quarter tile
+            if (s % SC == 0) arrived(rb, ru & 1u);
+            const C2* v = xs + (size_t)(1u + rb) * tsize + (uint32_t)(j0 + (s % SC) * js);
+            load(v, w.y);
+            load(v + tsize / 4, w.a);
+            load(v + tsize / 2, w.b);
+            load(v + 3 * (tsize / 4), w.c);
+            if (s % SC == SC - 1) release();
+          } else if (kStream && act) {
+            fetch_owned(s, w);
+          } else if (!REG && s + 1 < S && act) {
+            fetch_owned(s + 1, ow[(s + 1) & 1]);
+          }
+          if (!act) continue;
+          const uint32_t j = (uint32_t)(j0 + s * js), z0 = zb + j;
+          C2 own[H], nx[H];
+          load(xs + j, own);
+#pragma unroll
+          for (int q = 0; q < H; q++) {
+            R re = ar[s * H + q], im = ai[s * H + q];
+            const int code = tcls >= 0 ? s_code[j + q] : 0;
+            R d = sc.dt[code];
+            if (others) d += other_diagonal<R>(tab, sc, s_z + par * nz, tcls, code, z0 + q);
+            if (d != (R)0) {  // also keeps an infinite amplitude from turning an H without diagonal into NaN
+              re = fma_(d, own[q].x, re);
+              im = fma_(d, own[q].y, im);
+            }
+            const C2 fn = C2{im, -re};  // -i (re + i im)
+            C2 &y = w.y[q], &a = w.a[q], &b = w.b[q], &c = w.c[q], &rk = w.rk[q];
+            if (kind == 0 || kind == 5) {
+              if (kind == 0) {  // corrector (Adams-Moulton)
+                if (sizeof(R) == 8) {
+                  y.x = fma_(c9, fn.x, fma_(c19, a.x, fma_(-c5, b.x, fma_(h24, c.x, y.x))));
+                  y.y = fma_(c9, fn.y, fma_(c19, a.y, fma_(-c5, b.y, fma_(h24, c.y, y.y))));
+                } else {  // h/24 as hi + lo: a step size rounded to FP32 would drift over the run
+                  const R sx = fma_((R)9, fn.x, fma_((R)19, a.x, fma_((R)-5, b.x, c.x)));
+                  const R sy = fma_((R)9, fn.y, fma_((R)19, a.y, fma_((R)-5, b.y, c.y)));
+                  const R ix = fma_(h24, sx, h24lo * sx), iy = fma_(h24, sy, h24lo * sy);
+                  if (kComp) {
+                    y.x = add_compensated(y.x, w.yl[q].x, ix);
+                    y.y = add_compensated(y.y, w.yl[q].y, iy);
+                  } else {
+                    y.x += ix;
+                    y.y += iy;
+                  }
+                }
+                const R dx = y.x - own[q].x, dy = y.y - own[q].y;
+                t1 = fma_(dx, dx, fma_(dy, dy, t1));
+                if (last) t0 = fma_(y.x, y.x, fma_(y.y, y.y, t0));
+              }
+              if (sizeof(R) == 8) {  // predictor (Adams-Bashforth)
+                nx[q] = C2{fma_(p55, fn.x, fma_(-p59, a.x, fma_(p37, b.x, fma_(-p9, c.x, y.x)))),
+                           fma_(p55, fn.y, fma_(-p59, a.y, fma_(p37, b.y, fma_(-p9, c.y, y.y))))};
+              } else {
+                const R px = fma_((R)55, fn.x, fma_((R)-59, a.x, fma_((R)37, b.x, (R)-9 * c.x)));
+                const R py = fma_((R)55, fn.y, fma_((R)-59, a.y, fma_((R)37, b.y, (R)-9 * c.y)));
+                nx[q] = C2{y.x + fma_(h24, px, h24lo * px), y.y + fma_(h24, py, h24lo * py)};
+              }
+              c = b;
+              b = a;
+              a = fn;
+            } else if (kind == 1) {
+              c = b;
+              b = a;
+              a = fn;
+              rk = fn;
+              const R hh = (R)0.5 * h;
+              nx[q] = C2{fma_(hh, fn.x, y.x), fma_(hh, fn.y, y.y)};
+            } else if (kind == 2 || kind == 3) {
+              rk.x = fma_((R)2, fn.x, rk.x);
+              rk.y = fma_((R)2, fn.y, rk.y);
+              const R hh = kind == 2 ? (R)0.5 * h : h;
+              nx[q] = C2{fma_(hh, fn.x, y.x), fma_(hh, fn.y, y.y)};
+            } else if (kind == 4) {
+              const R h6 = h / (R)6;
+              y.x = fma_(h6, rk.x + fn.x, y.x);
+              y.y = fma_(h6, rk.y + fn.y, y.y);
+              nx[q] = y;
+            } else if (kind == 6) {
+              nx[q] = C2{re, im};
+            } else {
+              t0 = fma_(own[q].x, re, fma_(own[q].y, im, t0));
+              t1 = fma_(own[q].x, im, fma_(-own[q].y, re, t1));
+              nx[q] = own[q];
+            }
+          }
+          if (kind != 7) store(xout + z0, nx);
+          if (!last && !multi) store(xs + j, nx);
+          if (!REG) {
+            if (kind == 0 || kind == 5 || kind == 1) store(F(latest + 1) + z0, w.a);
+            if (kind == 0 || kind == 4) store((kind == 0 ? YO : Y) + z0, w.y);
+            if (kind >= 1 && kind <= 3) store(ACC + z0, w.rk);
+            if (kComp && kind == 0) store(YL + z0, w.yl);
+          }
+        }
+        if (!last && nq > 0) proxy_fence();  // this thread's stores, before asynchronous copies read them
+        red0 += (RED)t0;
+        red1 += (RED)t1;
+        q0 += (uint32_t)nq;
+        if (!last && multi) cta_sync();  // published before the next tile
+      }
+      if (kind == 0 || kind == 7) {
+        s_red[(size_t)par * nth + tid] = red1;
+        if (last) s_red[(size_t)2 * nth + tid] = red0;
+      }
+      if (kind == 0 || kind == 5 || kind == 1) latest++;
+      if (last) break;
+      cta_sync();  // this CTA's part of xout is stored, the next coefficients are ready
+      if (s_abort) break;  // uniform: the results are invalid and reported so
+      xin = xout;
+      xout = xout == XA ? XO : XA;
+    }
+    if (REG && act && !P.single) {  // the owned vectors back to global memory
+#pragma unroll
+      for (int s = 0; s < S; s++) {
+        const uint32_t z = (blockIdx.x << P.t) + (uint32_t)(j0 + s * js);
+        if (E > P.hist) store((P.n_pec ? YO : Y) + z, o[s].y);
+        if (latest > first_latest) store(F(latest) + z, o[s].a);
+        if (latest > first_latest + 1) store(F(latest - 1) + z, o[s].b);
+        if (latest > first_latest + 2) store(F(latest - 2) + z, o[s].c);
+        if (kComp && P.n_pec) store(YL + z, o[s].yl);
+      }
+    }
+  } else {
+    // evaluation e's reductions over the CTA: FP64 sums in a fixed order, eight per evaluation
+    // (the eight are added after the last one)
+    auto lane_sums = [&](const RED* r, double* out) {
+      double v = 0.0;
+      for (int i = lane; i < nth; i += 32) v += (double)r[i];
+      v += __shfl_down_sync(0xffffffffu, v, 16);
+      v += __shfl_down_sync(0xffffffffu, v, 8);
+      if (lane < 8) out[lane] = v;
+    };
+    double ident[3] = {tab->ident[0], tab->ident[1], tab->ident[2]};
+    const double tscale = tcls >= 0 ? tab->classes[tcls].scale : 0.0;
+    const int tgroup = tcls >= 0 ? tab->classes[tcls].group : 0;
+    auto prepare = [&](int e) {  // coefficients of evaluation e
+      const int par = e & 1;
+      if (svc == 0) coefficients<R>(P, s_w + 3 * e, s_base, s_pl + par * np, s_gen + par * ng);
+      if (svc == 1) diagonal_of<R>(P, s_w + 3 * e, s_z + par * nz, s_sc + par, ident, nz, ncls, tscale, tgroup);
+    };
+    prepare(0);
+    const C2* xin = src0;
+    for (int e = 0; e < E; e++) {
+      const bool last = e == E - 1;
+      for (uint32_t tile = blockIdx.x; tile < ntiles; tile += G) {
+        if (e == 0 || multi) {
+          if (multi) cta_sync();
+          cta_sync();
+        }
+        if (svc == 3 && nq > 0) copy_in(tile, xin, e, latest, q0);
+        q0 += (uint32_t)nq;
+        if (tile == blockIdx.x) {
+          if (!last) prepare(e + 1);
+          if (PEC && svc == 2 && e > 0) lane_sums(s_red + (size_t)((e - 1) & 1) * nth, s_lane + 8 * (e - 1));
+        }
+        if (!last && multi) {
+          cta_sync();
+          if (svc == 3 && lane == 0) flag_release(P.flags + kResFlagStride * tile, (unsigned)(e + 1));
+        }
+      }
+      const int kind = PEC ? 0 : kind_of(P, e);
+      if (kind == 0 || kind == 5 || kind == 1) latest++;
+      if (last) break;
+      cta_sync();
+      if (s_abort) break;
+      if (!multi && svc == 3 && lane == 0 && nd > 0) flag_release(P.flags + kResFlagStride * blockIdx.x, (unsigned)(e + 1));
+      xin = e & 1 ? XO : XA;
+    }
+    if (s_abort && svc == 3) {  // copies in flight land before the CTA leaves (bounded)
+      for (int b = lane; b < nbuf; b += 32)
+        for (uint32_t par = 0; par < 2; par++) (void)bar_wait_short(full0 + 8u * b, par);
+    }
+    if (PEC || P.single == 7) {
+      asm volatile("bar.sync 2, %0;\n" ::"r"((int)blockDim.x) : "memory");  // the last reductions are there
+      if (svc == 2) {
+        lane_sums(s_red + (size_t)((E - 1) & 1) * nth, s_lane + 8 * (E - 1));
+        lane_sums(s_red + (size_t)2 * nth, s_lane + 8 * E);
+      }
+    }
+  }
+  const bool reduced = P.n_pec > 0 || P.single == 7;
+  if (owner && (PEC || P.single == 7)) asm volatile("bar.sync 2, %0;\n" ::"r"((int)blockDim.x) : "memory");
+  if (P.single == 6) return;
+  __syncthreads();
+  if (reduced) {
+    for (int e = tid >> 5; e <= E; e += (int)blockDim.x >> 5) {
+      double v = 0.0;
+      if (lane == 0) {
+        for (int k = 0; k < 8; k++) v += s_lane[8 * e + k];
+        P.partials[(size_t)e * G + blockIdx.x] = v;
+      }
+    }
+  }
+  // the last CTA sums the CTAs' partials in CTA order and clears the flags for the next launch
+  __shared__ int s_last;
+  __syncthreads();
+  if (tid == 0) {
+    __threadfence();
+    s_last = atomicAdd(P.ticket, 1u) == G - 1 ? 1 : 0;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (reduced) {
+    for (int e = tid >> 5; e <= E; e += (int)blockDim.x >> 5) {
+      double v = 0.0;
+      for (uint32_t i = lane; i < G; i += 32) v += __ldcg(&P.partials[(size_t)e * G + i]);
+      v = warp_sum(v);
+      if (lane == 0) s_err[e] = (e < E && P.single == 0) ? (19.0 / 270.0) * sqrt(v) : v;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      if (P.single == 7) {
+        P.slots[kSlotDot] = s_err[E];
+        P.slots[kSlotDotIm] = s_err[0];
+      } else {
+        P.slots[kSlotNorm2] = s_err[E];
+        double m = P.slots[kSlotMaxErr];
+        for (int e = 0; e < E; e++)
+          if (!(s_err[e] <= m)) m = s_err[e];  // NaN propagates
+        P.slots[kSlotMaxErr] = m;
+        P.slots[kSlotLastErr] = s_err[E - 1];
+      }
+    }
+  }
+  for (uint32_t i = tid; i < ntiles; i += blockDim.x) P.flags[kResFlagStride * i] = 0u;
+  if (tid == 0) *P.ticket = 0u;
+}
+
+template <typename R, int S, bool REG, bool PEC, bool COMP>
+cudaError_t launch_t(const ResParams& p, int nth, int max_grid, int n_z, cudaStream_t s) {
+  const size_t smem = ResSmem<R>(1u << p.t, p.nbuf, p.np, p.ng, n_z, nth, !REG).total;
+  auto kern = k_resident<R, S, REG, PEC, COMP>;
+  static int configured = 0;
+  if ((int)smem > configured) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    configured = (int)smem;
+  }
+  int grid = 1 << (p.n - p.t);
+  if (grid > max_grid) grid = max_grid;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;  // CTAs that wait on one another are resident together
+  attr[0].val.cooperative = 1;
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(nth + kService);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = p.evals > 1 && grid > 1 ? 1 : 0;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, p);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <typename R, int S, bool REG>
+cudaError_t launch_c(const ResParams& p, int nth, int max_grid, int n_z, cudaStream_t s) {
+  if (p.n_pec == 0) return launch_t<R, S, REG, false, false>(p, nth, max_grid, n_z, s);
+  return p.ylo ? launch_t<R, S, REG, true, sizeof(R) == 4>(p, nth, max_grid, n_z, s)
+               : launch_t<R, S, REG, true, false>(p, nth, max_grid, n_z, s);
+}
+
+template <typename R>
+cudaError_t launch_r(const ResParams& p, int slots, int nth, int max_grid, int n_z, cudaStream_t s) {
+  const bool reg = (1 << (p.n - p.t)) <= max_grid;
+  switch (slots) {
+    case 1: return reg ? launch_c<R, 1, true>(p, nth, max_grid, n_z, s) : launch_c<R, 1, false>(p, nth, max_grid, n_z, s);
+    case 2: return reg ? launch_c<R, 2, true>(p, nth, max_grid, n_z, s) : launch_c<R, 2, false>(p, nth, max_grid, n_z, s);
+    case 4: return launch_c<R, 4, false>(p, nth, max_grid, n_z, s);
+    case 8: return launch_c<R, 8, false>(p, nth, max_grid, n_z, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+size_t resident_smem_bytes(int prec, int t, int nbuf, int np, int ng, int n_z, int nth, bool reg) {
+  const uint32_t tsize = 1u << t;
+  return prec == 0 ? ResSmem<double>(tsize, nbuf, np, ng, n_z, nth, !reg).total
+                   : ResSmem<float>(tsize, nbuf, np, ng, n_z, nth, !reg).total;
+}
+
+cudaError_t launch_resident(int prec, const ResParams& p, int slots, int nth, int max_grid, int n_z, cudaStream_t s) {
+  return prec == 0 ? launch_r<double>(p, slots, nth, max_grid, n_z, s) : launch_r<float>(p, slots, nth, max_grid, n_z, s);
+}
+
+}  // namespace aqc
