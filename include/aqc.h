@@ -233,7 +233,7 @@ int aqc_set_slab_bits(aqc_ctx *ctx, int slab_bits);
  * schedule weights, computed on the host by the same expression as the step-by-step path, into
  * the workspace; results are bit-identical to k_steps = 0.  k_steps: 0 = off, -1 = automatic
  * (default: off for n > 20; up to there K = 16, or 64 where one launch keeps the whole state on
- * the GPU for the K steps: AQC_C64 up to n = 20, AQC_C128 up to n = 19, with the default tiles and
+ * the GPU for the K steps: AQC_C64 up to n = 20, AQC_C128 up to n = 18, with the default tiles and
  * pass order), or a multiple of 4 in [4, 64].  The graph is
  * recaptured when the tables, the step size or the vectors change, and is not used under
  * step-size control, the slab order or a clause-by-clause sequence (those steps run one by

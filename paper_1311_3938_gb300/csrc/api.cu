@@ -260,10 +260,11 @@ struct DeviceGuard {
   }
 };
 
-// Largest sizes of resident launches: 128 tiles of 2^13 complex64 or 2^12 complex128 amplitudes,
-// one beside two partner buffers in a multiprocessor's shared memory.  (complex128 n = 20 on 256
-// tiles measured 182 us per step, on the layout passes 177 us: both at the FP64 rate.)
-constexpr int kResMaxN[2] = {19, 20};  // by precision
+// Largest sizes of resident launches: 128 tiles of 2^13 complex64 or 2^11 complex128 amplitudes, one
+// beside its partner buffers in a multiprocessor's shared memory.  (complex128, microseconds per step
+// resident / on layout passes, linear, nonlinear and XY path: n = 18 41 / 72, 81 / 164, 86 / 191;
+// n = 19 83 / 74, 169 / 180, 306 / 199.)
+constexpr int kResMaxN[2] = {18, 20};  // by precision
 
 uint32_t layout_mask(const Layout& L) {
   uint32_t m = L.c >= 32 ? 0xffffffffu : ((1u << L.c) - 1u);
@@ -636,6 +637,13 @@ int build_tables(aqc_ctx* c) {
         if ((f.zm != 0 || f.has2) && !is_hop(f)) t->flips[pos + k++] = f;
     } else {
       for (const DevFlip& f : per[l]) t->flips[pos + k++] = f;
+    }
+    // 4: below that the conversion costs more than the products; 16: the bits left for the sum
+    if (l < nl && c->prec == AQC_C128 && np >= 4 && np <= 16 && (int)per[l].size() == np) {
+      bool same = true;
+      for (int i = 1; i < np; i++)
+        same = same && t->flips[pos + i].coef == t->flips[pos].coef && t->flips[pos + i].group == t->flips[pos].group;
+      t->uniform_count[l] = same ? np : 0;
     }
     t->hop_count[l] = nh;
     t->plain_count[l] = np;

@@ -95,6 +95,8 @@ struct DevTables {
                                     // flip (class 0: neither, 1: the pair bit, 2: the half
                                     // bit, 3: both); ends of classes 0..2 within the hops'
                                     // range, class 3 ends at hop_count
+  int uniform_count[kMaxLayouts + 2];  // complex128: plain_count where a layout holds nothing but
+                                    // X strings of one coefficient and group (4 to 16), else 0
   int n_z;
   int n_classes;
   int table_class;                  // clause class whose counts are in the per-index byte table, or -1

@@ -59,6 +59,39 @@ struct PFlip<double> {
   double c;
 };
 
+// ---- sums of equal-coefficient products in 64-bit integers (complex128) -------------------------
+// FP64 instructions are the scarce resource of the complex128 passes (a warp's instruction holds
+// the pipe for about 19 cycles; integer instructions run about 40 times as fast).  The products of
+// the X driver share one coefficient, so their part of H psi is c * (sum of the partners): a tile's
+// amplitudes are converted once to integers scaled by the tile's largest exponent, summed exactly,
+// and the sum is converted back: two FP64 operations per amplitude instead of two per product.
+// Accuracy: the scale leaves the sum of the tile's products just below 2^62, so with up to 16
+// products an amplitude keeps 58 bits below the tile's largest one, and sums of them round once;
+// FP64 rounds every partial sum to 53 bits.
+__device__ __forceinline__ int64_t to_fixed(double v, int emax, int up) {
+  const int64_t b = __double_as_longlong(v);
+  const int e = (int)((b >> 52) & 0x7ff);
+  int64_t m = b & 0xfffffffffffffll;
+  if (e) m |= 1ll << 52;
+  const int sh = up - (emax - (e ? e : 1));
+  int64_t r;
+  if (sh >= 0)
+    r = m << sh;
+  else
+    r = sh < -62 ? 0 : (m + (1ll << (-sh - 1))) >> -sh;
+  return b < 0 ? -r : r;
+}
+// nearest double of an integer (ties upward), in integer instructions
+__device__ __forceinline__ double from_fixed(int64_t s) {
+  const uint64_t a = s < 0 ? (uint64_t)-s : (uint64_t)s;
+  if (a == 0) return 0.0;
+  const int lz = __clzll((long long)a);
+  const uint64_t t = a << lz;                          // leading bit at 63
+  const uint64_t m = (t >> 11) + ((t >> 10) & 1u);     // 53 bits; a carry moves into the exponent
+  const uint64_t b = ((uint64_t)(1022 + 63 - lz) << 52) + m;
+  return __longlong_as_double((long long)(b | (s < 0 ? 0x8000000000000000ull : 0ull)));
+}
+
 template <typename R>
 struct SZ {
   uint32_t zm;
@@ -232,6 +265,8 @@ struct TileCtx {
   Layout L;
   uint32_t tsize, tmask;
   int np, npf, nh, ngl, ng, nz, ncls, tcls, stage;
+  int nu;     // all np products are equal-coefficient X strings summed as integers (complex128), or 0
+  int up;     // their scale: left shift of the tile's largest exponent
   int hc[3];  // ends of hop classes 0..2 (DevTables::hop_class_end)
   R dconst, wtab, h;
   // h/24 of the PEC corrector and predictor as a sum hi + lo of two state-precision numbers
@@ -286,6 +321,8 @@ __device__ __forceinline__ void load_coefficients(TileCtx<R>& T, const DevTables
   T.hc[1] = tab->hop_class_end[li][1];
   T.hc[2] = tab->hop_class_end[li][2];
   T.ngl = tab->flip_begin[li + 1] - fb - T.np;
+  T.nu = sizeof(R) == 8 ? tab->uniform_count[li] : 0;
+  T.up = 62 - 53 - (32 - __clz(T.nu > 0 ? T.nu - 1 : 0));
   const int rb = tab->flip_begin[tab->n_layouts];
   const int nrem = with_remote ? tab->n_remote : 0;
   T.ng = T.ngl + nrem;
@@ -505,6 +542,39 @@ __device__ __forceinline__ void process_tile(const TileCtx<R>& T, uint32_t zb, u
   tile_sync<CL>();  // every part of the tile is staged
 
   const bool full = tsize >= 2 * HB;  // every state with more than 6 (complex64) / 5 qubits
+  // equal-coefficient products as integers: the tile is converted in place
+  bool uni = sizeof(R) == 8 && !CL && full && T.nu > 0;
+  double uscale = 0.0;
+  if constexpr (sizeof(R) == 8 && !CL) {
+    if (uni) {
+      uint32_t m = 0;
+      for (uint32_t j = threadIdx.x; j < tsize; j += blockDim.x) {
+        const C2 v = s_p[j];
+        m = max(m, max((uint32_t)__double2hiint(v.x) & 0x7fffffffu, (uint32_t)__double2hiint(v.y) & 0x7fffffffu));
+      }
+      m = __reduce_max_sync(0xffffffffu, m);
+      uint32_t* const s_max = reinterpret_cast<uint32_t*>(T.s_red);
+      if ((threadIdx.x & 31u) == 0u) s_max[threadIdx.x >> 5] = m;
+      __syncthreads();
+      m = 0;
+      for (uint32_t w = 0; w < (blockDim.x >> 5); w++) m = max(m, s_max[w]);
+      const int emax = (int)(m >> 20);
+      // tiles with infinities or NaN, and tiles so small that the scale would be subnormal, keep
+      // the FP64 products
+      uni = emax < 0x7ff && emax >= 256;
+      if (uni) {
+        for (uint32_t j = threadIdx.x; j < tsize; j += blockDim.x) {
+          const C2 v = s_p[j];
+          longlong2 q;
+          q.x = to_fixed(v.x, emax, T.up);
+          q.y = to_fixed(v.y, emax, T.up);
+          reinterpret_cast<longlong2*>(s_p)[j] = q;
+        }
+        uscale = T.s_pf[0].c * __longlong_as_double((long long)(emax - 1075 - T.up + 1023) << 52);
+        __syncthreads();
+      }
+    }
+  }
   const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   // the partial sum q and the clause bytes of a block are fetched one iteration ahead (software
   // pipelining), so their latency overlaps the previous block's work
@@ -626,7 +696,20 @@ __device__ __forceinline__ void process_tile(const TileCtx<R>& T, uint32_t zb, u
     }
     // own values of the source
     C2 own[G];
-    if (full) {
+    if (sizeof(R) == 8 && uni) {  // the tile holds integers: from memory (L2) where they are needed
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+        C2 t[H];
+        if (MODE != MODE_PARTIAL || T.nz > 0 || T.ncls > 0 || T.dconst != (R)0) {
+          ld16cg<C2, H>(src, zh[k], t);
+        } else {
+#pragma unroll
+          for (int q = 0; q < H; q++) t[q] = zero2;
+        }
+#pragma unroll
+        for (int q = 0; q < H; q++) own[k * H + q] = t[q];
+      }
+    } else if (full) {
       C2 t0[H], t1[H];
       ld16<C2, H>(s_p, jh[0], t0);
       ld16<C2, H>(s_p, jh[1], t1);
@@ -696,8 +779,28 @@ __device__ __forceinline__ void process_tile(const TileCtx<R>& T, uint32_t zb, u
       ar[g] = kFp64 ? qv[g].x : (R)0;
       ai[g] = kFp64 ? qv[g].y : (R)0;
     }
+    if constexpr (kFp64 && !CL) {
+      if (uni) {
+        int64_t sr[2] = {0, 0}, si[2] = {0, 0};
+        const longlong2* const qt = reinterpret_cast<const longlong2*>(s_p);
+#pragma unroll 4
+        for (int kk = 0; kk < T.nu; kk++) {
+          const uint32_t lx = T.s_pf[kk].lx;
+          const longlong2 a0 = qt[jh[0] ^ lx], a1 = qt[jh[1] ^ lx];
+          sr[0] += a0.x;
+          si[0] += a0.y;
+          sr[1] += a1.x;
+          si[1] += a1.y;
+        }
+#pragma unroll
+        for (int g = 0; g < 2; g++) {
+          ar[g] = fma((double)uscale, from_fixed(sr[g]), (double)ar[g]);
+          ai[g] = fma((double)uscale, from_fixed(si[g]), (double)ai[g]);
+        }
+      }
+    }
     // products flipping no register-held bit: one 16-byte shared load per half, no selects
-    if (full) {
+    if (full && !uni) {
       for (int kk = 0; kk < T.npf; kk++) {
         const PFlip<R> f = T.s_pf[kk];
         const uint32_t rk = f.lx >> pbits, lxl = f.lx & tmask;
@@ -714,7 +817,7 @@ __device__ __forceinline__ void process_tile(const TileCtx<R>& T, uint32_t zb, u
         }
       }
     }
-    for (int kk = full ? T.npf : 0; kk < T.np; kk++) {
+    for (int kk = uni ? T.np : (full ? T.npf : 0); kk < T.np; kk++) {
       const PFlip<R> f = T.s_pf[kk];
       C2 u[G];
       gather(f.lx, u);

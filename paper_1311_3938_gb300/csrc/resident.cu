@@ -26,7 +26,7 @@
 // Measured, microseconds per predictor-corrector step (before: one launch per layout pass, replayed
 // from a graph, each on as many CTAs as the state has 64 KiB tiles):
 //   complex64, nonlinear path: n = 12 31 -> 3.8, n = 16 43 -> 5.4, n = 18 46 -> 10.5, n = 20 50 -> 36
-//   complex128, linear path:   n = 10 20 -> 3.4, n = 16 about 55 -> 10.4, n = 19 88 -> 82
+//   complex128, linear path:   n = 10 20 -> 3.4, n = 16 about 55 -> 10.4, n = 18 72 -> 41
 // Below n = 14 a step is the exchange (about 1.5 us from the last store to the first partner read)
 // and one pass of dependent shared-memory reads; above it complex64 is bound by the
 // shared-memory reads of the partners (16 bytes per product and slot), complex128 by the FP64 pipe.

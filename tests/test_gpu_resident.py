@@ -1,4 +1,4 @@
-"""Resident launches (states up to 20 qubits in complex64, 19 in complex128): one launch runs many
+"""Resident launches (states up to 20 qubits in complex64, 18 in complex128): one launch runs many
 evaluations, tiles exchange the vector H acts on through partner copies.  Sizes at the edges of
 the tile rule (one tile; the first size with several; one, two, four and eight slots per thread),
 Hamiltonians with every kind of product, the options that change the launch, against the oracle
