@@ -86,9 +86,14 @@ std::vector<Layout> layouts_for(int n, int prec, int tile_bits, bool allow_clust
 }
 
 
+// partials of the reductions: two per k_apply CTA, one per k_norm2 CTA, (64 + 1) x 128 of a resident
+// launch; the ResArea lies behind them
+constexpr size_t kResPartials = (kResMaxEvals + 1) * 152;
+
 struct WsPlan {
   size_t off_tab, off_slots, off_counter, off_sync, off_perm, off_wdev, off_partials, off_dcode, off_vec, vec_bytes, total;
   size_t partial_doubles;
+  size_t off_res;  // ResArea, in the tail of the partials (no reduction uses that many)
 };
 
 WsPlan plan_workspace(int n, int prec, unsigned flags = 0) {
@@ -104,6 +109,8 @@ WsPlan plan_workspace(int n, int prec, unsigned flags = 0) {
   // k_apply grids are persistent (at most kMaxApplyGrid CTAs); k_norm2 uses reduce_grid()
   size_t g = std::max((size_t)kMaxApplyGrid, (size_t)reduce_grid((uint64_t)1 << n));
   w.partial_doubles = 3 * g;
+  w.off_res = w.off_partials + kResPartials * sizeof(double);
+  static_assert(kResPartials * sizeof(double) + sizeof(ResArea) <= 3 * kMaxApplyGrid * sizeof(double), "partials");
   w.off_dcode = align_up(w.off_partials + w.partial_doubles * sizeof(double), 256);
   w.off_vec = align_up(w.off_dcode + ((size_t)1 << n), 256);
   w.vec_bytes = align_up(((size_t)1 << n) * amp, 256);
@@ -120,7 +127,7 @@ thread_local std::string g_create_error;
 struct ResPlan {
   bool on = false;
   int t = 0, nth = 0, slots = 0;         // tile bits, threads that own amplitudes, slots per thread
-  int np = 0, ng = 0, npart = 0, nbuf = 0;  // as in ResParams
+  int np = 0, ng = 0, npart = 0, nbuf = 0, nruns = 0;  // as in ResParams
   int ncode = 0;
 };
 
@@ -140,6 +147,8 @@ struct aqc_ctx {
   double* d_partials = nullptr;
   uint8_t* d_dcode = nullptr;
   DevTables* h_tab = nullptr;
+  ResArea h_res;            // resident launches' tables, host side
+  ResArea* d_res = nullptr;
 
   std::vector<TermH> terms;
   std::vector<ClauseH> clauses;
@@ -266,6 +275,8 @@ struct DeviceGuard {
 // n = 19 83 / 74, 169 / 180, 306 / 199.)
 constexpr int kResMaxN[2] = {18, 20};  // by precision
 
+constexpr size_t kResSmem = 222 * 1024;  // dynamic shared memory of a resident CTA (beside 5 KiB static)
+
 uint32_t layout_mask(const Layout& L) {
   uint32_t m = L.c >= 32 ? 0xffffffffu : ((1u << L.c) - 1u);
   if (L.w > 0) m |= ((1u << L.w) - 1u) << L.h;
@@ -329,11 +340,9 @@ int to_library_order(aqc_ctx* c, void* dst, const void* src) { return permute_ga
 // library order -> qubit order: dst[z] = src[perm(z)]
 int to_qubit_order(aqc_ctx* c, void* dst, const void* src) { return permute_gather(c, dst, src, c->perm); }
 
-// Sizes that resident launches take (the default tiles; a context that asks for tiles of its own
-// gets them, and so does a batch member, whose steps run on the batch's tiles).
-bool resident_size(const aqc_ctx* c) {
-  return c->tile_bits == 0 && !c->in_batch && c->n <= kResMaxN[c->prec];
-}
+// Sizes that resident launches take (with the default tiles: a context that asks for tiles of its
+// own gets them).
+bool resident_size(const aqc_ctx* c) { return c->tile_bits == 0 && c->n <= kResMaxN[c->prec]; }
 
 // Order that minimises the products (weighted by how many share a flip mask) that no layout
 // holds: deterministic local search over transpositions, kept only if strictly better than the
@@ -446,7 +455,68 @@ void plan_slabs(aqc_ctx* c) {
   S.done = c->d_sync + 1;
 }
 
-// Shape of the resident launches and the order of their products (res_idx, res_part).
+// Products of a resident launch on tiles of 2^R.t by partner tile (the bits they flip above t; the
+// own tile, no such bit, first) into `rt`, and their counts and buffers into R.  False where the
+// tables leave no room for two partner buffers: such products stay on the layout passes.
+bool resident_tables(const aqc_ctx* c, ResPlan& R, ResTable* rt) {
+  const DevTables* t = c->h_tab;
+  const int total = t->flip_begin[t->n_layouts + 1];
+  auto plain = [&](const DevFlip& f) { return f.zm == 0 && !f.has2; };
+  auto hop = [&](const DevFlip& f) {
+    return f.has2 && f.zm == 0 && f.zm2 == f.x && (f.ipow2 & 3) == 2 && f.group2 == f.group && f.coef2 == f.coef &&
+           __builtin_popcount(f.x) == 2;
+  };
+  std::vector<uint32_t> hi(1, 0u);
+  for (int i = 0; i < total; i++) hi.push_back(t->flips[i].x >> R.t);
+  std::sort(hi.begin(), hi.end());
+  hi.erase(std::unique(hi.begin(), hi.end()), hi.end());
+  if (hi.size() > (size_t)kResMaxTiles) return false;
+  R.np = 0;
+  for (int i = 0; i < total; i++) R.np += plain(t->flips[i]) ? 1 : 0;
+  R.ng = total - R.np;
+  R.npart = (int)hi.size() - 1;
+  if (t->table_class >= 0) {
+    const DevClass& cl = t->classes[t->table_class];
+    R.ncode = (cl.pen == AQC_PEN_SQUARED ? 4 : 1) * (cl.end - cl.begin);
+  }
+  // a buffer per partner while they fit (two at least, so that one fills while the other is read),
+  // and four for the owned vectors' quarter tiles where they come through the buffers
+  R.nbuf = R.npart ? R.npart + (R.slots >= 4 ? 4 : 0) : 0;
+  auto bytes = [&]() { return resident_smem_bytes(c->prec, R.t, R.nbuf, R.np, R.ng, t->n_z, R.nth, false); };
+  while (R.nbuf > 2 && bytes() > kResSmem) R.nbuf--;
+  if (bytes() > kResSmem) return false;
+  // runs of one kind, cut between partners where those come one by one (the kernel's ring), between
+  // the own tile and the others everywhere
+  const bool ring = R.nbuf > 0 && (R.slots >= 4 || R.npart > R.nbuf);
+  std::vector<int> order(total);
+  for (int i = 0; i < total; i++) order[i] = i;
+  std::sort(order.begin(), order.end(), [&](int a, int b) { return t->flips[a].x < t->flips[b].x; });
+  int np = 0, ng = 0, nr = 0;
+  size_t d = 0;  // partner of the product before
+  rt->part[0] = ResPartner{0, 0};
+  bool cut = true;
+  for (int i : order) {
+    const DevFlip& f = t->flips[i];
+    while (hi[d] != (f.x >> R.t)) {
+      d++;
+      rt->part[d] = ResPartner{(uint16_t)hi[d], (uint16_t)nr};
+      cut = cut || ring || d == 1;
+    }
+    const int kind = plain(f) ? 0 : (hop(f) ? 1 : 2);
+    rt->idx[kind == 0 ? np++ : R.np + ng++] = (uint16_t)i;
+    if (cut || rt->run[nr - 1].kind != kind) {
+      if (nr == kResMaxRuns) return false;
+      rt->run[nr++].kind = (uint16_t)kind;
+      cut = false;
+    }
+    rt->run[nr - 1].end = (uint16_t)(kind == 0 ? np : ng);
+    rt->part[d].run_end = (uint16_t)nr;
+  }
+  R.nruns = nr;
+  return true;
+}
+
+// Shape of the context's own resident launches.
 void plan_resident(aqc_ctx* c) {
   DevTables* t = c->h_tab;
   c->res = ResPlan();
@@ -464,45 +534,7 @@ void plan_resident(aqc_ctx* c) {
   const int slots_all = std::max(1, (1 << R.t) / H);
   R.nth = std::max(32, std::min(kResMaxThreads, slots_all));
   R.slots = std::max(1, slots_all / R.nth);
-  // products by partner tile: the bits they flip above t, the own tile (no such bit) first
-  const int total = t->flip_begin[t->n_layouts + 1];
-  auto plain = [&](const DevFlip& f) { return f.zm == 0 && !f.has2; };
-  auto hop = [&](const DevFlip& f) {
-    return f.has2 && f.zm == 0 && f.zm2 == f.x && (f.ipow2 & 3) == 2 && f.group2 == f.group && f.coef2 == f.coef &&
-           __builtin_popcount(f.x) == 2;
-  };
-  std::vector<uint32_t> hi(1, 0u);
-  for (int i = 0; i < total; i++) hi.push_back(t->flips[i].x >> R.t);
-  std::sort(hi.begin(), hi.end());
-  hi.erase(std::unique(hi.begin(), hi.end()), hi.end());
-  for (int i = 0; i < total; i++) R.np += plain(t->flips[i]) ? 1 : 0;
-  R.ng = total - R.np;
-  R.npart = (int)hi.size() - 1;
-  int np = 0, ng = 0;
-  for (size_t d = 0; d < hi.size(); d++) {
-    ResPartner& pt = t->res_part[d];
-    pt.hi = (uint16_t)hi[d];
-    for (int pass = 0; pass < 3; pass++) {  // X strings with real coefficients, hops, the rest
-      for (int i = 0; i < total; i++) {
-        const DevFlip& f = t->flips[i];
-        if ((f.x >> R.t) != hi[d] || pass != (plain(f) ? 0 : (hop(f) ? 1 : 2))) continue;
-        t->res_idx[pass == 0 ? np++ : R.np + ng++] = (uint16_t)i;
-      }
-      if (pass == 1) pt.hop_end = (uint16_t)ng;
-    }
-    pt.plain_end = (uint16_t)np;
-    pt.gen_end = (uint16_t)ng;
-  }
-  if (t->table_class >= 0) {
-    const DevClass& cl = t->classes[t->table_class];
-    R.ncode = (cl.pen == AQC_PEN_SQUARED ? 4 : 1) * (cl.end - cl.begin);
-  }
-  // as many partner buffers as fit (two at least, so that one fills while the other is read);
-  // products whose tables leave no room stay on the layout passes
-  R.nbuf = R.npart ? R.npart + (R.slots >= 4 ? 4 : 0) : 0;
-  auto bytes = [&]() { return resident_smem_bytes(c->prec, R.t, R.nbuf, R.np, R.ng, t->n_z, R.nth, false); };
-  while (R.nbuf > 2 && bytes() > 222 * 1024) R.nbuf--;
-  R.on = bytes() <= 222 * 1024;
+  R.on = resident_tables(c, R, &c->h_res.alone);
   c->res = R;
 }
 
@@ -741,6 +773,8 @@ int build_tables(aqc_ctx* c) {
   c->step_m = c->step_class >= 0 ? classes[c->step_class].end - classes[c->step_class].begin : 0;
   c->table_class = t->table_class;
   CUDA_TRY(c, cudaMemcpyAsync(c->d_tab, t, sizeof(DevTables), cudaMemcpyHostToDevice, c->stream));
+  if (c->res.on)
+    CUDA_TRY(c, cudaMemcpyAsync(&c->d_res->alone, &c->h_res.alone, sizeof(ResTable), cudaMemcpyHostToDevice, c->stream));
   if (t->table_class >= 0) {
     CUDA_TRY(c, launch_diag_codes(c->d_dcode, c->N, c->d_tab, t->table_class, c->stream));
     c->launches++;
@@ -867,12 +901,14 @@ ResParams resident_params(aqc_ctx* c) {
   memset(&p, 0, sizeof(p));
   const ResPlan& R = c->res;
   p.tab = c->d_tab;
+  p.rt = &c->d_res->alone;
   p.n = c->n;
   p.t = R.t;
   p.np = R.np;
   p.ng = R.ng;
   p.npart = R.npart;
   p.nbuf = R.nbuf;
+  p.nruns = R.nruns;
   p.ncode = R.ncode;
   p.dcode = c->table_class >= 0 ? c->d_dcode : nullptr;
   p.h = c->h;
@@ -1440,6 +1476,17 @@ struct aqc_batch {
   int nitems[kMaxLayouts] = {0};
   int smem[kMaxLayouts] = {0};
   int nlevels = 0;
+  // resident members (res[slot]) run in waves, one launch each
+  struct Wave {
+    int slots, ctas;
+    size_t smem;
+    ResBatch members;
+  };
+  std::vector<char> res;
+  std::vector<int> res_t;  // tile bits of the member's batch tables on the device, or 0
+  std::vector<Wave> waves;
+  int sms = 0;
+  bool pulled = true;  // h_insts holds what the device has
   bool dirty = true;
   cudaGraphExec_t gexec = nullptr;
   cudaGraph_t graph = nullptr;
@@ -1493,11 +1540,14 @@ void fill_inst(const aqc_ctx* c, BatchInst* I) {
   I->nsteps = c->nsteps;
 }
 
+// The members' records as the device has them (waits for the batch stream), unless the host copy
+// is as new.
 int batch_pull(aqc_batch* b) {
-  if (b->max_members == 0) return AQC_OK;
+  if (b->max_members == 0 || b->pulled) return AQC_OK;
   BCUDA(b, cudaMemcpyAsync(b->h_insts.data(), b->d_insts, sizeof(BatchInst) * b->max_members, cudaMemcpyDeviceToHost,
                            b->stream));
   BCUDA(b, cudaStreamSynchronize(b->stream));
+  b->pulled = true;
   return AQC_OK;
 }
 
@@ -1508,16 +1558,124 @@ void drop_graph(aqc_batch* b) {
   b->graph = nullptr;
 }
 
+// A resident member on tiles of at most 2^tb: tile bits, slots per thread and CTAs.
+ResPlan member_plan(const aqc_ctx* c, int tb) {
+  ResPlan R;
+  R.t = std::min(c->n, tb);
+  R.nth = kResMaxThreads;
+  R.slots = std::max(1, (1 << R.t) / ((c->prec == AQC_C128 ? 1 : 2) * kResMaxThreads));
+  return R;
+}
+
+// Estimated microseconds of one step on a tile of 2^t amplitudes with `np` products.  Fitted to
+// steps of one state: complex64 on 2^10 / 2^12 / 2^13 tiles 5.3 / 13 / 24 us at 54 products, 15 at
+// 14 products on 2^13; complex128 (at the FP64 rate) 70 and 126 us on 2^12 at 14 and 42.
+double tile_cost(const aqc_ctx* c, int t) {
+  const DevTables* h = c->h_tab;
+  const double np = h->flip_begin[h->n_layouts + 1], amps = (double)(1 << t);
+  return c->prec == AQC_C128 ? 3.0 + amps * (2.0 * np + 24.0) * 3.5e-4 : 2.5 + amps * (9e-4 + 4e-5 * np);
+}
+
+// Waves of the resident members: a common tile size, the members of one slot count packed into
+// launches of at most one CTA per multiprocessor.  Larger tiles use a multiprocessor better (fewer
+// exchanges and partner copies per amplitude), smaller ones keep more of them busy: the size with
+// the least estimated time for one step of every member is taken.
+int batch_plan_waves(aqc_batch* b) {
+  b->waves.clear();
+  std::vector<int> who;
+  for (int slot = 0; slot < b->max_members; slot++)
+    if (b->members[slot] && b->res[slot]) who.push_back(slot);
+  if (who.empty()) return AQC_OK;
+  struct Job {
+    int slot, slots, ctas;
+    double cost;
+  };
+  auto pack = [&](int tb, std::vector<std::vector<Job>>* out) {  // estimated time, or infinity
+    double total = 0.0;
+    for (int S = 1; S <= 8; S *= 2) {
+      std::vector<Job> jobs;
+      for (int slot : who) {
+        const aqc_ctx* c = b->members[slot];
+        const ResPlan R = member_plan(c, tb);
+        if (R.slots != S) continue;
+        jobs.push_back(Job{slot, S, 1 << (c->n - R.t), tile_cost(c, R.t)});
+        if (jobs.back().ctas > std::min(b->sms, 128)) return (double)INFINITY;
+      }
+      std::stable_sort(jobs.begin(), jobs.end(), [](const Job& x, const Job& y) { return x.ctas > y.ctas; });
+      std::vector<std::vector<Job>> waves;
+      std::vector<int> room;
+      for (const Job& j : jobs) {
+        size_t w = 0;
+        while (w < waves.size() && room[w] < j.ctas) w++;
+        if (w == waves.size()) {
+          waves.emplace_back();
+          room.push_back(std::min(b->sms, kResMaxCtas));
+        }
+        waves[w].push_back(j);
+        room[w] -= j.ctas;
+      }
+      for (const auto& w : waves) {
+        double t = 0.0;
+        for (const Job& j : w) t = std::max(t, j.cost);
+        total += t;
+        if (out) out->push_back(w);
+      }
+    }
+    return total;
+  };
+  const int hi = b->prec == AQC_C128 ? 12 : 13;
+  int best = hi;
+  double least = INFINITY;
+  for (int tb = hi; tb >= 9; tb--) {
+    const double t = pack(tb, nullptr);
+    if (t < least) {
+      least = t;
+      best = tb;
+    }
+  }
+  std::vector<std::vector<Job>> waves;
+  pack(best, &waves);
+  for (const auto& w : waves) {
+    b->waves.emplace_back();
+    aqc_batch::Wave& W = b->waves.back();
+    W.slots = w[0].slots;
+    W.ctas = 0;
+    W.smem = 0;
+    memset(&W.members, 0, sizeof(W.members));
+    W.members.insts = b->d_insts;
+    for (const Job& j : w) {
+      aqc_ctx* c = b->members[j.slot];
+      ResPlan R = member_plan(c, best);
+      if (!resident_tables(c, R, &c->h_res.batch)) BFAIL(b, AQC_E_UNSUPPORTED, "member tables too large");
+      if (b->res_t[j.slot] != R.t) {
+        c->h_res.member = ResMember{c->n, R.t, R.np, R.ng, R.npart, R.nbuf, R.nruns, R.ncode, c->d_sync + 1, c->d_sync,
+                                    c->d_partials, c->d_slots};
+        BCUDA(b, cudaMemcpyAsync(&c->d_res->batch, &c->h_res.batch, sizeof(ResTable) + sizeof(ResMember),
+                                 cudaMemcpyHostToDevice, b->stream));
+        b->res_t[j.slot] = R.t;
+      }
+      W.members.area = c->wp.off_res - c->wp.off_tab;
+      W.members.slot[W.members.count] = (uint16_t)j.slot;
+      W.members.first[W.members.count++] = (uint16_t)W.ctas;
+      W.smem = std::max(W.smem, resident_smem_bytes(c->prec, R.t, R.nbuf, R.np, R.ng, c->n_z, R.nth, R.slots <= 2));
+      W.ctas += j.ctas;
+    }
+  }
+  BCUDA(b, cudaStreamSynchronize(b->stream));  // the members' tables are on the device
+  return AQC_OK;
+}
+
 // work lists + per-level shared memory + one captured graph of K batched grid steps
 int batch_rebuild(aqc_batch* b) {
   int rc = batch_pull(b);
+  if (!rc) rc = batch_plan_waves(b);
   if (rc) return rc;
   std::vector<BatchItem> items[kMaxLayouts];
   int smem[kMaxLayouts] = {0};
   int nlev = 0;
   for (int slot = 0; slot < b->max_members; slot++) {
     aqc_ctx* c = b->members[slot];
-    if (!c) continue;
+    if (!c || b->res[slot]) continue;
     BatchInst& I = b->h_insts[slot];
     const int nl = (int)c->layouts.size();
     nlev = std::max(nlev, nl);
@@ -1662,6 +1820,7 @@ int aqc_create(aqc_ctx** out, int device, int precision, int n_qubits, void* wor
   c->d_perm = (uint32_t*)(c->ws + wp.off_perm);
   c->d_partials = (double*)(c->ws + wp.off_partials);
   c->d_wdev = (double*)(c->ws + wp.off_wdev);
+  c->d_res = (ResArea*)(c->ws + wp.off_res);
   c->d_dcode = (uint8_t*)(c->ws + wp.off_dcode);
   for (int v = 0; v < V_COUNT; v++) c->vec[v] = c->ws + wp.off_vec + (size_t)v * wp.vec_bytes;
   if (workspace_bytes >= plan_workspace(n_qubits, precision, AQC_WS_STEP_CONTROL).total)
@@ -2437,6 +2596,9 @@ int aqc_batch_create(aqc_batch** out, int device, int precision, int max_members
   for (int l = 0; l < kMaxLayouts; l++)
     b->d_items[l] = (BatchItem*)(b->ws + bp.off_items + (size_t)l * (size_t)max_items * sizeof(BatchItem));
   b->d_partials = (double*)(b->ws + bp.off_partials);
+  b->res.assign(max_members, 0);
+  b->res_t.assign(max_members, 0);
+  if (cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) b->sms = 1;
   b->members.assign(max_members, nullptr);
   b->step_at_add.assign(max_members, 0);
   b->h_insts.assign(max_members, BatchInst());
@@ -2482,6 +2644,18 @@ int aqc_batch_set_shape(aqc_batch* b, int threads, int steps_per_round) {
   return AQC_OK;
 }
 
+// Whether a context's resident launches fit a batch's: its largest tiles on this device, its tables
+// beside them on every tile size that a wave may take.
+static bool batch_holds(const aqc_batch* b, aqc_ctx* c) {
+  const int hi = c->prec == AQC_C128 ? 12 : 13;
+  if ((1 << (c->n - std::min(c->n, hi))) > std::min(b->sms, kResMaxCtas)) return false;
+  for (int tb = 9; tb <= hi; tb++) {
+    ResPlan R = member_plan(c, tb);
+    if (c->n - R.t <= 7 && !resident_tables(c, R, &c->h_res.batch)) return false;
+  }
+  return true;
+}
+
 int aqc_batch_add(aqc_batch* b, aqc_ctx* c, int* slot_out) {
   if (!b || !c) return AQC_E_INVAL;
   if (c->device != b->device || c->prec != b->prec) BFAIL(b, AQC_E_INVAL, "context device/precision differ from the batch");
@@ -2500,40 +2674,50 @@ int aqc_batch_add(aqc_batch* b, aqc_ctx* c, int* slot_out) {
     }
   if (slot < 0) BFAIL(b, AQC_E_NOMEM, "batch is full (%d members)", b->max_members);
   DeviceGuard dg(b->device);
-  if (!c->in_batch) {
+  int rc = ensure_ready(c);
+  const bool res = rc == 0 && resident_on(c) && batch_holds(b, c);
+  if (!rc && !res && !c->in_batch) {
     c->in_batch = true;  // per-CTA tiles for the batched kernel
     c->dirty = true;
+    rc = ensure_ready(c);
   }
-  int rc = ensure_ready(c);
+  if (!rc) rc = plan_first_segment(c);
   if (rc) {
+    if (c->in_batch) c->dirty = true;
     c->in_batch = false;
-    c->dirty = true;
     BFAIL(b, rc, "member: %s", c->err.c_str());
   }
-  rc = plan_first_segment(c);
-  if (rc) {
-    c->in_batch = false;
-    c->dirty = true;
-    BFAIL(b, rc, "member: %s", c->err.c_str());
-  }
+  c->in_batch = true;
   // start-up on the batch stream: RK4 steps, f_3 and the first predictor (after the
   // context's own queued work, e.g. its initial state)
-  BCUDA(b, cudaStreamSynchronize(c->stream));
+  cudaEvent_t ev = nullptr;
+  BCUDA(b, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+  cudaError_t order = cudaEventRecord(ev, c->stream);
+  if (order == cudaSuccess) order = cudaStreamWaitEvent(b->stream, ev, 0);
+  cudaEventDestroy(ev);
+  BCUDA(b, order);
   cudaStream_t saved = c->stream;
   c->stream = b->stream;
-  while (rc == 0 && c->step < 3 && c->step < c->nsteps) {
+  if (res) {
+    const int m = (int)std::max<int64_t>(0, std::min<int64_t>(3 - c->step, c->nsteps - c->step));
+    const bool hist = !c->hist_ready && c->step + m == 3 && c->nsteps > 3;
+    if (m > 0 || hist) rc = resident_start(c, m, hist);
+    for (int i = 0; i < m && !rc; i++) count_step(c);
+  }
+  while (!res && rc == 0 && c->step < 3 && c->step < c->nsteps) {
     rc = rk4_step(c);
     if (!rc) count_step(c);
   }
-  if (rc == 0 && c->step >= 3 && c->step < c->nsteps && !c->hist_ready) rc = start_history(c);
+  if (!res && rc == 0 && c->step >= 3 && c->step < c->nsteps && !c->hist_ready) rc = start_history(c);
   c->stream = saved;
   if (rc) BFAIL(b, rc, "member start-up: %s", c->err.c_str());
-  rc = batch_pull(b);
+  rc = batch_pull(b);  // the host copies of the other members' records stay whole
   if (rc) return rc;
   fill_inst(c, &b->h_insts[slot]);
   BCUDA(b, cudaMemcpyAsync(b->d_insts + slot, &b->h_insts[slot], sizeof(BatchInst), cudaMemcpyHostToDevice, b->stream));
-  BCUDA(b, cudaStreamSynchronize(b->stream));
   b->members[slot] = c;
+  b->res[slot] = res ? 1 : 0;
+  b->res_t[slot] = 0;
   b->step_at_add[slot] = c->step;
   b->dirty = true;
   if (slot_out) *slot_out = slot;
@@ -2548,6 +2732,7 @@ int aqc_batch_remove(aqc_batch* b, int slot) {
   if (rc) return rc;
   aqc_ctx* c = b->members[slot];
   const BatchInst& I = b->h_insts[slot];
+  bool timed_out = false;
   c->evals += I.step - b->step_at_add[slot];
   c->step = I.step;
   c->steps_done = I.step;  // one segment from t = 0 (batch members run the fixed-step grid)
@@ -2565,13 +2750,24 @@ int aqc_batch_remove(aqc_batch* b, int slot) {
     cudaMemcpyAsync(c->d_slots + kSlotLastErr, &sl[2], sizeof(double), cudaMemcpyHostToDevice, b->stream);
     BCUDA(b, cudaStreamSynchronize(b->stream));
   }
+  if (b->res[slot]) {
+    double fault = 0.0;  // a wait inside a launch that gave up
+    BCUDA(b, cudaMemcpyAsync(&fault, c->d_slots + kSlotFault, sizeof(double), cudaMemcpyDeviceToHost, b->stream));
+    BCUDA(b, cudaStreamSynchronize(b->stream));
+    timed_out = fault != 0.0;
+    // the exchange vectors may have traded places
+    c->vec[V_P] = I.vec[kVecP];
+    c->vec[V_Q] = I.vec[kVecQ];
+  } else {
+    c->dirty = true;
+  }
   b->members[slot] = nullptr;
   c->in_batch = false;
-  c->dirty = true;
   memset(&b->h_insts[slot], 0, sizeof(BatchInst));
   BCUDA(b, cudaMemcpyAsync(b->d_insts + slot, &b->h_insts[slot], sizeof(BatchInst), cudaMemcpyHostToDevice, b->stream));
   BCUDA(b, cudaStreamSynchronize(b->stream));
   b->dirty = true;
+  if (timed_out) BFAIL(b, AQC_E_TIMEOUT, "a kernel gave up waiting (a partner's tile); the member's results are invalid");
   return AQC_OK;
 }
 
@@ -2582,6 +2778,15 @@ int aqc_batch_run(aqc_batch* b, int64_t rounds) {
   if (b->dirty) {
     int rc = batch_rebuild(b);
     if (rc) return rc;
+  }
+  if (rounds > 0) b->pulled = false;
+  for (const aqc_batch::Wave& w : b->waves) {
+    ResBatch rb = w.members;
+    for (int64_t left = rounds * b->steps_per_round; left > 0; left -= rb.evals) {
+      rb.evals = (int)std::min<int64_t>(left, kResMaxEvals);
+      BCUDA(b, launch_resident_batch(b->prec, rb, w.slots, w.ctas, w.smem, b->stream));
+      b->launches++;
+    }
   }
   if (!b->gexec) return AQC_OK;
   int per = 0;
@@ -2596,6 +2801,7 @@ int aqc_batch_run(aqc_batch* b, int64_t rounds) {
 int aqc_batch_poll(aqc_batch* b, int64_t* steps_done, int* active_out, int64_t* launches_out) {
   if (!b) return AQC_E_INVAL;
   DeviceGuard dg(b->device);
+  BCUDA(b, cudaStreamSynchronize(b->stream));
   int rc = batch_pull(b);
   if (rc) return rc;
   int active = 0;

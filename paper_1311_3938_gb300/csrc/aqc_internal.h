@@ -73,14 +73,24 @@ __host__ __device__ __forceinline__ uint32_t tile_z(const Layout& L, uint32_t j,
   return zb | (j & cm) | ((j >> L.c) << L.h);
 }
 
-// Products of a resident launch that read one partner tile (or the own one): ranges end at ...
+// Products of a resident launch, in ascending order of their flip mask: that order is by partner
+// tile (the bits flipped above the tile) whatever the tile size, so a result does not depend on how
+// a state was cut.  A run is a stretch of one kind.
+struct ResRun {
+  uint16_t kind;  // 0 X strings with real coefficients, 1 hops, 2 other products
+  uint16_t end;   // in the list of kind 0, or in the list of the others
+};
 struct ResPartner {
-  uint16_t hi;         // the partner is the tile whose number is the own one XOR hi (0: the own tile)
-  uint16_t plain_end;  // X strings with real coefficients, in the launch's list of them
-  uint16_t hop_end;    // hops, in the list of the other products
-  uint16_t gen_end;    // the rest
+  uint16_t hi;       // the partner is the tile whose number is the own one XOR hi (0: the own tile)
+  uint16_t run_end;  // its runs end here
 };
 constexpr int kResMaxTiles = 256;
+constexpr int kResMaxRuns = 512;
+struct ResTable {
+  uint16_t idx[kMaxFlips];  // products of kind 0, then the others
+  ResRun run[kResMaxRuns];
+  ResPartner part[kResMaxTiles];
+};
 
 struct DevTables {
   int n_layouts;
@@ -106,9 +116,6 @@ struct DevTables {
   uint32_t clause_mask[kMaxClauses];
   DevZ z[kMaxZ];
   DevFlip flips[kMaxFlips];
-  uint16_t res_idx[kMaxFlips];      // order of the products in a resident launch: the X strings with
-                                    // real coefficients by partner tile, then the others
-  ResPartner res_part[kResMaxTiles];
 };
 
 enum Mode : int {
@@ -209,9 +216,11 @@ constexpr int kResMaxEvals = 64;
 constexpr int kResFlagStride = 8;   // 32 bytes between tile flags: polls of one do not slow another
 struct ResParams {
   const DevTables* tab;
+  const ResTable* rt;
   int n, t;              // tile = 2^t consecutive indices
   int np, ng;            // X strings with real coefficients, other products
   int npart, nbuf;       // partner tiles beside the own one, shared-memory buffers for them
+  int nruns;
   int ncode;             // largest clause count in dcode
   int evals;             // evaluations in the launch
   int n_rk, hist, n_pec;
@@ -259,6 +268,28 @@ struct BatchInst {
 struct BatchItem {
   uint32_t inst;
   uint32_t tile;
+};
+
+// A batch member's resident launches: shape as in ResParams, and the flags, ticket, partials and
+// result slots of its own workspace.
+struct ResMember {
+  int n, t, np, ng, npart, nbuf, nruns, ncode;
+  unsigned *flags, *ticket;
+  double *partials, *slots;
+};
+// What resident launches keep in a context's workspace beside DevTables, behind the partials.
+struct ResArea {
+  ResTable alone, batch;
+  ResMember member;
+};
+// One resident launch of a batch: every CTA is a tile of a member; `evals` steps of each member
+// (fewer where its run ends).
+constexpr int kResMaxCtas = 160;
+struct ResBatch {
+  BatchInst* insts;
+  size_t area;    // ResArea of a member: bytes behind its DevTables
+  int evals, count;
+  uint16_t slot[kResMaxCtas], first[kResMaxCtas];  // members and their first CTAs
 };
 
 struct BatchLaunch {
@@ -333,6 +364,7 @@ size_t resident_smem_bytes(int prec, int t, int nbuf, int np, int ng, int n_z, i
 // slots: 16-byte slots per thread and tile; max_grid: CTAs at most (fewer than tiles: a CTA walks
 // several tiles and the owned vectors stay in global memory)
 cudaError_t launch_resident(int prec, const ResParams& p, int slots, int nth, int max_grid, int n_z, cudaStream_t s);
+cudaError_t launch_resident_batch(int prec, const ResBatch& b, int slots, int ctas, size_t smem, cudaStream_t s);
 int64_t fma64_count(int blocks, int iters);
 int reduce_grid(uint64_t N);
 cudaError_t launch_batch(int prec, int threads, const BatchLaunch& b, int nitems, int smem, cudaStream_t s);

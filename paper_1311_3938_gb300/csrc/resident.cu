@@ -209,7 +209,7 @@ __device__ __forceinline__ void coefficients(const ResParams& P, const double* w
     pl[k] = RPlain<R>{d.off, (R)(d.coef * pick(d.group))};
   }
   for (int k = lane; k < P.ng; k += 32) {
-    const DevFlip d = tab->flips[tab->res_idx[P.np + k]];
+    const DevFlip d = tab->flips[P.rt->idx[P.np + k]];
     double v[4] = {0.0, 0.0, 0.0, 0.0};  // c i^ipow of the product and of its companion
     auto phased = [](double c, int ipow, double* o) {
       o[0] = (ipow & 1) ? 0.0 : ((ipow & 2) ? -c : c);
@@ -279,8 +279,11 @@ __device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 0;\n" ::: "m
 // The warps take roles, each with its own loop over the evaluations: owners, the coefficients of
 // the next evaluation's products, those of its diagonal, the sums of the last one's error
 // partials, and the tile copies.
+// The body runs as one tile (number `cta` of G tiles or CTAs) of the state that P describes; inst: the
+// batch member, whose results go to its record (null: to P.slots).
 template <typename R, int S, bool REG, bool PEC, bool COMP>
-__global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const __grid_constant__ ResParams P) {
+__device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t cta, const uint32_t G,
+                                              BatchInst* const inst) {
   using C2 = typename RT<R>::C2;
   constexpr int H = RT<R>::H;
   constexpr int A = S * H;  // amplitudes per thread and tile
@@ -290,6 +293,7 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
   using RED = typename std::conditional<REG, R, double>::type;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ ResPartner s_part[kResMaxTiles];
+  __shared__ ResRun s_run[kResMaxRuns];
   __shared__ volatile int s_abort;
   __shared__ double s_err[kResMaxEvals + 2];
 
@@ -299,11 +303,11 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
   const bool owner = tid < nth;
   const int svc = (tid - nth) >> 5;  // service warp 0..3
   const uint32_t tsize = 1u << P.t, tmask = tsize - 1u, tbytes = tsize * (uint32_t)sizeof(C2);
-  const uint32_t ntiles = 1u << (P.n - P.t), G = gridDim.x;
+  const uint32_t ntiles = 1u << (P.n - P.t);
   const int np = P.np, ng = P.ng, nz = tab->n_z, ncls = tab->n_classes;
   const int nd = P.npart, nbuf = P.nbuf;  // partner tiles (beside the own one) and their buffers
   const int nq = nd + (kStream && nbuf > 0 ? 4 : 0);  // ring entries per tile visit
-  const bool ring = nq > nbuf || (kStream && nbuf > 0);  // else every partner has a buffer of its own
+  const bool ring = nbuf > 0 && (S >= 4 || nd > nbuf);  // else every partner has a buffer of its own
   const int tcls = P.dcode ? tab->table_class : -1;
   const int E = P.evals;
   const bool multi = ntiles > G;  // several tiles per CTA
@@ -328,7 +332,8 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
     }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
-  for (int k = tid; k <= nd; k += blockDim.x) s_part[k] = tab->res_part[k];
+  for (int k = tid; k <= nd; k += blockDim.x) s_part[k] = P.rt->part[k];
+  for (int k = tid; k < P.nruns; k += blockDim.x) s_run[k] = P.rt->run[k];
   for (int k = tid; k < 3 * E; k += blockDim.x)
     s_w[k] = P.wdev ? P.wdev[(size_t)P.wstride * (k / 3) + k % 3] : P.w[k];
   __syncthreads();
@@ -341,10 +346,10 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
     return (x & tmask) * (uint32_t)sizeof(C2) | p * tbytes;
   };
   for (int k = tid; k < np; k += blockDim.x) {
-    const DevFlip d = tab->flips[tab->res_idx[k]];
+    const DevFlip d = tab->flips[P.rt->idx[k]];
     s_base[k] = RBase{d.coef, place(d.x), d.group};
   }
-  for (int k = tid; k < ng; k += blockDim.x) s_gen[k].off = s_gen[ng + k].off = place(tab->flips[tab->res_idx[np + k]].x);
+  for (int k = tid; k < ng; k += blockDim.x) s_gen[k].off = s_gen[ng + k].off = place(tab->flips[P.rt->idx[np + k]].x);
   __syncthreads();
 
   // copies of partner tiles (and of owned quarter tiles) for one visit of a tile; q0: ring entries
@@ -436,7 +441,7 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
     if (REG && act && !P.single) {
 #pragma unroll
       for (int s = 0; s < S; s++) {
-        const uint32_t z = (blockIdx.x << P.t) + (uint32_t)(j0 + s * js);
+        const uint32_t z = (cta << P.t) + (uint32_t)(j0 + s * js);
         load(Y + z, o[s].y);
         if (latest >= 0) load(F(latest) + z, o[s].a);
         if (latest >= 1) load(F(latest - 1) + z, o[s].b);
@@ -453,7 +458,7 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
       const RGen<R>* const gen = s_gen + par * ng;
       const RScal<R>& sc = s_sc[par];
       RED red0 = (RED)0, red1 = (RED)0;
-      for (uint32_t tile = blockIdx.x; tile < ntiles; tile += G, visit++) {
+      for (uint32_t tile = cta; tile < ntiles; tile += G, visit++) {
         const uint32_t zb = tile << P.t;
         if (e == 0 || multi) {  // the own tile and its clause bytes (then kept up to date in place)
           if (multi) cta_sync();  // readers of the previous tile are done
@@ -532,8 +537,8 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
               }
             }
         };
-        // hops [k, hops) and other products [.., end)
-        auto general = [&](const unsigned char* t, int k, int hops, int end) {
+        // hops or other products [k, end)
+        auto general = [&](const unsigned char* t, int k, bool hop, int end) {
 #pragma unroll 1
           for (; k < end; k++) {
             const RGen<R> f = gen[k];
@@ -545,7 +550,7 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
                 const C2 w = *reinterpret_cast<const C2*>(t + (at ^ (uint32_t)(q * sizeof(C2))));
                 const int g = s * H + q;
                 const uint32_t z = zb + (uint32_t)(j0 + s * js + q);
-                if (k < hops) {  // 2c where the two bits of z differ (cr - cr2 = 2c)
+                if (hop) {  // 2c where the two bits of z differ (cr - cr2 = 2c)
                   const R cf = (__popc(f.x & z) & 1) ? f.cr - f.cr2 : (R)0;
                   ar[g] = fma_(cf, w.x, ar[g]);
                   ai[g] = fma_(cf, w.y, ai[g]);
@@ -567,21 +572,23 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
             s_abort = 1;
           }
         };
-        const unsigned char* const t0p = smem;
-        int gb = s_part[0].gen_end;
-        if (act) {
-          plain(t0p, 0, s_part[0].plain_end);
-          if (gb > 0) general(t0p, 0, s_part[0].hop_end, gb);
-        }
-        if (nd > 0 && !ring) {  // every partner in one go: the places name the buffers
-          arrived(0, visit & 1u);
-          if (act) {
-            plain(t0p, s_part[0].plain_end, np);
-            for (int p = 1; p <= nd && gb < ng; p++) {
-              general(t0p, gb, s_part[p].hop_end, s_part[p].gen_end);
-              gb = s_part[p].gen_end;
+        int pk = 0, gk = 0, run = 0;
+        auto runs_to = [&](const unsigned char* t, int end) {
+          for (; run < end; run++) {
+            const ResRun r = s_run[run];
+            if (r.kind == 0) {
+              plain(t, pk, r.end);
+              pk = r.end;
+            } else {
+              general(t, gk, r.kind == 1, r.end);
+              gk = r.end;
             }
           }
+        };
+        if (act) runs_to(smem, s_part[0].run_end);
+        if (nd > 0 && !ring) {  // every partner in one go: the places name the buffers
+          arrived(0, visit & 1u);
+          if (act) runs_to(smem, P.nruns);
         }
         uint32_t rb = ring ? q0 % (uint32_t)nbuf : 0u, ru = ring ? q0 / (uint32_t)nbuf : 0u;
         auto release = [&]() {  // this warp is done with buffer rb; on to the next ring entry
@@ -593,17 +600,9 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
           }
         };
         if (ring) {
-          int pb = s_part[0].plain_end;
           for (int p = 1; p <= nd; p++) {
-            const ResPartner pt = s_part[p];
             arrived(rb, ru & 1u);
-            if (act) {
-              const unsigned char* t = smem + (size_t)(1u + rb) * tbytes;
-              plain(t, pb, pt.plain_end);
-              if (pt.gen_end > gb) general(t, gb, pt.hop_end, pt.gen_end);
-            }
-            pb = pt.plain_end;
-            gb = pt.gen_end;
+            if (act) runs_to(smem + (size_t)(1u + rb) * tbytes, s_part[p].run_end);
             release();
           }
         }
@@ -743,7 +742,7 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
     if (REG && act && !P.single) {  // the owned vectors back to global memory
 #pragma unroll
       for (int s = 0; s < S; s++) {
-        const uint32_t z = (blockIdx.x << P.t) + (uint32_t)(j0 + s * js);
+        const uint32_t z = (cta << P.t) + (uint32_t)(j0 + s * js);
         if (E > P.hist) store((P.n_pec ? YO : Y) + z, o[s].y);
         if (latest > first_latest) store(F(latest) + z, o[s].a);
         if (latest > first_latest + 1) store(F(latest - 1) + z, o[s].b);
@@ -773,14 +772,14 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
     const C2* xin = src0;
     for (int e = 0; e < E; e++) {
       const bool last = e == E - 1;
-      for (uint32_t tile = blockIdx.x; tile < ntiles; tile += G) {
+      for (uint32_t tile = cta; tile < ntiles; tile += G) {
         if (e == 0 || multi) {
           if (multi) cta_sync();
           cta_sync();
         }
         if (svc == 3 && nq > 0) copy_in(tile, xin, e, latest, q0);
         q0 += (uint32_t)nq;
-        if (tile == blockIdx.x) {
+        if (tile == cta) {
           if (!last) prepare(e + 1);
           if (PEC && svc == 2 && e > 0) lane_sums(s_red + (size_t)((e - 1) & 1) * nth, s_lane + 8 * (e - 1));
         }
@@ -794,7 +793,7 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
       if (last) break;
       cta_sync();
       if (s_abort) break;
-      if (!multi && svc == 3 && lane == 0 && nd > 0) flag_release(P.flags + kResFlagStride * blockIdx.x, (unsigned)(e + 1));
+      if (!multi && svc == 3 && lane == 0 && nd > 0) flag_release(P.flags + kResFlagStride * cta, (unsigned)(e + 1));
       xin = e & 1 ? XO : XA;
     }
     if (s_abort && svc == 3) {  // copies in flight land before the CTA leaves (bounded)
@@ -818,7 +817,7 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
       double v = 0.0;
       if (lane == 0) {
         for (int k = 0; k < 8; k++) v += s_lane[8 * e + k];
-        P.partials[(size_t)e * G + blockIdx.x] = v;
+        P.partials[(size_t)e * G + cta] = v;
       }
     }
   }
@@ -845,17 +844,85 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
         P.slots[kSlotDot] = s_err[E];
         P.slots[kSlotDotIm] = s_err[0];
       } else {
-        P.slots[kSlotNorm2] = s_err[E];
-        double m = P.slots[kSlotMaxErr];
+        double m = inst ? inst->max_err : P.slots[kSlotMaxErr];
         for (int e = 0; e < E; e++)
           if (!(s_err[e] <= m)) m = s_err[e];  // NaN propagates
-        P.slots[kSlotMaxErr] = m;
-        P.slots[kSlotLastErr] = s_err[E - 1];
+        (inst ? inst->norm2 : P.slots[kSlotNorm2]) = s_err[E];
+        (inst ? inst->max_err : P.slots[kSlotMaxErr]) = m;
+        (inst ? inst->last_err : P.slots[kSlotLastErr]) = s_err[E - 1];
+        if (inst) {  // every CTA of the member has read its step count: on to the next steps
+          inst->step += E;
+          if (E & 1) {
+            void* const v = inst->vec[kVecP];
+            inst->vec[kVecP] = inst->vec[kVecQ];
+            inst->vec[kVecQ] = v;
+          }
+        }
       }
     }
   }
   for (uint32_t i = tid; i < ntiles; i += blockDim.x) P.flags[kResFlagStride * i] = 0u;
   if (tid == 0) *P.ticket = 0u;
+}
+
+template <typename R, int S, bool REG, bool PEC, bool COMP>
+__global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const __grid_constant__ ResParams P) {
+  resident_body<R, S, REG, PEC, COMP>(P, blockIdx.x, gridDim.x, nullptr);
+}
+
+// Predictor-corrector steps of many states in one launch: a CTA is one tile of one batch member,
+// and only the CTAs of a member exchange anything.  Weights come from the member's polynomials
+// (the expression of the host side).  A step of 24 complex64 members of 12 to 18 qubits (207 tiles
+// of 2^13) takes 53 us in three waves on tiles of 2^12; one launch per layout level over all tiles
+// took 93 us.
+template <typename R, int S>
+__global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident_batch(const __grid_constant__ ResBatch B) {
+  __shared__ ResParams P;
+  int m = 0;
+  while (m + 1 < B.count && B.first[m + 1] <= blockIdx.x) m++;
+  BatchInst* const I = B.insts + B.slot[m];
+  const int64_t step = I->step, left = I->nsteps - step;
+  if (left <= 0) return;  // finished: all its CTAs leave
+  const int E = left < (int64_t)B.evals ? (int)left : B.evals;
+  if (threadIdx.x == 0) {
+    const ResArea* const A = reinterpret_cast<const ResArea*>(reinterpret_cast<const char*>(I->tab) + B.area);
+    const ResMember M = A->member;
+    P.tab = I->tab;
+    P.rt = &A->batch;
+    P.n = M.n;
+    P.t = M.t;
+    P.np = M.np;
+    P.ng = M.ng;
+    P.npart = M.npart;
+    P.nbuf = M.nbuf;
+    P.nruns = M.nruns;
+    P.ncode = M.ncode;
+    P.evals = P.n_pec = E;
+    P.n_rk = P.hist = P.single = 0;
+    P.step0 = (int)(step & 3) + (step >= 4 ? 4 : 0);
+    P.wdev = nullptr;
+    P.wstride = 0;
+    P.h = I->h;
+    P.dcode = I->dcode;
+    P.src = I->vec[kVecP];
+    P.xout[0] = I->vec[kVecQ];
+    P.xout[1] = I->vec[kVecP];
+    P.y = P.yout = I->vec[kVecY];
+    for (int k = 0; k < 4; k++) P.f[k] = I->vec[kVecF0 + k];
+    P.acc = P.ylo = nullptr;
+    P.flags = M.flags;
+    P.ticket = M.ticket;
+    P.partials = M.partials;
+    P.slots = M.slots;
+  }
+  for (int k = threadIdx.x; k < 3 * E; k += blockDim.x) {
+    const double tau = (double)(step + k / 3 + 1) * I->h / I->T;
+    const double s = I->s_kind == 1 ? tau * tau * (3.0 - 2.0 * tau) : tau;
+    const double* const c = I->poly[k % 3];
+    P.w[k] = ((c[3] * s + c[2]) * s + c[1]) * s + c[0];
+  }
+  __syncthreads();
+  resident_body<R, S, (S <= 2), true, false>(P, blockIdx.x - B.first[m], 1u << (P.n - P.t), I);
 }
 
 template <typename R, int S, bool REG, bool PEC, bool COMP>
@@ -909,6 +976,44 @@ size_t resident_smem_bytes(int prec, int t, int nbuf, int np, int ng, int n_z, i
   const uint32_t tsize = 1u << t;
   return prec == 0 ? ResSmem<double>(tsize, nbuf, np, ng, n_z, nth, !reg).total
                    : ResSmem<float>(tsize, nbuf, np, ng, n_z, nth, !reg).total;
+}
+
+template <typename R, int S>
+static cudaError_t launch_batch_s(const ResBatch& b, int ctas, size_t smem, cudaStream_t s) {
+  auto kern = k_resident_batch<R, S>;
+  static int configured = 0;
+  if ((int)smem > configured) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    configured = (int)smem;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(kResMaxThreads + kService);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, b);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <typename R>
+static cudaError_t launch_batch_r(const ResBatch& b, int slots, int ctas, size_t smem, cudaStream_t s) {
+  switch (slots) {
+    case 1: return launch_batch_s<R, 1>(b, ctas, smem, s);
+    case 2: return launch_batch_s<R, 2>(b, ctas, smem, s);
+    case 4: return launch_batch_s<R, 4>(b, ctas, smem, s);
+    case 8: return launch_batch_s<R, 8>(b, ctas, smem, s);
+  }
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_resident_batch(int prec, const ResBatch& b, int slots, int ctas, size_t smem, cudaStream_t s) {
+  return prec == 0 ? launch_batch_r<double>(b, slots, ctas, smem, s) : launch_batch_r<float>(b, slots, ctas, smem, s);
 }
 
 cudaError_t launch_resident(int prec, const ResParams& p, int slots, int nth, int max_grid, int n_z, cudaStream_t s) {

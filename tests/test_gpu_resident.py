@@ -124,3 +124,55 @@ def test_options_on_resident_launches(n):
         assert not np.any(psi[ones != k])
     assert abs(ctx.norm2() - 1.0) < 1e-5
     ctx.close()
+
+
+@pytest.mark.parametrize("prec", [C64, C128])
+def test_batch_of_resident_and_other_members(prec):
+    """Members of every size class beside members on layout passes (too large, own tile bits), an odd
+    number of steps per round, members that end inside a round; removed before the end, they go on
+    alone."""
+    from paper_1311_3938_gb300 import hamiltonians as HB
+    from paper_1311_3938_gb300.engine import Batch, Context
+
+    def make(n, tile_bits, driver, total):
+        inst = generate_ec3(n, n)
+        ctx = Context(n, prec)
+        if tile_bits:
+            ctx.set_tile_bits(tile_bits)
+        if driver == "xy":
+            sched, k = HB.load_xy(ctx, inst, driver="xy", catalyst_alpha=8.0)
+            start = ("dicke", k)
+        else:
+            HB.load_ec3(ctx, inst, pairs=xx_pairs(n, n))
+            sched, start = HB.nonlinear_schedule(), "uniform"
+        ctx.set_schedule(0.02 * total / n, sched, 1)
+        ctx.set_integrator(total, 0.0)
+        ctx.set_initial_state(start)
+        return ctx
+
+    big = 21 if prec == C64 else 19
+    specs = [(6, 0, "x", 40), (9, 0, "xy", 20), (10, 0, "x", 80), (12, 0, "xy", 80), (13, 9, "x", 60), (14, 0, "x", 31),
+             (17, 0, "x", 40), (18, 0, "xy", 40), (big, 0, "x", 30)]
+    alone = []
+    for s in specs:
+        c = make(*s)
+        st = c.propagate(-1)
+        alone.append((c.state(), st["steps_done"]))
+        c.close()
+    tol = 2e-6 if prec == C64 else 1e-13
+    b = Batch(prec, max_members=16, max_items=4096, steps_per_round=7)
+    ctxs = [make(*s) for s in specs]
+    slots = [b.add(c) for c in ctxs[:5]]
+    b.run(2)
+    slots += [b.add(c) for c in ctxs[5:]]  # join while others are under way
+    b.run(3)
+    steps, active, launches = b.poll()
+    assert launches > 0 and active > 0
+    assert [steps[k] for k in slots] == [min(t, 3 + 7 * (5 if i < 5 else 3)) for i, (_, _, _, t) in enumerate(specs)]
+    for k, c, (want, total) in zip(slots, ctxs, alone):
+        b.remove(k)
+        st = c.propagate(-1)
+        assert st["steps_done"] == total and abs(st["norm2"] - 1.0) < 1e-4
+        assert rel_err(c.state(), want) < tol
+        c.close()
+    b.close()
