@@ -173,6 +173,7 @@ struct aqc_ctx {
   int relabel = 1;    // choose the qubit -> index-bit order that keeps flips inside layouts
   std::vector<int> perm;  // perm[q] = index bit of qubit q in the library's vectors
   bool permuted = false;  // perm is not the identity
+  bool res_declined = false;  // the products leave no room beside a resident tile: layout passes
   ResPlan res;        // resident launches (res.on: the state's size and products allow them)
   int sms = 0;        // multiprocessors of the device
   SlabParams slab;    // slab-ordered last passes of a PEC step (slab.n_slabs == 0: off)
@@ -350,7 +351,7 @@ bool resident_size(const aqc_ctx* c) { return c->tile_bits == 0 && c->n <= kResM
 std::vector<int> choose_order(const aqc_ctx* c) {
   std::vector<int> id(c->n);
   for (int q = 0; q < c->n; q++) id[q] = q;
-  if (!c->relabel || c->layouts.size() < 2 || resident_size(c)) return id;
+  if (!c->relabel || c->layouts.size() < 2 || (resident_size(c) && !c->res_declined)) return id;
   std::vector<std::pair<uint32_t, int>> masks;  // distinct multi-bit flip masks with counts
   for (const TermH& th : c->terms) {
     if (__builtin_popcount(th.x) < 2) continue;
@@ -770,6 +771,10 @@ int build_tables(aqc_ctx* c) {
     }
   }
   plan_resident(c);
+  if (resident_size(c) && !c->res.on && !c->res_declined) {
+    c->res_declined = true;  // the layout passes have an index order of their own
+    return build_tables(c);
+  }
   c->step_m = c->step_class >= 0 ? classes[c->step_class].end - classes[c->step_class].begin : 0;
   c->table_class = t->table_class;
   CUDA_TRY(c, cudaMemcpyAsync(c->d_tab, t, sizeof(DevTables), cudaMemcpyHostToDevice, c->stream));
@@ -1869,6 +1874,7 @@ int aqc_load_terms(aqc_ctx* ctx, int group, size_t n_terms, const uint64_t* xmas
     if (!isfinite(coef[k])) FAIL(ctx, AQC_E_INVAL, "term %zu: non-finite coefficient", k);
   }
   for (size_t k = 0; k < n_terms; k++) ctx->terms.push_back(TermH{(uint32_t)xmask[k], (uint32_t)zmask[k], coef[k], group});
+  ctx->res_declined = false;
   ctx->dirty = true;
   return AQC_OK;
 }
@@ -1901,6 +1907,7 @@ int aqc_load_clauses(aqc_ctx* ctx, int group, size_t m, const int32_t* bits, int
 
 int aqc_clear_hamiltonian(aqc_ctx* ctx) {
   if (!ctx) return AQC_E_INVAL;
+  ctx->res_declined = false;
   ctx->terms.clear();
   ctx->clauses.clear();
   ctx->dirty = true;

@@ -95,7 +95,7 @@ struct ResSmem {
     z = up16(gen + 2 * (size_t)ng * sizeof(RGen<R>));
     scal = up16(z + 2 * (size_t)nz * sizeof(R));
     red = up16(scal + 2 * sizeof(RScal<R>));
-    lane = up16(red + 3 * (size_t)nth * (dred ? sizeof(double) : sizeof(R)));
+    lane = up16(red + 2 * (size_t)nth * (dred ? sizeof(double) : sizeof(R)));
     bar = lane + 8 * (kResMaxEvals + 1) * sizeof(double);
     total = bar + 2 * (size_t)(nbuf > 0 ? nbuf : 1) * sizeof(uint64_t);
   }
@@ -320,7 +320,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
   RGen<R>* const s_gen = reinterpret_cast<RGen<R>*>(smem + M.gen);
   R* const s_z = reinterpret_cast<R*>(smem + M.z);
   RScal<R>* const s_sc = reinterpret_cast<RScal<R>*>(smem + M.scal);
-  RED* const s_red = reinterpret_cast<RED*>(smem + M.red);           // [parity][nth], then [nth] of the last
+  RED* const s_red = reinterpret_cast<RED*>(smem + M.red);           // [parity][nth]
   double* const s_lane = reinterpret_cast<double*>(smem + M.lane);  // [E + 1][8]
   const uint32_t full0 = saddr(smem + M.bar), empty0 = full0 + 8u * (uint32_t)nbuf;
 
@@ -408,6 +408,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
     }
     __syncwarp();
   };
+  auto all_sync = [&]() { asm volatile("bar.sync 2, %0;\n" ::"r"((int)blockDim.x) : "memory"); };
   const C2* const src0 = reinterpret_cast<const C2*>(P.src);
   C2* const XA = reinterpret_cast<C2*>(P.xout[0]);
   C2* const XO = reinterpret_cast<C2*>(P.xout[1]);
@@ -437,6 +438,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
     const int j0 = tid * H, js = nth * H;  // tile position of the first slot, slot stride
     const bool act = j0 < (int)tsize;      // tiles below one slot per thread: some idle
     const uint32_t jb = (uint32_t)j0 * sizeof(C2), jsb = (uint32_t)js * sizeof(C2);
+    const int jsl = 31 - __clz(js);
     Owned o[REG ? S : 1];
     if (REG && act && !P.single) {
 #pragma unroll
@@ -451,6 +453,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
     }
     const C2* xin = src0;
     C2* xout = XA;
+    RED final0 = (RED)0;  // the last evaluation's first reduction (||y||^2, Re <src|H|src>)
     for (int e = 0; e < E; e++) {
       const int kind = PEC ? 0 : kind_of(P, e), par = e & 1;
       const bool last = e == E - 1;
@@ -537,31 +540,65 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
               }
             }
         };
-        // hops or other products [k, end)
-        auto general = [&](const unsigned char* t, int k, bool hop, int end) {
+        // one slot's partner amplitudes at place `off`
+        auto partner = [&](const unsigned char* t, uint32_t off, int s, bool sw, C2 (&u)[H]) {
+          if constexpr (S >= 4) {
+            const uint32_t at = (jb ^ (off & ~15u)) ^ ((uint32_t)s * jsb);
+            C2 v[H];
+            unpack<C2, H>(*reinterpret_cast<const float4*>(t + at), v);
+#pragma unroll
+            for (int q = 0; q < H; q++) u[q] = sw ? v[H - 1 - q] : v[q];
+          } else {
+            const uint32_t at = (jb ^ off) ^ ((uint32_t)s * jsb);
+#pragma unroll
+            for (int q = 0; q < H; q++) u[q] = *reinterpret_cast<const C2*>(t + (at ^ (uint32_t)(q * sizeof(C2))));
+          }
+        };
+        // hops [k, end): 2c (= cr - cr2) where the two bits of z differ, else 0.  The thread's
+        // amplitudes differ in bit 0 and in the slot bits only, so one parity per hop is computed
+        // and the slots' come from the flip's slot bits (the same for all threads)
+        auto hops = [&](const unsigned char* t, int k, int end) {
+          const uint32_t zt = zb + (uint32_t)j0;
+#pragma unroll(S >= 4 ? 1 : 2)
+          for (; k < end; k++) {
+            const uint32_t x = gen[k].x, off = gen[k].off;
+            const R c2 = gen[k].cr - gen[k].cr2;
+            const bool odd = __popc(x & zt) & 1, sw = H == 2 && (x & 1u);
+            const R cA = odd ? c2 : (R)0, cB = odd ? (R)0 : c2;
+            const uint32_t xs_ = (x & tmask) >> jsl;
+#pragma unroll
+            for (int s = 0; s < S; s++) {
+              C2 u[H];
+              partner(t, off, s, sw, u);
+              const bool ps = __popc(xs_ & (uint32_t)s) & 1;
+#pragma unroll
+              for (int q = 0; q < H; q++) {
+                const R cf = (ps != (sw && q)) ? cB : cA;
+                ar[s * H + q] = fma_(cf, u[q].x, ar[s * H + q]);
+                ai[s * H + q] = fma_(cf, u[q].y, ai[s * H + q]);
+              }
+            }
+          }
+        };
+        // other products [k, end)
+        auto general = [&](const unsigned char* t, int k, int end) {
 #pragma unroll 1
           for (; k < end; k++) {
             const RGen<R> f = gen[k];
+            const bool sw = H == 2 && (f.x & 1u);
 #pragma unroll
             for (int s = 0; s < S; s++) {
-              const uint32_t at = (jb ^ f.off) ^ ((uint32_t)s * jsb);
+              C2 u[H];
+              partner(t, f.off, s, sw, u);
 #pragma unroll
               for (int q = 0; q < H; q++) {
-                const C2 w = *reinterpret_cast<const C2*>(t + (at ^ (uint32_t)(q * sizeof(C2))));
                 const int g = s * H + q;
-                const uint32_t z = zb + (uint32_t)(j0 + s * js + q);
-                if (hop) {  // 2c where the two bits of z differ (cr - cr2 = 2c)
-                  const R cf = (__popc(f.x & z) & 1) ? f.cr - f.cr2 : (R)0;
-                  ar[g] = fma_(cf, w.x, ar[g]);
-                  ai[g] = fma_(cf, w.y, ai[g]);
-                } else {
-                  const uint32_t zsrc = z ^ f.x;
-                  const bool n1 = __popc(f.zm & zsrc) & 1, n2 = __popc(f.zm2 & zsrc) & 1;
-                  const R cr = (n1 ? -f.cr : f.cr) + (n2 ? -f.cr2 : f.cr2);
-                  const R ci = (n1 ? -f.ci : f.ci) + (n2 ? -f.ci2 : f.ci2);
-                  ar[g] = fma_(cr, w.x, fma_(-ci, w.y, ar[g]));
-                  ai[g] = fma_(cr, w.y, fma_(ci, w.x, ai[g]));
-                }
+                const uint32_t zsrc = (zb + (uint32_t)(j0 + s * js + q)) ^ f.x;
+                const bool n1 = __popc(f.zm & zsrc) & 1, n2 = __popc(f.zm2 & zsrc) & 1;
+                const R cr = (n1 ? -f.cr : f.cr) + (n2 ? -f.cr2 : f.cr2);
+                const R ci = (n1 ? -f.ci : f.ci) + (n2 ? -f.ci2 : f.ci2);
+                ar[g] = fma_(cr, u[q].x, fma_(-ci, u[q].y, ar[g]));
+                ai[g] = fma_(cr, u[q].y, fma_(ci, u[q].x, ai[g]));
               }
             }
           }
@@ -580,7 +617,10 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
               plain(t, pk, r.end);
               pk = r.end;
             } else {
-              general(t, gk, r.kind == 1, r.end);
+              if (r.kind == 1)
+                hops(t, gk, r.end);
+              else
+                general(t, gk, r.end);
               gk = r.end;
             }
           }
@@ -730,7 +770,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
       }
       if (kind == 0 || kind == 7) {
         s_red[(size_t)par * nth + tid] = red1;
-        if (last) s_red[(size_t)2 * nth + tid] = red0;
+        if (last) final0 = red0;
       }
       if (kind == 0 || kind == 5 || kind == 1) latest++;
       if (last) break;
@@ -749,6 +789,11 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
         if (latest > first_latest + 2) store(F(latest - 2) + z, o[s].c);
         if (kComp && P.n_pec) store(YL + z, o[s].yl);
       }
+    }
+    if (PEC || P.single == 7) {
+      all_sync();  // the sums of the evaluation before the last are done: its place is free
+      s_red[(size_t)(E & 1) * nth + tid] = final0;
+      all_sync();
     }
   } else {
     // evaluation e's reductions over the CTA: FP64 sums in a fixed order, eight per evaluation
@@ -801,15 +846,15 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
         for (uint32_t par = 0; par < 2; par++) (void)bar_wait_short(full0 + 8u * b, par);
     }
     if (PEC || P.single == 7) {
-      asm volatile("bar.sync 2, %0;\n" ::"r"((int)blockDim.x) : "memory");  // the last reductions are there
+      all_sync();
+      all_sync();  // the last reductions are there
       if (svc == 2) {
         lane_sums(s_red + (size_t)((E - 1) & 1) * nth, s_lane + 8 * (E - 1));
-        lane_sums(s_red + (size_t)2 * nth, s_lane + 8 * E);
+        lane_sums(s_red + (size_t)(E & 1) * nth, s_lane + 8 * E);
       }
     }
   }
   const bool reduced = P.n_pec > 0 || P.single == 7;
-  if (owner && (PEC || P.single == 7)) asm volatile("bar.sync 2, %0;\n" ::"r"((int)blockDim.x) : "memory");
   if (P.single == 6) return;
   __syncthreads();
   if (reduced) {
