@@ -156,8 +156,11 @@ struct aqc_ctx {
   std::vector<Layout> layouts;
   std::vector<int> nplain, ngeneral;  // local X-string / general products per layout
   std::vector<int> nhop;              // of the general ones, the hops (leading)
-  std::vector<char> xpartial;        // layout l's partial pass can run as k_partial_x
+  std::vector<char> tile_x;          // layout l's passes can run as k_tile_x
   int n_remote = 0, n_z = 0;
+  bool remote_x = false;             // the products no layout holds are X strings and hops
+  bool store_y = true;               // this step's y_{n+1} is read after it: the last of a call
+  bool short_ring = false;           // f_{n-3} is not in its ring slot (resident launches keep three)
   int table_class = -1;
   int step_class = -1, step_m = 0;  // clause-by-clause sequence (class index, length)
   double eval_s = 0.0;              // path parameter s of the evaluation being issued
@@ -173,6 +176,8 @@ struct aqc_ctx {
   int relabel = 1;    // choose the qubit -> index-bit order that keeps flips inside layouts
   std::vector<int> perm;  // perm[q] = index bit of qubit q in the library's vectors
   bool permuted = false;  // perm is not the identity
+  bool far = false;           // the top bits lie in no layout (plan_layouts)
+  bool far_declined = false;  // some products need the layout passes of k_apply: a layout for every bit
   bool res_declined = false;  // the products leave no room beside a resident tile: layout passes
   ResPlan res;        // resident launches (res.on: the state's size and products allow them)
   int sms = 0;        // multiprocessors of the device
@@ -296,7 +301,29 @@ uint32_t compress_mask(const Layout& L, uint32_t x) {
   return r;
 }
 
-void plan_layouts(aqc_ctx* c) { c->layouts = layouts_for(c->n, c->prec, c->tile_bits, !c->in_batch); }
+// Tile layouts of a context.  complex64 states beyond two layouts whose products are X strings and hops
+// leave their top bits to no layout: the strided layout's pass reads those partners from memory (L2),
+// which costs less than a third pass over the state (read it, read and write the partial sum) while
+// the bits are few.  Microseconds per step with three layouts / with two: linear path n = 22 94 / 83,
+// n = 24 288 / 264, n = 26 1057 / 1005, n = 27 2076 / 2039, n = 28 4135 / 4198; nonlinear n = 24 475 / 443,
+// n = 25 884 / 847; XY n = 22 166 / 157, n = 24 632 / 615, n = 25 1117 / 1145.
+void plan_layouts(aqc_ctx* c) {
+  c->layouts = layouts_for(c->n, c->prec, c->tile_bits, !c->in_batch);
+  c->far = false;
+  if (c->prec != AQC_C64 || c->tile_bits != 0 || c->in_batch || c->slab_req || c->turn_req || c->far_declined ||
+      c->layouts.size() != 3)
+    return;
+  int most = 6;
+  for (const TermH& t : c->terms) {
+    if (t.x == 0) continue;
+    if (__builtin_popcount(t.x) > 1) most = std::min(most, t.zm ? 3 : 4);
+    if (t.zm != 0 && t.zm != t.x) most = 0;
+  }
+  const Layout& top = c->layouts[1];
+  if (c->n - (top.h + top.w) > most) return;
+  c->layouts.pop_back();
+  c->far = true;
+}
 
 // ---- qubit relabelling ----------------------------------------------------------------------
 // The library may store qubit q at index bit perm[q] (a relabelling of the tensor factors of
@@ -632,7 +659,7 @@ int build_tables(aqc_ctx* c) {
   c->nplain.assign(nl, 0);
   c->ngeneral.assign(nl, 0);
   c->nhop.assign(nl, 0);
-  c->xpartial.assign(nl, 0);
+  c->tile_x.assign(nl, 0);
   for (int l = 0; l <= nl; l++) {
     t->flip_begin[l] = pos;
     if (pos + (int)per[l].size() > kMaxFlips) FAIL(c, AQC_E_UNSUPPORTED, "more than %d off-diagonal products", kMaxFlips);
@@ -686,10 +713,11 @@ int build_tables(aqc_ctx* c) {
       c->ngeneral[l] = (int)per[l].size() - np;
       c->nhop[l] = nh;
     }
-    if (l > 0 && l < nl) {  // X strings and hops only: the TMA-fed partial kernel
-      const bool ok = c->prec == AQC_C64 && xpartial_layout_ok(c->layouts[l]) && c->ngeneral[l] == nh &&
-                      xpartial_smem_bytes(np + nh) <= 227 * 1024;
-      c->xpartial[l] = ok ? 1 : 0;
+    if (l < nl)  // X strings and hops only: the TMA-fed kernel
+      c->tile_x[l] = c->prec == AQC_C64 && tile_x_layout_ok(c->layouts[l]) && c->ngeneral[l] == nh;
+    if (l == nl) {
+      c->remote_x = true;
+      for (const DevFlip& f : per[l]) c->remote_x = c->remote_x && ((f.zm == 0 && !f.has2) || is_hop(f));
     }
     pos += (int)per[l].size();
   }
@@ -773,6 +801,10 @@ int build_tables(aqc_ctx* c) {
   plan_resident(c);
   if (resident_size(c) && !c->res.on && !c->res_declined) {
     c->res_declined = true;  // the layout passes have an index order of their own
+    return build_tables(c);
+  }
+  if (c->far && !(c->remote_x && c->tile_x[1])) {
+    c->far_declined = true;
     return build_tables(c);
   }
   c->step_m = c->step_class >= 0 ? classes[c->step_class].end - classes[c->step_class].begin : 0;
@@ -900,6 +932,59 @@ ApplyParams base_params(aqc_ctx* c) {
   return p;
 }
 
+// Whether a layout pass runs as k_tile_x, and its parameters: complex64, nothing but X strings and hops
+// in the layout (and, in the first pass, among the products no layout holds), 16-byte-aligned
+// vectors.  Its step forms p_{n+2} from p_{n+1} and four derivatives, so it serves the plain
+// corrector on the fixed grid; the compensated one, step-size control (a rejected step keeps y_n) and
+// the turn of layouts run k_apply.
+bool tile_x_pass(const aqc_ctx* c, const ApplyParams& p, XParams* x) {
+  const int l = p.layout_index;
+  const bool remote = p.with_remote && c->n_remote > 0;
+  if (!c->tile_x[l] || (c->step_class >= 0 && p.with_diag)) return false;
+  if (remote && (!c->remote_x || p.mode != MODE_PARTIAL || p.with_diag)) return false;
+  if (p.mode == MODE_STEP && (p.yout || p.ylo || p.turn || c->short_ring)) return false;
+  if (p.L.w > 0 && (p.mode != MODE_PARTIAL || p.with_diag)) return false;
+  const uintptr_t all = (uintptr_t)p.src | (uintptr_t)p.qin | (uintptr_t)p.qout;
+  if (all & 15u) return false;
+  const int nf = c->nplain[l] + c->nhop[l] + (remote ? c->n_remote : 0);
+  if (tile_x_smem_bytes(nf, p.with_diag ? c->n_z : 0, p.with_diag && p.dcode) > 227 * 1024) return false;
+  memset(x, 0, sizeof(*x));
+  if (p.L.w > 0) {
+    x->tma_rank = encode_tile_map(&x->tmap, p.src, c->n, p.L);
+    if (!x->tma_rank) return false;
+  }
+  x->tab = c->d_tab;
+  x->L = p.L;
+  x->layout_index = l;
+  x->mode = p.mode;
+  x->stage = p.stage;
+  x->with_diag = p.with_diag;
+  x->with_remote = remote;
+  x->top_bits = remote ? c->n - p.L.h - p.L.w : 0;
+  for (int g = 0; g < 3; g++) x->w[g] = p.w[g];
+  x->wdev = p.wdev;
+  x->max_grid = c->grid_limit;
+  x->h = p.h;
+  x->dcode = p.with_diag ? p.dcode : nullptr;
+  x->src = p.src;
+  x->qin = p.qin;
+  x->qout = p.qout;
+  x->f[0] = p.f0;
+  x->f[1] = p.f1;
+  x->f[2] = p.f2;
+  x->f[3] = p.fout;  // f_{n-3}, in the ring slot that f_{n+1} takes
+  x->fout = p.fout;
+  x->pout = p.pout;
+  x->y = p.y;
+  x->yout = p.mode == MODE_STEP && c->store_y ? p.y : nullptr;
+  x->acc = p.acc;
+  x->ntiles = p.ntiles;
+  x->partials = c->d_partials;
+  x->counter = c->d_counter;
+  x->slots = c->d_slots;
+  return true;
+}
+
 // Fields of a resident launch that do not depend on what it runs.
 ResParams resident_params(aqc_ctx* c) {
   ResParams p;
@@ -978,6 +1063,7 @@ int resident_steps(aqc_ctx* c, int n_rk, bool hist, int n_pec) {
   p.acc = c->vec[V_ACC];
   p.ylo = c->ycomp && n_pec ? c->vec_save : nullptr;
   c->q_ready = -1;
+  c->short_ring = true;
   int rc = launch_resident_on(c, p);
   if (rc) return rc;
   if (p.evals & 1) std::swap(c->vec[V_P], c->vec[V_Q]);
@@ -1016,26 +1102,11 @@ int evaluate(aqc_ctx* c, const double w[3], const void* src, ApplyParams fin, vo
     }
     p.dcode = (diag && c->table_class >= 0) ? c->d_dcode : nullptr;
     p.ntiles = 1u << (c->n - p.L.t);
-    // X-string-only strided layouts: TMA-fed partial kernel
-    if (!last && !diag && c->xpartial[l] && !(first && c->n_remote > 0)) {
-      XPartialParams x;
-      memset(&x, 0, sizeof(x));
-      x.tma_rank = encode_tile_map(&x.tmap, src, c->n, p.L);
-      if (x.tma_rank) {
-        x.tab = c->d_tab;
-        x.L = p.L;
-        x.layout_index = l;
-        for (int g = 0; g < 3; g++) x.w[g] = w[g];
-        x.wdev = c->cur_wdev;
-        x.max_grid = c->grid_limit;
-        x.qin = p.qin;
-        x.qout = p.qout;
-        x.ntiles = p.ntiles;
-        x.slots = c->d_slots;
-        CUDA_TRY(c, launch_partial_x(x, (int)xpartial_smem_bytes(c->nplain[l] + c->nhop[l]), c->stream));
-        c->launches++;
-        continue;
-      }
+    XParams x;
+    if (tile_x_pass(c, p, &x)) {
+      CUDA_TRY(c, launch_tile_x(x, c->nplain[l] + c->nhop[l] + (first ? c->n_remote : 0), diag ? c->n_z : 0, c->stream));
+      c->launches++;
+      continue;
     }
     const size_t smem = apply_smem_bytes(c->prec, p.L.t - p.L.cb, c->nplain[l],
                                          c->ngeneral[l] + (first ? c->n_remote : 0), diag ? c->n_z : 0);
@@ -1178,25 +1249,11 @@ int pec_step_turn(aqc_ctx* c, const ApplyParams& fin0, const double w[3]) {
     p.qout = c->vec[V_Q];
     p.ntiles = 1u << (c->n - p.L.t);
     any = true;
-    if (c->xpartial[l] && !(first && c->n_remote > 0)) {
-      XPartialParams x;
-      memset(&x, 0, sizeof(x));
-      x.tma_rank = encode_tile_map(&x.tmap, p.src, c->n, p.L);
-      if (x.tma_rank) {
-        x.tab = c->d_tab;
-        x.L = p.L;
-        x.layout_index = l;
-        for (int g = 0; g < 3; g++) x.w[g] = w[g];
-        x.wdev = c->cur_wdev;
-        x.max_grid = c->grid_limit;
-        x.qin = p.qin;
-        x.qout = p.qout;
-        x.ntiles = p.ntiles;
-        x.slots = c->d_slots;
-        CUDA_TRY(c, launch_partial_x(x, (int)xpartial_smem_bytes(c->nplain[l] + c->nhop[l]), c->stream));
-        c->launches++;
-        continue;
-      }
+    XParams x;
+    if (tile_x_pass(c, p, &x)) {
+      CUDA_TRY(c, launch_tile_x(x, c->nplain[l] + c->nhop[l] + (first ? c->n_remote : 0), 0, c->stream));
+      c->launches++;
+      continue;
     }
     const size_t smem = apply_smem_bytes(c->prec, p.L.t, c->nplain[l], c->ngeneral[l] + (first ? c->n_remote : 0), 0);
     if (smem > 227 * 1024) FAIL(c, AQC_E_UNSUPPORTED, "shared memory %zu bytes too large", smem);
@@ -1273,6 +1330,7 @@ int begin_segment(aqc_ctx* c, double t0, double hp, int64_t m_given = 0) {
   c->hist_ready = false;
   c->q_ready = -1;
   c->small_run = 0;
+  c->short_ring = false;
   c->seg_done0 = c->steps_done;
   if (c->adaptive)  // kept until the segment's first PEC step is accepted
     CUDA_TRY(c, cudaMemcpyAsync(c->vec_save, c->vec[V_Y], (size_t)c->N * c->amp, cudaMemcpyDeviceToDevice,
@@ -1400,6 +1458,7 @@ int capture_steps(aqc_ctx* c, int K) {
     }
     for (int j = 0; j < K && rc == AQC_OK && !resident_on(c); j++) {
       c->cur_wdev = c->d_wdev + kGraphStepWeights * j;
+      c->store_y = j == K - 1;
       rc = pec_step(c);
       c->step++;
     }
@@ -1874,7 +1933,7 @@ int aqc_load_terms(aqc_ctx* ctx, int group, size_t n_terms, const uint64_t* xmas
     if (!isfinite(coef[k])) FAIL(ctx, AQC_E_INVAL, "term %zu: non-finite coefficient", k);
   }
   for (size_t k = 0; k < n_terms; k++) ctx->terms.push_back(TermH{(uint32_t)xmask[k], (uint32_t)zmask[k], coef[k], group});
-  ctx->res_declined = false;
+  ctx->res_declined = ctx->far_declined = false;
   ctx->dirty = true;
   return AQC_OK;
 }
@@ -1907,7 +1966,7 @@ int aqc_load_clauses(aqc_ctx* ctx, int group, size_t m, const int32_t* bits, int
 
 int aqc_clear_hamiltonian(aqc_ctx* ctx) {
   if (!ctx) return AQC_E_INVAL;
-  ctx->res_declined = false;
+  ctx->res_declined = ctx->far_declined = false;
   ctx->terms.clear();
   ctx->clauses.clear();
   ctx->dirty = true;
@@ -2042,6 +2101,7 @@ int aqc_wait_selftest(aqc_ctx* ctx, int64_t polls) {
 int aqc_set_layout_turns(aqc_ctx* ctx, int mode) {
   if (!ctx) return AQC_E_INVAL;
   if (mode < -1 || mode > 1) FAIL(ctx, AQC_E_INVAL, "mode must be -1, 0 or 1");
+  if ((mode != 0) != (ctx->turn_req != 0)) ctx->dirty = true;  // the layouts may differ
   ctx->turn_req = mode;
   ctx->q_ready = -1;
   DeviceGuard dg(ctx->device);
@@ -2067,6 +2127,7 @@ int aqc_get_graph_replays(const aqc_ctx* ctx, int64_t* out) {
 int aqc_set_slab_bits(aqc_ctx* ctx, int slab_bits) {
   if (!ctx) return AQC_E_INVAL;
   if (slab_bits < -1 || slab_bits > 11) FAIL(ctx, AQC_E_INVAL, "slab_bits must be -1, 0 or 1..11");
+  if ((slab_bits != 0) != (ctx->slab_req != 0)) ctx->dirty = true;  // the layouts may differ
   ctx->slab_req = slab_bits;
   if (!ctx->dirty) plan_slabs(ctx);
   return AQC_OK;
@@ -2234,6 +2295,7 @@ int aqc_propagate(aqc_ctx* ctx, int64_t max_steps, aqc_stats* stats) {
         for (int i = 0; i < m; i++) count_step(ctx);
         continue;
       }
+      ctx->store_y = left == 1;
       rc = pec_step(ctx);
       if (!rc) {
         if (ctx->adaptive)

@@ -189,22 +189,35 @@ struct SlabParams {
 };
 constexpr int kMaxSlabs = 2048;  // also the room of the resident launches' flags (kResMaxTiles x kResFlagStride)
 
-// Partial-sum pass of a strided layout holding only X strings with real coefficients
-// (complex64, kernel k_partial_x): the source tile arrives by TMA through `tmap`.
+// Layout pass holding only X strings with real coefficients and hops (complex64, kernel k_tile_x).
 constexpr int kXTileBits = 13;
-struct XPartialParams {
-  CUtensorMap tmap;      // source as a 4-D float tensor (chunk, gap bits, tile rows, top bits),
-                         // 5-D when the chunk exceeds one box row (chunk split in two dims)
+struct XParams {
+  CUtensorMap tmap;      // strided layouts: the source as a 4-D float tensor (chunk, gap bits, tile rows,
+                         // top bits), 5-D when the chunk exceeds one box row (chunk split in two dims)
   int tma_rank;          // 4 or 5
   const DevTables* tab;
   Layout L;
   int layout_index;
+  int mode, stage;       // as in ApplyParams
+  int with_diag, with_remote;
+  int top_bits;          // > 0: visit tiles that differ in this many top index bits side by side
   double w[3];
   const double* wdev;    // nullable: weights from device memory (as ApplyParams::wdev)
   int max_grid;          // > 0: at most this many CTAs
+  double h;
+  const uint8_t* dcode;  // nullable
+  const void* src;
   const void* qin;       // nullable
-  void* qout;
+  void* qout;            // PARTIAL
+  const void* f[4];      // STEP: f_n, f_{n-1}, f_{n-2}, f_{n-3}
+  void* fout;            // STEP: f_{n+1} (may be f[3]); DERIV: f; RK4 stage 1: history f_n
+  void* pout;            // STEP: p_{n+2}; RK4: next stage input
+  void* y;               // RK4
+  void* yout;            // STEP: nullable, y_{n+1}
+  void* acc;             // RK4 accumulator
   uint32_t ntiles;
+  double* partials;      // two per CTA
+  unsigned* counter;
   double* slots;         // kSlotFault is set if a tile copy never completes
 };
 
@@ -333,9 +346,9 @@ int apply_grid(int prec, int mode, uint32_t ntiles, int smem_bytes);
 size_t apply_smem_bytes(int prec, int t, int n_plain, int n_general, int n_z);
 size_t table_smem_bytes(int prec, int t, int n_plain, int n_general, int n_z);
 cudaError_t launch_slab(int prec, const SlabParams& p, int smem_bytes, cudaStream_t s);
-bool xpartial_layout_ok(const Layout& L);
-size_t xpartial_smem_bytes(int n_flips);
-cudaError_t launch_partial_x(const XPartialParams& p, int smem_bytes, cudaStream_t s);
+bool tile_x_layout_ok(const Layout& L);
+size_t tile_x_smem_bytes(int n_flips, int n_z, bool codes);
+cudaError_t launch_tile_x(const XParams& p, int n_flips, int n_z, cudaStream_t s);
 uint32_t lanczos_dot_blocks(uint64_t N);
 cudaError_t launch_dotc_multi(int prec, const void* V, uint64_t ld, uint32_t m, const void* w, uint64_t N,
                               double* partials, double* out, double* acc, cudaStream_t s);

@@ -1,19 +1,35 @@
-// Partial-sum pass over a strided tile layout whose products are all X strings with real
-// coefficients (the driver term of Eq. Hix and the XX couplings of the nonlinear path) or hops
-// X_iX_j + Y_iY_j (Eq. Hixy), complex64 only:
-//   q_out(z) = q_in(z) + sum_k c_k [hop_k: bits i_k, j_k of z differ] psi(z ^ x_k)
-// for every z of the tile (gather form of the per-qubit action, Sec. I.A).
+// Layout passes whose products are all X strings with real coefficients (the driver term of Eq. Hix
+// and the XX couplings of the nonlinear path) or hops X_iX_j + Y_iY_j (Eq. Hixy), complex64 only:
+//   r(z) = q(z) + [d(z) psi(z)] + sum_k c_k [hop_k: bits i_k, j_k of z differ] psi(z ^ x_k)
+// for every z of the tile (gather form of the per-qubit action, Sec. I.A), then r is stored as a
+// partial sum, or the contiguous layout's pass finishes the evaluation: the fused
+// predictor-corrector step, a Runge-Kutta stage, the derivative or the energy.
 //
 // GB300 structure: one CTA of 512 threads per SM, persistent over tiles.  The 64 KiB source
 // tile (2^13 amplitudes) is brought into shared memory by one TMA tensor copy
-// (cp.async.bulk.tensor, 4-D map: chunk, gap bits, tile rows, top bits) into one of two buffers,
-// completion tracked by an mbarrier, so the next tile streams in while this one is computed.
-// Each thread holds 16 amplitudes in registers: pairs (tile bit 0) at 8 positions spanning tile
-// bits 6..8.  Products flipping only bits 6..8 are register permutations; all others read one
-// 16-byte shared-memory vector per pair, at one base address plus immediate offsets.  The
-// partial sum streams through registers: loaded before the tile wait, stored after the flips.
+// (cp.async.bulk.tensor, 4-D map: chunk, gap bits, tile rows, top bits; the contiguous layout's by one
+// plain bulk copy, with its 8 KiB of clause bytes) into one of two buffers, completion tracked by an
+// mbarrier, so the next tile streams in while this one is computed.  Each thread holds 16 amplitudes
+// in registers: pairs (tile bit 0) at 8 positions spanning tile bits 6..8.  Products flipping only
+// bits 6..8 are register permutations; all others inside the tile read one 16-byte shared-memory
+// vector per pair, at one base address plus immediate offsets.  Products that no layout holds
+// read their partner from memory, one 16-byte vector per pair, in the pass that runs first.  The
+// partial sum and the other vectors of a pass stream through registers, those of the epilogue one
+// pair ahead.
+//
+// The step keeps y out of memory: with D1 = f_{n+1} - f_n, D2 = f_n - f_{n-1}, ... it forms
+//   p_{n+2} = p_{n+1} + h/24 (24 f_{n+1} + 40 D1 - 55 D2 + 36 D3 - 9 D4)
+// (corrector and predictor in one), and y_{n+1} = p_{n+1} + h/24 9 (D1 - 3 D2 + 3 D3 - D4) for the
+// error estimate; y is stored by the last step of a call only.  Eight vectors move instead of nine,
+// and the state is rounded once per step, after a sum whose large terms cancelled in differences.
+//
+// Measured (GB300): every pass of 28 qubits runs at the copy rate of 6.7 TB/s: partial passes 0.65 and
+// 0.90 ms, the step 2.59 ms (17.4 GB; as k_apply with y in memory 2.83 ms); at 23 qubits the step
+// 112 -> 96 us, the XY step of 24 qubits (78 hops) 486 -> 389 us, the last pass of H psi at 26 qubits
+// 403 -> 289 us, the XY pass with products that no layout holds 178 -> 98 us.
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <type_traits>
@@ -82,6 +98,14 @@ __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map
       "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
       " [%0], [%1, {%2, %3, %4, %5, %6}], [%7];\n" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
+      : "memory");
+}
+
+// contiguous bytes (16-byte aligned on both sides)
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst), "l"(src),
+      "r"(bytes), "r"(bar)
       : "memory");
 }
 
@@ -162,29 +186,78 @@ __device__ __forceinline__ void reg_hop(float cA, float cB, const float4 (&own)[
   one(std::integral_constant<int, 7>{});
 }
 
-__device__ __forceinline__ double weight_of(const XPartialParams& P, int g) {
+__device__ __forceinline__ double weight_of(const XParams& P, int g) {
   if (P.wdev) return P.wdev[g];
   return g == 0 ? P.w[0] : (g == 1 ? P.w[1] : P.w[2]);
 }
 
-__global__ void __launch_bounds__(kXThreads, 1) k_partial_x(const __grid_constant__ XPartialParams P) {
+struct XSmem {  // [pad to 1 KiB][tile 0][tile 1][clause bytes 0, 1][flips][Z strings][reduction][2 mbarriers]
+  size_t code, flips, z, red, bar, total;
+  __host__ __device__ XSmem(int n_flips, int n_z, bool codes) {
+    code = 2 * (size_t)kXTileBytes;
+    flips = code + (codes ? 2u << kXTileBits : 0u);
+    z = (flips + (size_t)n_flips * sizeof(XFlip) + 15) & ~(size_t)15;
+    red = (z + (size_t)n_z * sizeof(float2) + 15) & ~(size_t)15;
+    bar = red + 2 * (kXThreads / 32) * sizeof(double);
+    total = bar + 16 + 1024;
+  }
+};
+
+// clause classes other than the byte table's and Z strings at index z (rare)
+__device__ __noinline__ float x_other_diagonal(const XParams& P, const float2* s_z, int code, uint32_t z) {
+  const DevTables* tab = P.tab;
+  const int tcls = P.dcode ? tab->table_class : -1;
+  float d = 0.f;
+  for (int cc = 0; cc < tab->n_classes; cc++) {
+    if (cc == tcls) continue;
+    const DevClass cl = tab->classes[cc];
+    const bool derived = cl.derived && tcls >= 0;
+    const int b = derived ? cl.dbegin : cl.begin, e = derived ? cl.dend : cl.end;
+    int cnt = 0;
+    for (int k = b; k < e; k++) {
+      const int o = 1 - __popc(tab->clause_mask[k] & z);
+      cnt += cl.pen == 0 ? (o != 0) : o * o;
+    }
+    d = fmaf((float)(cl.scale * weight_of(P, cl.group)), (float)(derived ? code - cnt : cnt), d);
+  }
+  for (int m = 0; m < tab->n_z; m++) d += (__popc(__float_as_uint(s_z[m].x) & z) & 1) ? -s_z[m].y : s_z[m].y;
+  return d;
+}
+
+// MODE as in ApplyParams.  DIAG: this pass adds the diagonal (the contiguous layout).  FAR: it reads
+// the partners of products that no layout holds.
+template <int MODE, bool DIAG, bool FAR>
+__global__ void __launch_bounds__(kXThreads, 1) k_tile_x(const __grid_constant__ XParams P) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  // [pad to 1 KiB][tile buffer 0][tile buffer 1][flips][2 mbarriers]
   unsigned char* base = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
   unsigned char* const buf0 = base;
   unsigned char* const buf1 = base + kXTileBytes;
   const DevTables* tab = P.tab;
-  const int fb = tab->flip_begin[P.layout_index];
-  const int np = tab->plain_count[P.layout_index] + tab->hop_count[P.layout_index];  // X strings, then hops
+  const int fb = tab->flip_begin[P.layout_index], rb = tab->flip_begin[tab->n_layouts];
   const int npl = tab->plain_count[P.layout_index];
-  XFlip* s_f = reinterpret_cast<XFlip*>(base + 2 * kXTileBytes);
-  uint64_t* s_bar = reinterpret_cast<uint64_t*>(base + 2 * kXTileBytes + ((np * sizeof(XFlip) + 15) & ~(size_t)15));
+  const int np = npl + tab->hop_count[P.layout_index];  // X strings, then hops
+  const int nf = np + (FAR ? tab->n_remote : 0);
+  const int nz = DIAG ? tab->n_z : 0, ncls = DIAG ? tab->n_classes : 0;
+  const XSmem M(nf, nz, DIAG && P.dcode);
+  XFlip* s_f = reinterpret_cast<XFlip*>(base + M.flips);
+  float2* s_z = reinterpret_cast<float2*>(base + M.z);
+  double* s_red = reinterpret_cast<double*>(base + M.red);
+  uint64_t* s_bar = reinterpret_cast<uint64_t*>(base + M.bar);
   const uint32_t bar0 = smem_addr(s_bar), bar1 = smem_addr(s_bar + 1);
   const uint32_t tid = threadIdx.x;
-  for (int k = tid; k < np; k += blockDim.x) {
-    const DevFlip d = tab->flips[fb + k];
-    const bool hop = k >= npl;  // X_iX_j + Y_iY_j: 2c where the bits differ
-    s_f[k] = XFlip{d.lx, (float)((hop ? 2.0 : 1.0) * d.coef * weight_of(P, d.group)), hop ? d.x : 0u, 0u};
+  for (int k = tid; k < nf; k += blockDim.x) {
+    const DevFlip d = tab->flips[k < np ? fb + k : rb + (k - np)];
+    const bool hop = k < np ? k >= npl : d.has2 != 0;  // X_iX_j + Y_iY_j: 2c where the bits differ
+    s_f[k] = XFlip{k < np ? d.lx : d.x, (float)((hop ? 2.0 : 1.0) * d.coef * weight_of(P, d.group)), hop ? d.x : 0u, 0u};
+  }
+  for (int k = tid; k < nz; k += blockDim.x)
+    s_z[k] = make_float2(__uint_as_float(tab->z[k].zm), (float)(tab->z[k].coef * weight_of(P, tab->z[k].group)));
+  float dconst = 0.f, wtab = 0.f;
+  bool others = false;
+  if (DIAG) {
+    dconst = (float)(tab->ident[0] * weight_of(P, 0) + tab->ident[1] * weight_of(P, 1) + tab->ident[2] * weight_of(P, 2));
+    if (P.dcode) wtab = (float)(tab->classes[tab->table_class].scale * weight_of(P, tab->classes[tab->table_class].group));
+    others = nz > 0 || ncls > (P.dcode ? 1 : 0);
   }
   if (tid == 0) {
     mbar_init(bar0, 1);
@@ -202,26 +275,43 @@ __global__ void __launch_bounds__(kXThreads, 1) k_partial_x(const __grid_constan
   for (int r = 0; r < 8; r++) zoff[r] = tile_z(L, jw | ((uint32_t)r << 6), 0u);
 
   const uint32_t first = blockIdx.x, stride = gridDim.x, ntiles = P.ntiles;
-  auto issue = [&](uint32_t tile, int b) {  // thread 0: TMA copy of a tile into buffer b
+  // number of the tile visited t-th: with products read from memory, tiles that differ in their top
+  // bits run side by side, so that a partner's lines are in L2 when they are read
+  auto number = [&](uint32_t t) {
+    return FAR ? ((t & ((1u << P.top_bits) - 1u)) << gap) | (t >> P.top_bits) : t;
+  };
+  const float2* const src = reinterpret_cast<const float2*>(P.src);
+  auto issue = [&](uint32_t t, int b) {  // thread 0: copy of the t-th tile into buffer b
+    const uint32_t tile = number(t);
     const int x1 = (int)(tile & ((1u << gap) - 1u)), x3 = (int)(tile >> gap);
     asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    const uint32_t bb = b ? bar1 : bar0;
-    mbar_expect_tx(bb, kXTileBytes);
-    if (P.tma_rank == 5)
-      tma_load_5d(smem_addr(b ? buf1 : buf0), &P.tmap, bb, 0, 0, x1, 0, x3);
-    else
-      tma_load_4d(smem_addr(b ? buf1 : buf0), &P.tmap, bb, 0, x1, 0, x3);
+    const uint32_t bb = b ? bar1 : bar0, dst = smem_addr(b ? buf1 : buf0);
+    if (L.w == 0) {  // contiguous
+      const size_t z = (size_t)tile << kXTileBits;
+      mbar_expect_tx(bb, kXTileBytes + (DIAG && P.dcode ? 1u << kXTileBits : 0u));
+      bulk_load(dst, src + z, kXTileBytes, bb);
+      if (DIAG && P.dcode) bulk_load(smem_addr(base + M.code + ((size_t)b << kXTileBits)), P.dcode + z, 1u << kXTileBits, bb);
+    } else {
+      mbar_expect_tx(bb, kXTileBytes);
+      if (P.tma_rank == 5)
+        tma_load_5d(dst, &P.tmap, bb, 0, 0, x1, 0, x3);
+      else
+        tma_load_4d(dst, &P.tmap, bb, 0, x1, 0, x3);
+    }
   };
   if (tid == 0) {
     if (first < ntiles) issue(first, 0);
     if (first + stride < ntiles) issue(first + stride, 1);
   }
-  const float2* __restrict__ qin = reinterpret_cast<const float2*>(P.qin);
-  float2* __restrict__ qout = reinterpret_cast<float2*>(P.qout);
+  const float2* const qin = reinterpret_cast<const float2*>(P.qin);
+  const float hh = (float)P.h;
+  const double e24 = P.h / 24.0;
+  const float h24 = (float)e24, h24lo = (float)(e24 - (double)h24);  // a step size rounded to FP32 would drift
+  double red0 = 0.0, red1 = 0.0;
   uint32_t k = 0;
-  for (uint32_t tile = first; tile < ntiles; tile += stride, k++) {
+  for (uint32_t t_ = first; t_ < ntiles; t_ += stride, k++) {
     const int b = (int)(k & 1u);
-    const uint32_t zb = tile_base(L, tile);
+    const uint32_t zb = tile_base(L, number(t_));
     const uint32_t zj = zb | zoff[0];  // index of the thread's first amplitude
     float4 acc[8];
     if (qin) {
@@ -230,6 +320,45 @@ __global__ void __launch_bounds__(kXThreads, 1) k_partial_x(const __grid_constan
     } else {
 #pragma unroll
       for (int r = 0; r < 8; r++) acc[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if constexpr (FAR) {
+      // products that no layout holds (the pass waits on these loads): half of the pairs are added
+      // while the other half's partners are on their way
+      auto far_load = [&](const XFlip& f, int r0, float4 (&g)[4]) {
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+          g[r] = __ldcg(reinterpret_cast<const float4*>(src + ((zb + zoff[r0 + r]) ^ (f.lx & ~1u))));
+      };
+      auto far_add = [&](const XFlip& f, int r0, const float4 (&g)[4]) {
+        const bool sw = (f.lx & 1u) != 0u;
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+          const int r = r0 + i;
+          const float4 v = sw ? swap_pair(g[i]) : g[i];
+          if (f.par) {
+            const bool odd = (__popc((zb + zoff[r]) & f.par) & 1u) != 0u;
+            const float c0 = odd ? f.c : 0.f, c1 = odd != sw ? f.c : 0.f;
+            acc[r].x = fmaf(c0, v.x, acc[r].x);
+            acc[r].y = fmaf(c0, v.y, acc[r].y);
+            acc[r].z = fmaf(c1, v.z, acc[r].z);
+            acc[r].w = fmaf(c1, v.w, acc[r].w);
+          } else {
+            fma4(acc[r], f.c, v);
+          }
+        }
+      };
+      float4 g0[4], g1[4];
+      XFlip f = s_f[np];
+      far_load(f, 0, g0);
+      far_load(f, 4, g1);
+      for (int kk = np; kk < nf; kk++) {
+        const XFlip fn = s_f[kk + 1 < nf ? kk + 1 : kk];
+        far_add(f, 0, g0);
+        if (kk + 1 < nf) far_load(fn, 0, g0);
+        far_add(f, 4, g1);
+        if (kk + 1 < nf) far_load(fn, 4, g1);
+        f = fn;
+      }
     }
     const bool ok = mbar_wait(b ? bar1 : bar0, (k >> 1) & 1u);
     if (__syncthreads_or(!ok)) {  // uniform: a copy that never completed (not expected)
@@ -313,10 +442,98 @@ __global__ void __launch_bounds__(kXThreads, 1) k_partial_x(const __grid_constan
         }
       }
     }
+    // epilogue, one pair after the other; the vectors it reads come one pair ahead
+    constexpr int NV = MODE == MODE_STEP ? 4 : (MODE == MODE_RK4 ? 2 : 0);
+    float4 in[2][NV > 0 ? NV : 1];
+    auto fetch = [&](int r, float4 (&v)[NV > 0 ? NV : 1]) {
+      const uint32_t z = zb + zoff[r];
+      if constexpr (MODE == MODE_STEP) {
 #pragma unroll
-    for (int r = 0; r < 8; r++) *reinterpret_cast<float4*>(qout + (zb + zoff[r])) = acc[r];
+        for (int i = 0; i < 4; i++) v[i] = *reinterpret_cast<const float4*>(reinterpret_cast<const float2*>(P.f[i]) + z);
+      } else if constexpr (MODE == MODE_RK4) {
+        v[0] = *reinterpret_cast<const float4*>(reinterpret_cast<const float2*>(P.y) + z);
+        if (P.stage > 1) v[1] = *reinterpret_cast<const float4*>(reinterpret_cast<const float2*>(P.acc) + z);
+      }
+    };
+    if (NV > 0) fetch(0, in[0]);
+    const uint8_t* const code = base + M.code + ((size_t)b << kXTileBits);
+    float t0 = 0.f, t1 = 0.f;
+#pragma unroll
+    for (int r = 0; r < 8; r++) {
+      if (NV > 0 && r < 7) fetch(r + 1, in[(r + 1) & 1]);
+      const uint32_t z = zb + zoff[r], j = jw | ((uint32_t)r << 6);
+      float4 a = acc[r];
+      const float4 w = own[r];
+      if (DIAG) {
+        int k0 = 0, k1 = 0;
+        if (P.dcode) {
+          const uint32_t two = *reinterpret_cast<const uint16_t*>(code + j);
+          k0 = (int)(two & 0xffu);
+          k1 = (int)(two >> 8);
+        }
+        float d0 = fmaf(wtab, (float)k0, dconst), d1 = fmaf(wtab, (float)k1, dconst);
+        if (others) {
+          d0 += x_other_diagonal(P, s_z, k0, z);
+          d1 += x_other_diagonal(P, s_z, k1, z + 1u);
+        }
+        if (d0 != 0.f) {
+          a.x = fmaf(d0, w.x, a.x);
+          a.y = fmaf(d0, w.y, a.y);
+        }
+        if (d1 != 0.f) {
+          a.z = fmaf(d1, w.z, a.z);
+          a.w = fmaf(d1, w.w, a.w);
+        }
+      }
+      auto put = [&](void* v, const float4& x) { *reinterpret_cast<float4*>(reinterpret_cast<float2*>(v) + z) = x; };
+      const float4 fn = make_float4(a.y, -a.x, a.w, -a.z);  // -i r
+      if constexpr (MODE == MODE_PARTIAL) {
+        put(P.qout, a);
+      } else if constexpr (MODE == MODE_DERIV) {
+        put(P.fout, fn);
+      } else if constexpr (MODE == MODE_ENERGY) {
+        t0 += (w.x * a.x + w.y * a.y) + (w.z * a.z + w.w * a.w);
+        t1 += (w.x * a.y - w.y * a.x) + (w.z * a.w - w.w * a.z);
+      } else if constexpr (MODE == MODE_STEP) {
+        const float4(&v)[NV] = in[r & 1];  // f_n, f_{n-1}, f_{n-2}, f_{n-3}
+        float4 pn, yn;
+        auto one = [&](float p, float f, float f0, float f1, float f2, float f3, float& po, float& yo) {
+          const float d1 = f - f0, d2 = f0 - f1, d3 = f1 - f2, d4 = f2 - f3;
+          const float s = fmaf(24.f, f, fmaf(40.f, d1, fmaf(-55.f, d2, fmaf(36.f, d3, -9.f * d4))));
+          const float c = 9.f * ((d1 - d4) + 3.f * (d3 - d2));
+          po = p + fmaf(h24, s, h24lo * s);
+          const float e = fmaf(h24, c, h24lo * c);
+          yo = p + e;
+          t1 = fmaf(e, e, t1);  // y - p
+        };
+        one(w.x, fn.x, v[0].x, v[1].x, v[2].x, v[3].x, pn.x, yn.x);
+        one(w.y, fn.y, v[0].y, v[1].y, v[2].y, v[3].y, pn.y, yn.y);
+        one(w.z, fn.z, v[0].z, v[1].z, v[2].z, v[3].z, pn.z, yn.z);
+        one(w.w, fn.w, v[0].w, v[1].w, v[2].w, v[3].w, pn.w, yn.w);
+        put(P.fout, fn);
+        put(P.pout, pn);
+        if (P.yout) put(P.yout, yn);
+      } else if constexpr (MODE == MODE_RK4) {
+        const float4 y = in[r & 1][0];
+        float4 s = in[r & 1][1];
+        if (P.stage == 1) {
+          put(P.fout, fn);  // history f_n
+          s = fn;
+        } else {
+          const float m = P.stage == 4 ? 1.f : 2.f;
+          s = make_float4(fmaf(m, fn.x, s.x), fmaf(m, fn.y, s.y), fmaf(m, fn.z, s.z), fmaf(m, fn.w, s.w));
+        }
+        const float c = P.stage == 4 ? hh / 6.f : (P.stage == 3 ? hh : 0.5f * hh);
+        const float4 u = P.stage == 4 ? s : fn;
+        const float4 x = make_float4(fmaf(c, u.x, y.x), fmaf(c, u.y, y.y), fmaf(c, u.z, y.z), fmaf(c, u.w, y.w));
+        if (P.stage < 4) put(P.acc, s);
+        put(P.stage < 4 ? P.pout : P.y, x);
+      }
+    }
+    red0 += (double)t0;
+    red1 += (double)t1;
     __syncthreads();  // every read of buffer b is done: it can take the tile after next
-    if (tid == 0 && tile + 2 * stride < ntiles) issue(tile + 2 * stride, b);
+    if (tid == 0 && t_ + 2 * stride < ntiles) issue(t_ + 2 * stride, b);
   }
   // A CTA that gave up at tile k leaves only after the copies issued for tiles k and k + 1 have
   // landed (bounded); after a normal end no copy is outstanding.
@@ -325,44 +542,100 @@ __global__ void __launch_bounds__(kXThreads, 1) k_partial_x(const __grid_constan
       if (first + kq * stride < ntiles) (void)mbar_wait((kq & 1u) ? bar1 : bar0, (kq >> 1) & 1u);
   }
   __syncthreads();
+  if (MODE != MODE_STEP && MODE != MODE_ENERGY) return;
+  // FP64 sums: lanes, warps and CTAs in a fixed order; the last CTA writes the result slots
+  auto cta_sum = [&](double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if (lane == 0) s_red[warp] = v;
+    __syncthreads();
+    double s = 0.0;
+    if (tid == 0)
+      for (int w = 0; w < kXThreads / 32; w++) s += s_red[w];
+    return s;
+  };
+  __shared__ int s_last;
+  const double v0 = MODE == MODE_ENERGY ? cta_sum(red0) : 0.0, v1 = cta_sum(red1);
+  if (tid == 0) {
+    P.partials[2 * blockIdx.x] = v0;
+    P.partials[2 * blockIdx.x + 1] = v1;
+    __threadfence();
+    s_last = atomicAdd(P.counter, 1u) == gridDim.x - 1 ? 1 : 0;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  double a0 = 0.0, a1 = 0.0;
+  for (uint32_t i = tid; i < gridDim.x; i += blockDim.x) {
+    a0 += __ldcg(&P.partials[2 * i]);
+    a1 += __ldcg(&P.partials[2 * i + 1]);
+  }
+  a0 = cta_sum(a0);
+  a1 = cta_sum(a1);
+  if (tid == 0) {
+    if (MODE == MODE_ENERGY) {
+      P.slots[kSlotDot] = a0;
+      P.slots[kSlotDotIm] = a1;
+    } else {
+      const double e = (19.0 / 270.0) * sqrt(a1);
+      P.slots[kSlotLastErr] = e;
+      if (!(e <= P.slots[kSlotMaxErr])) P.slots[kSlotMaxErr] = e;  // NaN propagates
+    }
+    *P.counter = 0u;
+  }
 }
 
-}  // namespace
-
-bool xpartial_layout_ok(const Layout& L) {
-  // TMA box: the chunk as 2^(c+1) floats (one box row up to c = 7, else 256 x 2^(c-7)), 2^w <= 256
-  // rows; a strided tile of 2^13 amplitudes
-  return L.cb == 0 && L.t == kXTileBits && L.c >= 1 && L.c <= 12 && L.w >= 1 && L.w <= 8 && L.h > L.c;
-}
-
-size_t xpartial_smem_bytes(int n_flips) {
-  return 1024 + 2 * (size_t)kXTileBytes + (((size_t)n_flips * sizeof(XFlip) + 15) & ~(size_t)15) + 16;
-}
-
-cudaError_t launch_partial_x(const XPartialParams& p, int smem, cudaStream_t s) {
-  static int configured = 0, cached_dev = -1, cached_smem = -1, cached_g = 0;
-  if (smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_partial_x, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+template <int MODE, bool DIAG, bool FAR = false>
+cudaError_t launch_x(const XParams& p, int n_flips, int n_z, cudaStream_t s) {
+  const size_t smem = XSmem(n_flips, n_z, DIAG && p.dcode).total;
+  auto kern = k_tile_x<MODE, DIAG, FAR>;
+  static int configured = 0, cached_dev = -1, cached_g = 0;
+  if ((int)smem > configured) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    configured = smem;
+    configured = (int)smem;
   }
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (!(dev == cached_dev && smem == cached_smem)) {
-    int sms = 0, per = 0;
+  if (dev != cached_dev) {  // one CTA per multiprocessor (two tiles fill its shared memory)
+    int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_partial_x, kXThreads, smem);
     if (e != cudaSuccess) return e;
     cached_dev = dev;
-    cached_smem = smem;
-    cached_g = sms * (per < 1 ? 1 : per);
+    cached_g = sms;
   }
   int g = cached_g;
   if (p.max_grid > 0 && g > p.max_grid) g = p.max_grid;
   if ((uint32_t)g > p.ntiles) g = (int)p.ntiles;
-  k_partial_x<<<g, kXThreads, smem, s>>>(p);
+  kern<<<g, kXThreads, smem, s>>>(p);
   return cudaGetLastError();
+}
+
+}  // namespace
+
+bool tile_x_layout_ok(const Layout& L) {
+  if (L.cb != 0 || L.t != kXTileBits) return false;
+  // TMA box: the chunk as 2^(c+1) floats (one box row up to c = 7, else 256 x 2^(c-7)), 2^w <= 256
+  // rows; or a contiguous tile
+  return L.w == 0 || (L.c >= 1 && L.c <= 12 && L.w <= 8 && L.h > L.c);
+}
+
+size_t tile_x_smem_bytes(int n_flips, int n_z, bool codes) { return XSmem(n_flips, n_z, codes).total; }
+
+cudaError_t launch_tile_x(const XParams& p, int n_flips, int n_z, cudaStream_t s) {
+  if (p.with_remote && (p.mode != MODE_PARTIAL || p.with_diag)) return cudaErrorInvalidValue;
+  switch (p.mode) {
+    case MODE_PARTIAL: return p.with_diag ? launch_x<MODE_PARTIAL, true>(p, n_flips, n_z, s)
+                             : p.with_remote ? launch_x<MODE_PARTIAL, false, true>(p, n_flips, 0, s)
+                                             : launch_x<MODE_PARTIAL, false>(p, n_flips, 0, s);
+    case MODE_STEP: return launch_x<MODE_STEP, true>(p, n_flips, n_z, s);
+    case MODE_RK4: return launch_x<MODE_RK4, true>(p, n_flips, n_z, s);
+    case MODE_DERIV: return launch_x<MODE_DERIV, true>(p, n_flips, n_z, s);
+    case MODE_ENERGY: return launch_x<MODE_ENERGY, true>(p, n_flips, n_z, s);
+  }
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace aqc
