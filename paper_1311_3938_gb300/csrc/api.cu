@@ -2920,6 +2920,74 @@ int aqc_tridiag_eigvals(int k, const double* a, const double* b, int n_eig, doub
   return AQC_OK;
 }
 
+namespace {
+
+// The Lanczos recurrence on H(t) with weights w: basis vectors in `work`, the coefficients alpha_j
+// and beta_j^2 on the device (the context's partials; no pass of a matvec uses them), read a few
+// steps at a time so that the GPU does not wait for the host between steps.
+struct Lanczos {
+  aqc_ctx* c;
+  const double* w;
+  const LzPlan* P;
+  char* base;
+  int max_iter;
+  double *alpha, *nrm2, *coef, *scal;
+  LzScratch sc;
+
+  Lanczos(aqc_ctx* ctx, const double* weights, const LzPlan& plan, void* work, int iters)
+      : c(ctx), w(weights), P(&plan), base((char*)work), max_iter(iters) {
+    alpha = c->d_partials;
+    nrm2 = alpha + iters;
+    coef = (double*)(base + plan.off_coef);
+    scal = (double*)(base + plan.off_scal);
+    sc = LzScratch{(double*)(base + plan.off_partials), 2 * ((uint64_t)iters + 1) * plan.G, c->d_counter};
+  }
+  uint64_t ld() const { return P->ld_bytes / c->amp; }
+  void* V(int i) const { return base + (size_t)i * P->ld_bytes; }
+
+  int begin(const void* start) {  // v_0 = start / ||start||
+    if (c->permuted) {
+      int rc = to_library_order(c, V(0), start);
+      if (rc) return rc;
+    } else {
+      CUDA_TRY(c, cudaMemcpyAsync(V(0), start, c->N * c->amp, cudaMemcpyDeviceToDevice, c->stream));
+    }
+    CUDA_TRY(c, launch_dotc_multi(c->prec, V(0), ld(), 1, V(0), c->N, sc, scal, nullptr, 0, c->stream));
+    CUDA_TRY(c, launch_scale_to(c->prec, V(0), V(0), c->N, scal, c->stream));
+    c->launches += 2;
+    return AQC_OK;
+  }
+  int step(int j) {  // v_{j+1}, alpha_j and ||r_j||^2 = beta_j^2 (classical Gram-Schmidt, twice)
+    ApplyParams fin = base_params(c);
+    fin.mode = MODE_PARTIAL;
+    int rc = evaluate(c, w, V(j), fin, V(j + 1));
+    if (rc) return rc;
+    for (int pass = 0; pass < 2; pass++) {
+      CUDA_TRY(c, launch_dotc_multi(c->prec, V(0), ld(), (uint32_t)(j + 1), V(j + 1), c->N, sc, coef, alpha + j, pass + 1,
+                                    c->stream));
+      CUDA_TRY(c, launch_sub_multi(c->prec, V(j + 1), V(0), ld(), (uint32_t)(j + 1), coef, c->N, sc,
+                                   pass ? nrm2 + j : nullptr, c->stream));
+    }
+    CUDA_TRY(c, launch_scale_to(c->prec, V(j + 1), V(j + 1), c->N, nrm2 + j, c->stream));
+    c->launches += 5;
+    return AQC_OK;
+  }
+  // steps [j, j + count) and their coefficients (steps past an invariant subspace are harmless: the
+  // caller ignores what they give)
+  int steps(int j, int count, double* a, double* n2) {
+    for (int i = 0; i < count; i++) {
+      int rc = step(j + i);
+      if (rc) return rc;
+    }
+    CUDA_TRY(c, cudaMemcpyAsync(a, alpha + j, count * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(c, cudaMemcpyAsync(n2, nrm2 + j, count * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    return AQC_OK;
+  }
+};
+
+}  // namespace
+
 int aqc_lanczos(aqc_ctx* ctx, double t, const void* start, void* work, size_t work_bytes, int max_iter, int n_eig,
                 double tol, double* eig, double* conv, int* iters_out) {
   if (!ctx) return AQC_E_INVAL;
@@ -2937,68 +3005,41 @@ int aqc_lanczos(aqc_ctx* ctx, double t, const void* start, void* work, size_t wo
   }
   double w[3];
   sched_weights(ctx, t, w);
-  char* base = (char*)work;
-  const uint64_t ld = P.ld_bytes / ctx->amp;  // elements between basis vectors
-  auto V = [&](int i) { return (void*)(base + (size_t)i * P.ld_bytes); };
-  double* partials = (double*)(base + P.off_partials);
-  double* coef = (double*)(base + P.off_coef);
-  double* h = (double*)(base + P.off_h);
-  double* scal = (double*)(base + P.off_scal);
   cudaStream_t s = ctx->stream;
-  const uint64_t N = ctx->N;
-  // v_0 = start / ||start||
-  if (ctx->permuted) {
-    int rc = to_library_order(ctx, V(0), start);
-    if (rc) return rc;
-  } else {
-    CUDA_TRY(ctx, cudaMemcpyAsync(V(0), start, N * ctx->amp, cudaMemcpyDeviceToDevice, s));
-  }
-  CUDA_TRY(ctx, launch_dotc_multi(ctx->prec, V(0), ld, 1, V(0), N, partials, scal, nullptr, s));
-  CUDA_TRY(ctx, launch_scale_to(ctx->prec, V(0), V(0), N, scal, s));
-  ctx->launches += 3;
+  Lanczos K(ctx, w, P, work, max_iter);
+  int rc = K.begin(start);
+  if (rc) return rc;
+  constexpr int kChunk = 8;  // steps between convergence checks
+  double ca[kChunk], cn[kChunk];
   std::vector<double> alpha, beta, prev(n_eig, 0.0), cur(n_eig, 0.0), chg(n_eig, INFINITY);
   int iters = 0;
-  bool have_prev = false;
-  for (int j = 0; j < max_iter; j++) {
-    void* wv = V(j + 1);
-    ApplyParams fin = base_params(ctx);
-    fin.mode = MODE_PARTIAL;
-    int rc = evaluate(ctx, w, V(j), fin, wv);
+  bool have_prev = false, stop = false;
+  for (int j0 = 0; j0 < max_iter && !stop; j0 += kChunk) {
+    const int count = std::min(kChunk, max_iter - j0);
+    rc = K.steps(j0, count, ca, cn);
     if (rc) return rc;
-    CUDA_TRY(ctx, cudaMemsetAsync(h, 0, (size_t)(j + 1) * 2 * sizeof(double), s));
-    for (int pass = 0; pass < 2; pass++) {  // classical Gram-Schmidt, twice
-      CUDA_TRY(ctx, launch_dotc_multi(ctx->prec, V(0), ld, (uint32_t)(j + 1), wv, N, partials, coef, h, s));
-      CUDA_TRY(ctx, launch_sub_multi(ctx->prec, wv, V(0), ld, (uint32_t)(j + 1), coef, N, s));
-      ctx->launches += 3;
-    }
-    CUDA_TRY(ctx, launch_dotc_multi(ctx->prec, wv, ld, 1, wv, N, partials, scal, nullptr, s));
-    ctx->launches += 2;
-    double hj[2], nrm2[2];
-    CUDA_TRY(ctx, cudaMemcpyAsync(hj, h + 2 * j, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(ctx, cudaMemcpyAsync(nrm2, scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(ctx, cudaStreamSynchronize(s));
-    if (!std::isfinite(hj[0]) || !std::isfinite(nrm2[0])) FAIL(ctx, AQC_E_NUMERIC, "non-finite Lanczos coefficient");
-    alpha.push_back(hj[0]);
-    const double bj = sqrt(std::max(nrm2[0], 0.0));
-    iters = j + 1;
-    const bool invariant = bj <= 1e-13 * std::max(1.0, fabs(hj[0]));
-    const int m = std::min(n_eig, iters);
-    const bool check = invariant || iters == max_iter || iters % 8 == 0;
-    if (check && iters >= n_eig) {
-      for (int e = 0; e < m; e++) cur[e] = tridiag_eig(alpha.data(), beta.data(), iters, e);
-      bool done = have_prev;
-      for (int e = 0; e < m; e++) {
-        chg[e] = have_prev ? fabs(cur[e] - prev[e]) : INFINITY;
-        done = done && chg[e] <= tol * std::max(1.0, fabs(cur[e]));
+    for (int i = 0; i < count && !stop; i++) {
+      if (!std::isfinite(ca[i]) || !std::isfinite(cn[i])) FAIL(ctx, AQC_E_NUMERIC, "non-finite Lanczos coefficient");
+      alpha.push_back(ca[i]);
+      const double bj = sqrt(std::max(cn[i], 0.0));
+      iters = j0 + i + 1;
+      const bool invariant = bj <= 1e-13 * std::max(1.0, fabs(ca[i]));
+      const int m = std::min(n_eig, iters);
+      const bool check = invariant || iters == max_iter || iters % kChunk == 0;
+      if (check && iters >= n_eig) {
+        for (int e = 0; e < m; e++) cur[e] = tridiag_eig(alpha.data(), beta.data(), iters, e);
+        bool done = have_prev;
+        for (int e = 0; e < m; e++) {
+          chg[e] = have_prev ? fabs(cur[e] - prev[e]) : INFINITY;
+          done = done && chg[e] <= tol * std::max(1.0, fabs(cur[e]));
+        }
+        prev = cur;
+        have_prev = true;
+        stop = done;
       }
-      prev = cur;
-      have_prev = true;
-      if (done || invariant) break;
+      stop = stop || invariant;
+      if (!stop) beta.push_back(bj);
     }
-    if (invariant) break;
-    beta.push_back(bj);
-    CUDA_TRY(ctx, launch_scale_to(ctx->prec, wv, wv, N, scal, s));
-    ctx->launches++;
   }
   CUDA_TRY(ctx, cudaStreamSynchronize(s));  // the caller's work buffer is free on return
   const int m = std::min(n_eig, iters);
@@ -3027,61 +3068,40 @@ int aqc_lanczos_ground(aqc_ctx* ctx, double t, const void* start, void* work, si
   }
   double w[3];
   sched_weights(ctx, t, w);
-  char* base = (char*)work;
-  const uint64_t ld = P.ld_bytes / ctx->amp;
-  auto V = [&](int i) { return (void*)(base + (size_t)i * P.ld_bytes); };
-  double* partials = (double*)(base + P.off_partials);
-  double* coef = (double*)(base + P.off_coef);
-  double* h = (double*)(base + P.off_h);
-  double* scal = (double*)(base + P.off_scal);
   cudaStream_t s = ctx->stream;
   const uint64_t N = ctx->N;
   const size_t bytes = (size_t)N * ctx->amp;
-  if (ctx->permuted) {
-    int rc = to_library_order(ctx, V(0), start);
-    if (rc) return rc;
-  } else {
-    CUDA_TRY(ctx, cudaMemcpyAsync(V(0), start, bytes, cudaMemcpyDeviceToDevice, s));
-  }
-  CUDA_TRY(ctx, launch_dotc_multi(ctx->prec, V(0), ld, 1, V(0), N, partials, scal, nullptr, s));
-  CUDA_TRY(ctx, launch_scale_to(ctx->prec, V(0), V(0), N, scal, s));
-  ctx->launches += 3;
+  Lanczos K(ctx, w, P, work, max_iter);
+  const uint64_t ld = K.ld();
+  double *const coef = K.coef, *const scal = K.scal;
+  auto V = [&](int i) { return K.V(i); };
+  int rc = K.begin(start);
+  if (rc) return rc;
+  constexpr int kChunk = 4;  // steps between residual checks
+  double ca[kChunk], cn[kChunk];
   std::vector<double> alpha, beta, sv;
   int iters = 0;
   double theta = 0.0;
-  for (int j = 0; j < max_iter; j++) {
-    void* wv = V(j + 1);
-    ApplyParams fin = base_params(ctx);
-    fin.mode = MODE_PARTIAL;
-    int rc = evaluate(ctx, w, V(j), fin, wv);
+  bool stop = false;
+  for (int j0 = 0; j0 < max_iter && !stop; j0 += kChunk) {
+    const int count = std::min(kChunk, max_iter - j0);
+    rc = K.steps(j0, count, ca, cn);
     if (rc) return rc;
-    CUDA_TRY(ctx, cudaMemsetAsync(h, 0, (size_t)(j + 1) * 2 * sizeof(double), s));
-    for (int pass = 0; pass < 2; pass++) {  // classical Gram-Schmidt, twice
-      CUDA_TRY(ctx, launch_dotc_multi(ctx->prec, V(0), ld, (uint32_t)(j + 1), wv, N, partials, coef, h, s));
-      CUDA_TRY(ctx, launch_sub_multi(ctx->prec, wv, V(0), ld, (uint32_t)(j + 1), coef, N, s));
-      ctx->launches += 3;
+    for (int i = 0; i < count && !stop; i++) {
+      if (!std::isfinite(ca[i]) || !std::isfinite(cn[i])) FAIL(ctx, AQC_E_NUMERIC, "non-finite Lanczos coefficient");
+      alpha.push_back(ca[i]);
+      const double bj = sqrt(std::max(cn[i], 0.0));
+      iters = j0 + i + 1;
+      const bool invariant = bj <= 1e-13 * std::max(1.0, fabs(ca[i]));
+      if (invariant || iters == max_iter || iters % kChunk == 0) {
+        // Ritz residual of the lowest pair: ||H x - theta x|| = beta_j |s_last|
+        theta = tridiag_eig(alpha.data(), beta.data(), iters, 0);
+        sv.assign(iters, 0.0);
+        tridiag_eigvec(alpha.data(), beta.data(), iters, theta, sv.data());
+        stop = invariant || bj * fabs(sv[iters - 1]) <= tol * std::max(1.0, fabs(theta));
+      }
+      if (!stop) beta.push_back(bj);
     }
-    CUDA_TRY(ctx, launch_dotc_multi(ctx->prec, wv, ld, 1, wv, N, partials, scal, nullptr, s));
-    ctx->launches += 2;
-    double hj[2], nrm2[2];
-    CUDA_TRY(ctx, cudaMemcpyAsync(hj, h + 2 * j, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(ctx, cudaMemcpyAsync(nrm2, scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
-    CUDA_TRY(ctx, cudaStreamSynchronize(s));
-    if (!std::isfinite(hj[0]) || !std::isfinite(nrm2[0])) FAIL(ctx, AQC_E_NUMERIC, "non-finite Lanczos coefficient");
-    alpha.push_back(hj[0]);
-    const double bj = sqrt(std::max(nrm2[0], 0.0));
-    iters = j + 1;
-    const bool invariant = bj <= 1e-13 * std::max(1.0, fabs(hj[0]));
-    if (invariant || iters == max_iter || iters % 4 == 0) {
-      // Ritz residual of the lowest pair: ||H x - theta x|| = beta_j |s_last|
-      theta = tridiag_eig(alpha.data(), beta.data(), iters, 0);
-      sv.assign(iters, 0.0);
-      tridiag_eigvec(alpha.data(), beta.data(), iters, theta, sv.data());
-      if (invariant || bj * fabs(sv[iters - 1]) <= tol * std::max(1.0, fabs(theta)) || iters == max_iter) break;
-    }
-    beta.push_back(bj);
-    CUDA_TRY(ctx, launch_scale_to(ctx->prec, wv, wv, N, scal, s));
-    ctx->launches++;
   }
   // x = sum_i s_i v_i into V(iters) (free: the last, unnormalised residual), then unit norm
   void* x = V(iters);
@@ -3089,28 +3109,26 @@ int aqc_lanczos_ground(aqc_ctx* ctx, double t, const void* start, void* work, si
   for (int i = 0; i < iters; i++) c[2 * (size_t)i] = -sv[i];
   CUDA_TRY(ctx, cudaMemcpyAsync(coef, c.data(), c.size() * sizeof(double), cudaMemcpyHostToDevice, s));
   CUDA_TRY(ctx, cudaMemsetAsync(x, 0, bytes, s));
-  CUDA_TRY(ctx, launch_sub_multi(ctx->prec, x, V(0), ld, (uint32_t)iters, coef, N, s));
-  CUDA_TRY(ctx, launch_dotc_multi(ctx->prec, x, ld, 1, x, N, partials, scal, nullptr, s));
+  CUDA_TRY(ctx, launch_sub_multi(ctx->prec, x, V(0), ld, (uint32_t)iters, coef, N, K.sc, scal, s));
   CUDA_TRY(ctx, launch_scale_to(ctx->prec, x, x, N, scal, s));
-  ctx->launches += 4;
+  ctx->launches += 2;
   // residual ||H x - theta x|| with one more matvec (into the scratch vector)
   {
     ApplyParams fin = base_params(ctx);
     fin.mode = MODE_PARTIAL;
-    int rc = evaluate(ctx, w, x, fin, ctx->vec[V_ACC]);
+    rc = evaluate(ctx, w, x, fin, ctx->vec[V_ACC]);
     if (rc) return rc;
     const double th[2] = {theta, 0.0};
     CUDA_TRY(ctx, cudaMemcpyAsync(coef, th, sizeof(th), cudaMemcpyHostToDevice, s));
-    CUDA_TRY(ctx, launch_sub_multi(ctx->prec, ctx->vec[V_ACC], x, ld, 1, coef, N, s));
-    CUDA_TRY(ctx, launch_dotc_multi(ctx->prec, ctx->vec[V_ACC], ld, 1, ctx->vec[V_ACC], N, partials, scal, nullptr, s));
-    ctx->launches += 3;
+    CUDA_TRY(ctx, launch_sub_multi(ctx->prec, ctx->vec[V_ACC], x, ld, 1, coef, N, K.sc, scal, s));
+    ctx->launches += 1;
     double r2[2];
     CUDA_TRY(ctx, cudaMemcpyAsync(r2, scal, sizeof(r2), cudaMemcpyDeviceToHost, s));
     CUDA_TRY(ctx, cudaStreamSynchronize(s));
     if (resid_out) *resid_out = sqrt(std::max(r2[0], 0.0));
   }
   if (ctx->permuted) {
-    int rc = to_qubit_order(ctx, ground_out, x);
+    rc = to_qubit_order(ctx, ground_out, x);
     if (rc) return rc;
   } else {
     CUDA_TRY(ctx, cudaMemcpyAsync(ground_out, x, bytes, cudaMemcpyDeviceToDevice, s));

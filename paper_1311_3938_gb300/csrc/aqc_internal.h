@@ -350,10 +350,16 @@ bool tile_x_layout_ok(const Layout& L);
 size_t tile_x_smem_bytes(int n_flips, int n_z, bool codes);
 cudaError_t launch_tile_x(const XParams& p, int n_flips, int n_z, cudaStream_t s);
 uint32_t lanczos_dot_blocks(uint64_t N);
+// scratch of the Lanczos reductions: partial sums and a ticket (zero between launches)
+struct LzScratch {
+  double* partials;
+  uint64_t doubles;
+  unsigned* counter;
+};
 cudaError_t launch_dotc_multi(int prec, const void* V, uint64_t ld, uint32_t m, const void* w, uint64_t N,
-                              double* partials, double* out, double* acc, cudaStream_t s);
+                              const LzScratch& sc, double* out, double* acc, int mode, cudaStream_t s);
 cudaError_t launch_sub_multi(int prec, void* w, const void* V, uint64_t ld, uint32_t m, const double* c, uint64_t N,
-                             cudaStream_t s);
+                             const LzScratch& sc, double* norm, cudaStream_t s);
 cudaError_t launch_scale_to(int prec, void* v, const void* w, uint64_t N, const double* nrm2, cudaStream_t s);
 cudaError_t launch_diag_codes(uint8_t* out, uint64_t N, const DevTables* tab, int cls, cudaStream_t s);
 cudaError_t launch_init(int prec, void* y, uint64_t N, int kind, uint64_t basis, double amp, cudaStream_t s);
