@@ -483,6 +483,13 @@ void plan_slabs(aqc_ctx* c) {
   S.done = c->d_sync + 1;
 }
 
+// Threads that own a tile of so many slots: 512 with one or two each, 256 with eight or sixteen (512
+// threads beside the service warps leave 96 registers: four and eight slots each spilled; complex64,
+// nonlinear path, n = 20 38.1 -> 35.9 us per step, n = 19 22.1 -> 21.7).
+int resident_threads(int slots) {
+  return slots >= 4 * kResMaxThreads ? kResMaxThreads / 2 : std::max(32, std::min(kResMaxThreads, slots));
+}
+
 // Products of a resident launch on tiles of 2^R.t by partner tile (the bits they flip above t; the
 // own tile, no such bit, first) into `rt`, and their counts and buffers into R.  False where the
 // tables leave no room for two partner buffers: such products stay on the layout passes.
@@ -551,16 +558,22 @@ void plan_resident(aqc_ctx* c) {
   if (!resident_size(c)) return;
   ResPlan R;
   const int H = c->prec == AQC_C128 ? 1 : 2;
-  // One tile while a step on one CTA takes less than an exchange between several; then at most
-  // 128 tiles (one per multiprocessor) of at least 2^8 complex64 / 2^7 complex128 amplitudes.
-  // Microseconds per step (linear / nonlinear path): complex64 n = 9 on one tile 1.8 / 2.2, on two
-  // 3.0 / 3.2; n = 10 on one 2.6 / 3.5, on four 2.7 / 2.9; n = 12 with tiles of 2^7 3.5 / 3.9, 2^8
-  // 3.2 / 3.8, 2^10 3.6 / 4.5; n = 16 with 2^9 4.6 / 5.4, 2^11 5.3 / 9.1.  complex128 n = 7 on one
-  // tile 3.0 / 4.3, on two 3.6 / 4.8; n = 8 on one 4.6 / 6.5, on two 3.9 / 5.1.
+  // One tile while a step on one CTA takes less than an exchange between several; then at most 16
+  // tiles, one cluster, while their work is short beside an exchange through memory; then at most 128
+  // tiles (one per multiprocessor).  Microseconds per step (linear / nonlinear path): complex64 n = 9 on
+  // one tile 1.8 / 2.3, on a cluster of two 2.2 / 2.9; n = 13 on 16 tiles 3.0 / 3.8, on 32 beyond a
+  // cluster 3.6 / 3.9; n = 14 on 16 tiles 3.6 / 5.5, on 64 3.8 / 4.4.  complex128 n = 7 on one tile 3.1 / 4.4, on
+  // a cluster of four 3.4 / 4.6; n = 10 on 16 tiles 3.6 / 5.5, on 8 3.9 / 5.6; n = 12 on 16 tiles 5.3 / 8.6, on
+  // 32 beyond a cluster 4.7 / 6.4.
   const bool c128 = c->prec == AQC_C128;
-  R.t = c->n <= (c128 ? 7 : 9) ? c->n : std::max(c128 ? 7 : 8, c->n - 7);
+  if (c->n <= (c128 ? 7 : 9))
+    R.t = c->n;
+  else if (c128)
+    R.t = c->n <= 10 ? 6 : std::max(7, c->n - 7);
+  else
+    R.t = c->n <= 13 ? std::max(8, c->n - 4) : std::max(8, c->n - 7);
   const int slots_all = std::max(1, (1 << R.t) / H);
-  R.nth = std::max(32, std::min(kResMaxThreads, slots_all));
+  R.nth = resident_threads(slots_all);
   R.slots = std::max(1, slots_all / R.nth);
   R.on = resident_tables(c, R, &c->h_res.alone);
   c->res = R;
@@ -1010,6 +1023,20 @@ ResParams resident_params(aqc_ctx* c) {
 }
 
 int launch_resident_on(aqc_ctx* c, const ResParams& p) {
+  const int tiles = 1 << (c->n - c->res.t);
+  if (tiles > 1 && tiles <= kResMaxCluster && c->res.slots == 1 && p.evals > 1 && p.npart > 0 &&
+      c->grid_limit == 0) {
+    ResParams q = p;
+    q.nbuf = 2 * p.npart;
+    if (resident_smem_bytes(c->prec, p.t, q.nbuf, p.np, p.ng, c->n_z, c->res.nth, true) <= kResSmem) {
+      const cudaError_t e = launch_resident_cluster(c->prec, q, c->res.nth, c->n_z, c->stream);
+      if (e == cudaSuccess) {
+        c->launches++;
+        return AQC_OK;
+      }
+      if (e != cudaErrorNotSupported) CUDA_TRY(c, e);  // no room for such a cluster on this device: flags
+    }
+  }
   const int limit = c->grid_limit > 0 ? std::min(c->grid_limit, c->sms) : c->sms;
   CUDA_TRY(c, launch_resident(c->prec, p, c->res.slots, c->res.nth, limit, c->n_z, c->stream));
   c->launches++;
@@ -1626,8 +1653,10 @@ void drop_graph(aqc_batch* b) {
 ResPlan member_plan(const aqc_ctx* c, int tb) {
   ResPlan R;
   R.t = std::min(c->n, tb);
-  R.nth = kResMaxThreads;
-  R.slots = std::max(1, (1 << R.t) / ((c->prec == AQC_C128 ? 1 : 2) * kResMaxThreads));
+  const int slots = (1 << R.t) / (c->prec == AQC_C128 ? 1 : 2);
+  R.nth = std::max(kResMaxThreads / 2, resident_threads(slots));
+  if (slots < kResMaxThreads) R.nth = kResMaxThreads;  // a launch's threads are those of its slot count
+  R.slots = std::max(1, slots / R.nth);
   return R;
 }
 
@@ -1656,7 +1685,7 @@ int batch_plan_waves(aqc_batch* b) {
   };
   auto pack = [&](int tb, std::vector<std::vector<Job>>* out) {  // estimated time, or infinity
     double total = 0.0;
-    for (int S = 1; S <= 8; S *= 2) {
+    for (int S = 1; S <= 16; S *= 2) {
       std::vector<Job> jobs;
       for (int slot : who) {
         const aqc_ctx* c = b->members[slot];

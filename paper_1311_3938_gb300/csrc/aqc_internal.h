@@ -383,6 +383,10 @@ size_t resident_smem_bytes(int prec, int t, int nbuf, int np, int ng, int n_z, i
 // slots: 16-byte slots per thread and tile; max_grid: CTAs at most (fewer than tiles: a CTA walks
 // several tiles and the owned vectors stay in global memory)
 cudaError_t launch_resident(int prec, const ResParams& p, int slots, int nth, int max_grid, int n_z, cudaStream_t s);
+// the same as one thread-block cluster (at most kResMaxCluster tiles of one slot per thread, a buffer
+// set of p.npart partner tiles for each parity of the evaluation: p.nbuf = 2 p.npart)
+constexpr int kResMaxCluster = 16;
+cudaError_t launch_resident_cluster(int prec, const ResParams& p, int nth, int n_z, cudaStream_t s);
 cudaError_t launch_resident_batch(int prec, const ResBatch& b, int slots, int ctas, size_t smem, cudaStream_t s);
 int64_t fma64_count(int blocks, int iters);
 int reduce_grid(uint64_t N);

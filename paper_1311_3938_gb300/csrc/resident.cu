@@ -23,13 +23,17 @@
 // multiprocessor's pipe for about 19 cycles, so reducing by shuffles in every warp would take
 // longer than a small state's step.
 //
+// Up to 16 tiles run as one thread-block cluster and push their tiles into one another's shared
+// memory instead: no flags, no trip through L2.
+//
 // Measured, microseconds per predictor-corrector step (before: one launch per layout pass, replayed
 // from a graph, each on as many CTAs as the state has 64 KiB tiles):
-//   complex64, nonlinear path: n = 12 31 -> 3.8, n = 16 43 -> 5.4, n = 18 46 -> 10.5, n = 20 50 -> 36
-//   complex128, linear path:   n = 10 20 -> 3.4, n = 16 about 55 -> 10.4, n = 18 72 -> 41
-// Below n = 14 a step is the exchange (about 1.5 us from the last store to the first partner read)
-// and one pass of dependent shared-memory reads; above it complex64 is bound by the
-// shared-memory reads of the partners (16 bytes per product and slot), complex128 by the FP64 pipe.
+//   complex64, nonlinear path: n = 8 11 -> 1.8, n = 12 31 -> 2.4, n = 16 43 -> 4.3, n = 18 46 -> 8.8, n = 20 50 -> 36
+//   complex128, linear path:   n = 10 20 -> 3.6, n = 14 68 -> 4.9, n = 16 71 -> 11, n = 18 72 -> 42
+// An exchange takes about 0.8 us in a cluster and 1.5 us through memory (from the last store to the
+// first partner read); the rest of a small state's step is dependent shared-memory reads and, in
+// complex128, FP64 latency.  Above n = 14 complex64 is bound by the shared-memory reads of the
+// partners (16 bytes per product and slot), complex128 by the FP64 pipe.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -78,6 +82,10 @@ struct RScal {        // diagonal of one evaluation
 
 constexpr uint32_t kResPolls = 1u << 22;  // flag and mbarrier polls before a wait gives up
 constexpr int kService = 128;             // threads beside those that own amplitudes: four warps
+
+// threads that own amplitudes, at most: sixteen slots per thread need more registers than 512 threads
+// (and the service warps) leave
+__host__ __device__ constexpr int owners(int slots) { return slots >= 8 ? kResMaxThreads / 2 : kResMaxThreads; }
 
 __host__ __device__ inline size_t up16(size_t v) { return (v + 15) & ~(size_t)15; }
 
@@ -152,6 +160,22 @@ __device__ __forceinline__ void tile_copy(uint32_t dst, const void* src, uint32_
       "r"(bytes), "r"(b)
       : "memory");
 }
+// bytes from this CTA's shared memory into that of CTA `rank` of the cluster at the same place, counted
+// on its barrier
+__device__ __forceinline__ void tile_push(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t b, uint32_t rank) {
+  asm volatile(
+      "{\n .reg .b32 d, m;\n mapa.shared::cluster.u32 d, %0, %4;\n mapa.shared::cluster.u32 m, %3, %4;\n"
+      " cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [d], [%1], %2, [m];\n}\n" ::"r"(dst),
+      "r"(src), "r"(bytes), "r"(b), "r"(rank)
+      : "memory");
+}
+__device__ __forceinline__ void push_sources_read() {  // this thread's pushes have read their source
+  asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group.read 0;\n" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive;\nbarrier.cluster.wait;\n" ::: "memory");
+}
+__device__ __forceinline__ void proxy_fence_shared() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
 __device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async;\n" ::: "memory"); }
 
 template <typename C2, int H>
@@ -281,7 +305,12 @@ __device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 0;\n" ::: "m
 // partials, and the tile copies.
 // The body runs as one tile (number `cta` of G tiles or CTAs) of the state that P describes; inst: the
 // batch member, whose results go to its record (null: to P.slots).
-template <typename R, int S, bool REG, bool PEC, bool COMP>
+//
+// CLU: the CTAs are one thread-block cluster (at most 16, one slot per thread).  A finished tile goes
+// straight into the partners' shared memory (cp.async.bulk between CTAs, completion on the
+// partner's mbarrier), into one of two sets of buffers by the evaluation's parity: having a
+// partner's data of one evaluation says that it is past the reads of the set written next.
+template <typename R, int S, bool REG, bool PEC, bool COMP, bool CLU>
 __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t cta, const uint32_t G,
                                               BatchInst* const inst) {
   using C2 = typename RT<R>::C2;
@@ -351,6 +380,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
   }
   for (int k = tid; k < ng; k += blockDim.x) s_gen[k].off = s_gen[ng + k].off = place(tab->flips[P.rt->idx[np + k]].x);
   __syncthreads();
+  if (CLU) cluster_sync();  // every CTA's barriers are ready for the others' copies
 
   // copies of partner tiles (and of owned quarter tiles) for one visit of a tile; q0: ring entries
   // so far, visit: tile visits so far
@@ -427,11 +457,27 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
     const double e24 = P.h / 24.0;
     const R h24 = (R)e24, h24lo = sizeof(R) == 8 ? (R)0 : (R)(e24 - (double)h24);
     const R c9 = (R)9 * h24, c19 = (R)19 * h24, c5 = (R)5 * h24;
-    const R p55 = (R)55 * h24, p59 = (R)59 * h24, p37 = (R)37 * h24, p9 = (R)9 * h24;
+    const R c64 = (R)64 * h24, p55 = (R)55 * h24, p59 = (R)59 * h24, p37 = (R)37 * h24, p9 = (R)9 * h24;
     const bool others = nz > 0 || ncls > (tcls >= 0 ? 1 : 0);
     // y, f of the last three steps, Runge-Kutta accumulator and low part of y of one slot
     struct Owned {
       C2 y[H], a[H], b[H], c[H], rk[H], yl[H];
+    };
+    // The past's part of the corrector (cq) and of the predictor (pq): in FP64 with y in both, so that
+    // one multiply-add with f_{n+1} completes either (9 and 9 + 55 = 64 times h/24); in FP32 the
+    // weighted sums of derivatives, before the scaling by h/24.
+    auto past = [&](const Owned& w, int q, int kind, C2& cq, C2& pq) {
+      const C2 &y = w.y[q], &a = w.a[q], &b = w.b[q], &c = w.c[q];
+      if (sizeof(R) == 8) {
+        cq = kind == 0 ? C2{fma_(c19, a.x, fma_(-c5, b.x, fma_(h24, c.x, y.x))),
+                            fma_(c19, a.y, fma_(-c5, b.y, fma_(h24, c.y, y.y)))}
+                       : y;  // (the start of the history corrects nothing)
+        pq = C2{fma_(-p59, a.x, fma_(p37, b.x, fma_(-p9, c.x, cq.x))),
+                fma_(-p59, a.y, fma_(p37, b.y, fma_(-p9, c.y, cq.y)))};
+      } else {
+        cq = C2{fma_((R)19, a.x, fma_((R)-5, b.x, c.x)), fma_((R)19, a.y, fma_((R)-5, b.y, c.y))};
+        pq = C2{fma_((R)-59, a.x, fma_((R)37, b.x, (R)-9 * c.x)), fma_((R)-59, a.y, fma_((R)37, b.y, (R)-9 * c.y))};
+      }
     };
     auto load = [&](const C2* v, C2 (&d)[H]) { unpack<C2, H>(*reinterpret_cast<const float4*>(v), d); };
     auto store = [&](C2* v, const C2 (&d)[H]) { *reinterpret_cast<float4*>(v) = pack<C2, H>(d); };
@@ -476,83 +522,80 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
         R ar[A], ai[A];
 #pragma unroll
         for (int g = 0; g < A; g++) ar[g] = ai[g] = (R)0;
-        // X strings with real coefficients [k, end) out of the tiles from `t` on; the two complex64
-        // amplitudes of a slot are read one by one, so a flip of index bit 0 needs no swap
+        // X strings with real coefficients [k, end) out of the tiles from `t` on, one 16-byte load per
+        // slot (two 8-byte loads, which need no swap for a flip of index bit 0, hit each bank twice)
         auto plain = [&](const unsigned char* t, int k, int end) {
           constexpr int U = S >= 4 ? 1 : 4 / S;  // products in flight
-          if constexpr (S >= 4) {  // many slots: one 16-byte load each, the swap chosen per product
+          auto some = [&](auto count, int k) {
+            constexpr int C = decltype(count)::value;
+            RPlain<R> f[C];
+            float4 v[C][S];
+#pragma unroll
+            for (int i = 0; i < C; i++) {
+              f[i] = pl[k + i];
+              const uint32_t at = jb ^ (f[i].off & ~15u);
+#pragma unroll
+              for (int s = 0; s < S; s++) v[i][s] = *reinterpret_cast<const float4*>(t + (at ^ ((uint32_t)s * jsb)));
+            }
+#pragma unroll
+            for (int i = 0; i < C; i++) {
+              const bool sw = H == 2 && (f[i].off & 15u);
+#pragma unroll
+              for (int s = 0; s < S; s++) {
+                C2 u[H];
+                unpack<C2, H>(v[i][s], u);
+#pragma unroll
+                for (int q = 0; q < H; q++) {
+                  const C2 x = sw ? u[H - 1 - q] : u[q];
+                  ar[s * H + q] = fma_(f[i].c, x.x, ar[s * H + q]);
+                  ai[s * H + q] = fma_(f[i].c, x.y, ai[s * H + q]);
+                }
+              }
+            }
+          };
+          if constexpr (S >= 4) {  // one product at a time, up to eight slots' loads at once
 #pragma unroll 1
             for (; k < end; k++) {
               const RPlain<R> f = pl[k];
               const uint32_t at = jb ^ (f.off & ~15u);
-              float4 v[S];
-#pragma unroll
-              for (int s = 0; s < S; s++) v[s] = *reinterpret_cast<const float4*>(t + (at ^ ((uint32_t)s * jsb)));
               const bool sw = H == 2 && (f.off & 15u);
+              constexpr int L = S < 8 ? S : 8;  // loads in flight
 #pragma unroll
-              for (int s = 0; s < S; s++) {
-                C2 u[H];
-                unpack<C2, H>(v[s], u);
+              for (int s0 = 0; s0 < S; s0 += L) {
+                float4 v[L];
 #pragma unroll
-                for (int q = 0; q < H; q++) {
-                  const C2 x = sw ? u[H - 1 - q] : u[q];
-                  ar[s * H + q] = fma_(f.c, x.x, ar[s * H + q]);
-                  ai[s * H + q] = fma_(f.c, x.y, ai[s * H + q]);
+                for (int i = 0; i < L; i++) v[i] = *reinterpret_cast<const float4*>(t + (at ^ ((uint32_t)(s0 + i) * jsb)));
+#pragma unroll
+                for (int i = 0; i < L; i++) {
+                  C2 u[H];
+                  unpack<C2, H>(v[i], u);
+#pragma unroll
+                  for (int q = 0; q < H; q++) {
+                    const int g = (s0 + i) * H + q;
+                    const C2 x = sw ? u[H - 1 - q] : u[q];
+                    ar[g] = fma_(f.c, x.x, ar[g]);
+                    ai[g] = fma_(f.c, x.y, ai[g]);
+                  }
                 }
               }
             }
             return;
           }
-          auto one = [&](const RPlain<R>& f, int s, const C2 (&u)[H]) {
-#pragma unroll
-            for (int q = 0; q < H; q++) {
-              ar[s * H + q] = fma_(f.c, u[q].x, ar[s * H + q]);
-              ai[s * H + q] = fma_(f.c, u[q].y, ai[s * H + q]);
-            }
-          };
-          auto get = [&](uint32_t off, int s, C2 (&u)[H]) {
-            const uint32_t at = (jb ^ off) ^ ((uint32_t)s * jsb);
-#pragma unroll
-            for (int q = 0; q < H; q++) u[q] = *reinterpret_cast<const C2*>(t + (at ^ (uint32_t)(q * sizeof(C2))));
-          };
-          for (; k + U <= end; k += U) {
-            RPlain<R> f[U];
-            C2 u[U][S][H];
-#pragma unroll
-            for (int i = 0; i < U; i++) {
-              f[i] = pl[k + i];
-#pragma unroll
-              for (int s = 0; s < S; s++) get(f[i].off, s, u[i][s]);
-            }
-#pragma unroll
-            for (int i = 0; i < U; i++)
-#pragma unroll
-              for (int s = 0; s < S; s++) one(f[i], s, u[i][s]);
+#pragma unroll 1
+          for (; k + U <= end; k += U) some(std::integral_constant<int, U>{}, k);
+          if (U > 2 && k + 2 <= end) {
+            some(std::integral_constant<int, 2>{}, k);
+            k += 2;
           }
-          if (U > 1)
-            for (; k < end; k++) {
-              const RPlain<R> f = pl[k];
-#pragma unroll
-              for (int s = 0; s < S; s++) {
-                C2 u[H];
-                get(f.off, s, u);
-                one(f, s, u);
-              }
-            }
+          if (U > 1 && k < end) some(std::integral_constant<int, 1>{}, k);
         };
         // one slot's partner amplitudes at place `off`
         auto partner = [&](const unsigned char* t, uint32_t off, int s, bool sw, C2 (&u)[H]) {
-          if constexpr (S >= 4) {
-            const uint32_t at = (jb ^ (off & ~15u)) ^ ((uint32_t)s * jsb);
-            C2 v[H];
-            unpack<C2, H>(*reinterpret_cast<const float4*>(t + at), v);
+          const uint32_t at = (jb ^ (off & ~15u)) ^ ((uint32_t)s * jsb);
+          C2 v[H];
+          unpack<C2, H>(*reinterpret_cast<const float4*>(t + at), v);
 #pragma unroll
-            for (int q = 0; q < H; q++) u[q] = sw ? v[H - 1 - q] : v[q];
-          } else {
-            const uint32_t at = (jb ^ off) ^ ((uint32_t)s * jsb);
-#pragma unroll
-            for (int q = 0; q < H; q++) u[q] = *reinterpret_cast<const C2*>(t + (at ^ (uint32_t)(q * sizeof(C2))));
-          }
+          for (int q = 0; q < H; q++) u[q] = sw ? v[H - 1 - q] : v[q];
         };
         // hops [k, end): 2c (= cr - cr2) where the two bits of z differ, else 0.  The thread's
         // amplitudes differ in bit 0 and in the slot bits only, so one parity per hop is computed
@@ -626,9 +669,28 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
           }
         };
         if (act) runs_to(smem, s_part[0].run_end);
+        // what does not need the partners, while their tiles are on their way (owned vectors in
+        // registers): the diagonal and the past's part of the corrector and the predictor
+        auto diagonal = [&](uint32_t j, int q) {
+          const int code = tcls >= 0 ? s_code[j + q] : 0;
+          R d = sc.dt[code];
+          if (others) d += other_diagonal<R>(tab, sc, s_z + par * nz, tcls, code, zb + j + q);
+          return d;
+        };
+        C2 cb[REG ? A : 1], pb[REG ? A : 1];
+        R dg[REG ? A : 1];
+        if (REG && act)
+#pragma unroll
+          for (int g = 0; g < A; g++) {
+            dg[REG ? g : 0] = diagonal((uint32_t)(j0 + (g / H) * js), g % H);
+            if (kind == 0 || kind == 5) past(o[REG ? g / H : 0], g % H, kind, cb[REG ? g : 0], pb[REG ? g : 0]);
+          }
         if (nd > 0 && !ring) {  // every partner in one go: the places name the buffers
-          arrived(0, visit & 1u);
-          if (act) runs_to(smem, P.nruns);
+          if (CLU)
+            arrived((uint32_t)par, (uint32_t)(e >> 1) & 1u);
+          else
+            arrived(0, visit & 1u);
+          if (act) runs_to(smem + (CLU && par ? (size_t)nd * tbytes : 0), P.nruns);
         }
         uint32_t rb = ring ? q0 % (uint32_t)nbuf : 0u, ru = ring ? q0 / (uint32_t)nbuf : 0u;
         auto release = [&]() {  // this warp is done with buffer rb; on to the next ring entry
@@ -647,7 +709,8 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
           }
         }
         // every owner is past the products that read the own tile: it can be overwritten
-        asm volatile("bar.sync 1, %0;\n" ::"r"(nth) : "memory");
+        // (in a cluster also by the copies that push it)
+        asm volatile("bar.sync 1, %0;\n" ::"r"(CLU ? nth + 32 : nth) : "memory");
         R t0 = (R)0, t1 = (R)0;
         auto fetch_owned = [&](int s, Owned& w) {  // of one slot, from global memory
           const uint32_t z = zb + (uint32_t)(j0 + s * js);
@@ -687,23 +750,27 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
 #pragma unroll
           for (int q = 0; q < H; q++) {
             R re = ar[s * H + q], im = ai[s * H + q];
-            const int code = tcls >= 0 ? s_code[j + q] : 0;
-            R d = sc.dt[code];
-            if (others) d += other_diagonal<R>(tab, sc, s_z + par * nz, tcls, code, z0 + q);
-            if (d != (R)0) {  // also keeps an infinite amplitude from turning an H without diagonal into NaN
+            const R d = REG ? dg[REG ? s * H + q : 0] : diagonal(j, q);
+            if (d != (R)0) {  // an infinite amplitude must not make NaN of an H without diagonal
               re = fma_(d, own[q].x, re);
               im = fma_(d, own[q].y, im);
             }
             const C2 fn = C2{im, -re};  // -i (re + i im)
             C2 &y = w.y[q], &a = w.a[q], &b = w.b[q], &c = w.c[q], &rk = w.rk[q];
             if (kind == 0 || kind == 5) {
+              C2 cq, pq;
+              if (REG) {
+                cq = cb[REG ? s * H + q : 0];
+                pq = pb[REG ? s * H + q : 0];
+              } else {
+                past(w, q, kind, cq, pq);
+              }
               if (kind == 0) {  // corrector (Adams-Moulton)
                 if (sizeof(R) == 8) {
-                  y.x = fma_(c9, fn.x, fma_(c19, a.x, fma_(-c5, b.x, fma_(h24, c.x, y.x))));
-                  y.y = fma_(c9, fn.y, fma_(c19, a.y, fma_(-c5, b.y, fma_(h24, c.y, y.y))));
+                  y.x = fma_(c9, fn.x, cq.x);
+                  y.y = fma_(c9, fn.y, cq.y);
                 } else {  // h/24 as hi + lo: a step size rounded to FP32 would drift over the run
-                  const R sx = fma_((R)9, fn.x, fma_((R)19, a.x, fma_((R)-5, b.x, c.x)));
-                  const R sy = fma_((R)9, fn.y, fma_((R)19, a.y, fma_((R)-5, b.y, c.y)));
+                  const R sx = fma_((R)9, fn.x, cq.x), sy = fma_((R)9, fn.y, cq.y);
                   const R ix = fma_(h24, sx, h24lo * sx), iy = fma_(h24, sy, h24lo * sy);
                   if (kComp) {
                     y.x = add_compensated(y.x, w.yl[q].x, ix);
@@ -718,11 +785,10 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
                 if (last) t0 = fma_(y.x, y.x, fma_(y.y, y.y, t0));
               }
               if (sizeof(R) == 8) {  // predictor (Adams-Bashforth)
-                nx[q] = C2{fma_(p55, fn.x, fma_(-p59, a.x, fma_(p37, b.x, fma_(-p9, c.x, y.x)))),
-                           fma_(p55, fn.y, fma_(-p59, a.y, fma_(p37, b.y, fma_(-p9, c.y, y.y))))};
+                const R cf = kind == 0 ? c64 : p55;
+                nx[q] = C2{fma_(cf, fn.x, pq.x), fma_(cf, fn.y, pq.y)};
               } else {
-                const R px = fma_((R)55, fn.x, fma_((R)-59, a.x, fma_((R)37, b.x, (R)-9 * c.x)));
-                const R py = fma_((R)55, fn.y, fma_((R)-59, a.y, fma_((R)37, b.y, (R)-9 * c.y)));
+                const R px = fma_((R)55, fn.x, pq.x), py = fma_((R)55, fn.y, pq.y);
                 nx[q] = C2{y.x + fma_(h24, px, h24lo * px), y.y + fma_(h24, py, h24lo * py)};
               }
               c = b;
@@ -753,7 +819,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
               nx[q] = own[q];
             }
           }
-          if (kind != 7) store(xout + z0, nx);
+          if (kind != 7 && (!CLU || last)) store(xout + z0, nx);  // partners of a cluster get it from the tile
           if (!last && !multi) store(xs + j, nx);
           if (!REG) {
             if (kind == 0 || kind == 5 || kind == 1) store(F(latest + 1) + z0, w.a);
@@ -762,7 +828,12 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
             if (kComp && kind == 0) store(YL + z0, w.yl);
           }
         }
-        if (!last && nq > 0) proxy_fence();  // this thread's stores, before asynchronous copies read them
+        // this thread's stores, before asynchronous copies read them (a cluster's copies read the tile
+        // in shared memory; the wider fence waits for the global stores, 800 cycles)
+        if (CLU)
+          proxy_fence_shared();
+        else if (!last && nq > 0)
+          proxy_fence();
         red0 += (RED)t0;
         red1 += (RED)t1;
         q0 += (uint32_t)nq;
@@ -822,7 +893,21 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
           if (multi) cta_sync();
           cta_sync();
         }
-        if (svc == 3 && nq > 0) copy_in(tile, xin, e, latest, q0);
+        if (CLU && svc == 3) {
+          if (e == 0) {
+            copy_in(tile, xin, e, latest, q0);
+          } else {  // the own tile to the partners
+            if (lane == 0) expect(full0 + 8u * (e & 1), (uint32_t)nd * tbytes);
+            for (int p = lane; p < nd; p += 32)
+              tile_push(saddr(xs + (size_t)(1 + p + ((e & 1) ? nd : 0)) * tsize), saddr(xs), tbytes, full0 + 8u * (e & 1),
+                        cta ^ s_part[p + 1].hi);
+            push_sources_read();
+            __syncwarp();
+          }
+          asm volatile("bar.sync 1, %0;\n" ::"r"(nth + 32) : "memory");
+        } else if (svc == 3 && nq > 0) {
+          copy_in(tile, xin, e, latest, q0);
+        }
         q0 += (uint32_t)nq;
         if (tile == cta) {
           if (!last) prepare(e + 1);
@@ -838,7 +923,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
       if (last) break;
       cta_sync();
       if (s_abort) break;
-      if (!multi && svc == 3 && lane == 0 && nd > 0) flag_release(P.flags + kResFlagStride * cta, (unsigned)(e + 1));
+      if (!CLU && !multi && svc == 3 && lane == 0 && nd > 0) flag_release(P.flags + kResFlagStride * cta, (unsigned)(e + 1));
       xin = e & 1 ? XO : XA;
     }
     if (s_abort && svc == 3) {  // copies in flight land before the CTA leaves (bounded)
@@ -855,6 +940,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
     }
   }
   const bool reduced = P.n_pec > 0 || P.single == 7;
+  if (CLU) cluster_sync();  // no CTA leaves while others may still write into its shared memory
   if (P.single == 6) return;
   __syncthreads();
   if (reduced) {
@@ -911,8 +997,13 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
 }
 
 template <typename R, int S, bool REG, bool PEC, bool COMP>
-__global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const __grid_constant__ ResParams P) {
-  resident_body<R, S, REG, PEC, COMP>(P, blockIdx.x, gridDim.x, nullptr);
+__global__ void __launch_bounds__(owners(S) + kService, 1) k_resident(const __grid_constant__ ResParams P) {
+  resident_body<R, S, REG, PEC, COMP, false>(P, blockIdx.x, gridDim.x, nullptr);
+}
+
+template <typename R, bool PEC, bool COMP>
+__global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident_cluster(const __grid_constant__ ResParams P) {
+  resident_body<R, 1, true, PEC, COMP, true>(P, blockIdx.x, gridDim.x, nullptr);
 }
 
 // Predictor-corrector steps of many states in one launch: a CTA is one tile of one batch member,
@@ -921,7 +1012,7 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident(const
 // of 2^13) takes 53 us in three waves on tiles of 2^12; one launch per layout level over all tiles
 // took 93 us.
 template <typename R, int S>
-__global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident_batch(const __grid_constant__ ResBatch B) {
+__global__ void __launch_bounds__(owners(S) + kService, 1) k_resident_batch(const __grid_constant__ ResBatch B) {
   __shared__ ResParams P;
   int m = 0;
   while (m + 1 < B.count && B.first[m + 1] <= blockIdx.x) m++;
@@ -967,7 +1058,7 @@ __global__ void __launch_bounds__(kResMaxThreads + kService, 1) k_resident_batch
     P.w[k] = ((c[3] * s + c[2]) * s + c[1]) * s + c[0];
   }
   __syncthreads();
-  resident_body<R, S, (S <= 2), true, false>(P, blockIdx.x - B.first[m], 1u << (P.n - P.t), I);
+  resident_body<R, S, (S <= 2), true, false, false>(P, blockIdx.x - B.first[m], 1u << (P.n - P.t), I);
 }
 
 template <typename R, int S, bool REG, bool PEC, bool COMP>
@@ -1003,14 +1094,55 @@ cudaError_t launch_c(const ResParams& p, int nth, int max_grid, int n_z, cudaStr
                : launch_t<R, S, REG, true, false>(p, nth, max_grid, n_z, s);
 }
 
+// One cluster of 2^(n - t) CTAs.  p.nbuf: two sets of partner buffers.
+template <typename R, bool PEC, bool COMP>
+cudaError_t launch_cluster_t(const ResParams& p, int nth, int n_z, cudaStream_t s) {
+  const size_t smem = ResSmem<R>(1u << p.t, p.nbuf, p.np, p.ng, n_z, nth, false).total;
+  auto kern = k_resident_cluster<R, PEC, COMP>;
+  static int configured = 0;
+  if ((int)smem > configured) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    configured = (int)smem;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1u << (p.n - p.t);
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(1u << (p.n - p.t));
+  cfg.blockDim = dim3(nth + kService);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  static int known[3] = {-1, -1, -1}, fits = 0;  // whether the device holds such a cluster
+  const int shape[3] = {(int)cfg.gridDim.x, nth, (int)smem};
+  if (shape[0] != known[0] || shape[1] != known[1] || shape[2] != known[2]) {
+    cudaError_t q = cudaOccupancyMaxActiveClusters(&fits, kern, &cfg);
+    if (q != cudaSuccess) return q;
+    for (int i = 0; i < 3; i++) known[i] = shape[i];
+  }
+  if (fits < 1) return cudaErrorNotSupported;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, p);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t launch_cluster_r(const ResParams& p, int nth, int n_z, cudaStream_t s) {
+  if (p.n_pec == 0) return launch_cluster_t<R, false, false>(p, nth, n_z, s);
+  return p.ylo ? launch_cluster_t<R, true, sizeof(R) == 4>(p, nth, n_z, s) : launch_cluster_t<R, true, false>(p, nth, n_z, s);
+}
+
 template <typename R>
 cudaError_t launch_r(const ResParams& p, int slots, int nth, int max_grid, int n_z, cudaStream_t s) {
   const bool reg = (1 << (p.n - p.t)) <= max_grid;
   switch (slots) {
     case 1: return reg ? launch_c<R, 1, true>(p, nth, max_grid, n_z, s) : launch_c<R, 1, false>(p, nth, max_grid, n_z, s);
     case 2: return reg ? launch_c<R, 2, true>(p, nth, max_grid, n_z, s) : launch_c<R, 2, false>(p, nth, max_grid, n_z, s);
-    case 4: return launch_c<R, 4, false>(p, nth, max_grid, n_z, s);
     case 8: return launch_c<R, 8, false>(p, nth, max_grid, n_z, s);
+    case 16: return launch_c<R, 16, false>(p, nth, max_grid, n_z, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -1037,7 +1169,7 @@ static cudaError_t launch_batch_s(const ResBatch& b, int ctas, size_t smem, cuda
   attr[0].id = cudaLaunchAttributeCooperative;
   attr[0].val.cooperative = 1;
   cfg.gridDim = dim3(ctas);
-  cfg.blockDim = dim3(kResMaxThreads + kService);
+  cfg.blockDim = dim3(owners(S) + kService);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = attr;
@@ -1051,8 +1183,8 @@ static cudaError_t launch_batch_r(const ResBatch& b, int slots, int ctas, size_t
   switch (slots) {
     case 1: return launch_batch_s<R, 1>(b, ctas, smem, s);
     case 2: return launch_batch_s<R, 2>(b, ctas, smem, s);
-    case 4: return launch_batch_s<R, 4>(b, ctas, smem, s);
     case 8: return launch_batch_s<R, 8>(b, ctas, smem, s);
+    case 16: return launch_batch_s<R, 16>(b, ctas, smem, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -1063,6 +1195,10 @@ cudaError_t launch_resident_batch(int prec, const ResBatch& b, int slots, int ct
 
 cudaError_t launch_resident(int prec, const ResParams& p, int slots, int nth, int max_grid, int n_z, cudaStream_t s) {
   return prec == 0 ? launch_r<double>(p, slots, nth, max_grid, n_z, s) : launch_r<float>(p, slots, nth, max_grid, n_z, s);
+}
+
+cudaError_t launch_resident_cluster(int prec, const ResParams& p, int nth, int n_z, cudaStream_t s) {
+  return prec == 0 ? launch_cluster_r<double>(p, nth, n_z, s) : launch_cluster_r<float>(p, nth, n_z, s);
 }
 
 }  // namespace aqc

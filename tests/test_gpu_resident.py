@@ -43,7 +43,7 @@ def _random(n, prec, seed, T=0.6, steps=90):
 
 
 @pytest.mark.parametrize("prec", [C128, C64])
-@pytest.mark.parametrize("n", [1, 2, 3, 5, 7, 8, 9, 10, 11, 15, 17, 18, 19, 20])
+@pytest.mark.parametrize("n", [1, 2, 3, 5, 7, 8, 9, 10, 11, 13, 14, 15, 17, 18, 19, 20])
 def test_solve_matvec_and_energy_against_the_oracle(n, prec):
     steps = 90 if n < 15 else 12
     ctx, H, sched = _random(n, prec, 40 + n, steps=steps)
@@ -66,10 +66,11 @@ def test_solve_matvec_and_energy_against_the_oracle(n, prec):
 
 
 @pytest.mark.parametrize("prec", [C128, C64])
-@pytest.mark.parametrize("n", [9, 13, 17, 19])
+@pytest.mark.parametrize("n", [9, 11, 13, 14, 17, 19])
 def test_fewer_ctas_and_single_steps_keep_the_bits(n, prec):
-    """A limit on the CTAs (several tiles per CTA, owned vectors in memory), one step per launch,
-    and calls that end anywhere give the same state and error estimate."""
+    """A limit on the CTAs (several tiles per CTA, owned vectors in memory, no cluster), one step per
+    launch, and calls that end anywhere give the same state and norm: cluster and memory exchange,
+    owned vectors in registers and in memory."""
     ref = None
     for limit, k, calls in ((0, -1, (-1,)), (1, -1, (-1,)), (5, 0, (-1,)), (0, 0, (1, 1, 2, 1, 30, -1)),
                             (0, 8, (2, 3, 17, -1))):
