@@ -99,7 +99,7 @@ def peaks():
 
 def kernel_hash():
     h = hashlib.sha256()
-    for f in ("kernels.cu", "xpartial.cu", "api.cu", "aqc_internal.h"):
+    for f in ("kernels.cu", "xpartial.cu", "resident.cu", "api.cu", "aqc_internal.h"):
         h.update(open(os.path.join(ROOT, "paper_1311_3938_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -848,7 +848,7 @@ def run_ours(a):
             "bound": "hbm",
             "kernel": ("fused PEC step, per grid step: k_apply partial pass(es) + k_slab (last partial layout "
                        "and step over L2-sized slabs)" if a.slab_bits != 0 else
-                       "fused PEC step, per grid step: k_partial_x (TMA) partial passes + k_apply MODE_STEP"),
+                       "fused PEC step, per grid step: k_tile_x (TMA-fed) partial passes and step"),
             "achieved": r64["pec_step_gbs"],
             "peak": hbm_peak,
             "peak_kind": peak_kind,

@@ -1329,6 +1329,7 @@ int pec_step(aqc_ctx* c) {
   // under step-size control y_{n+1} goes to the scratch vector, so a rejected step keeps y_n
   fin.yout = c->adaptive ? c->vec[V_ACC] : nullptr;
   fin.ylo = c->ycomp ? c->vec_save : nullptr;
+  fin.want_norm = c->adaptive;
   int rc;
   if (turn_applies(c))
     rc = pec_step_turn(c, fin, w);

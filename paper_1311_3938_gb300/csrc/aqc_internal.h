@@ -136,6 +136,7 @@ struct ApplyParams {
   int with_remote;
   int mode;
   int stage;         // RK4 stage 1..4
+  int want_norm;     // STEP: also reduce ||y_{n+1}||^2 (step-size control reads it)
   double w[3];       // group weights A, B, C at the evaluation time
   const double* wdev; // nullable: read the weights from this device array instead of w (steps
                       // replayed from a CUDA graph, whose weights the host writes before a replay)

@@ -81,16 +81,43 @@ __device__ __forceinline__ int64_t to_fixed(double v, int emax, int up) {
     r = sh < -62 ? 0 : (m + (1ll << (-sh - 1))) >> -sh;
   return b < 0 ? -r : r;
 }
-// nearest double of an integer (ties upward), in integer instructions
-__device__ __forceinline__ double from_fixed(int64_t s) {
+// nearest double of s 2^k (ties upward; s 2^k normal or zero), in integer instructions
+__device__ __forceinline__ double from_fixed(int64_t s, int k = 0) {
   const uint64_t a = s < 0 ? (uint64_t)-s : (uint64_t)s;
   if (a == 0) return 0.0;
   const int lz = __clzll((long long)a);
   const uint64_t t = a << lz;                          // leading bit at 63
   const uint64_t m = (t >> 11) + ((t >> 10) & 1u);     // 53 bits; a carry moves into the exponent
-  const uint64_t b = ((uint64_t)(1022 + 63 - lz) << 52) + m;
+  const uint64_t b = ((uint64_t)(1022 + 63 - lz + k) << 52) + m;
   return __longlong_as_double((long long)(b | (s < 0 ? 0x8000000000000000ull : 0ull)));
 }
+
+// One component of the corrector and the predictor (Sec. I.B): y += h24 (9 f + 19 a - 5 b + c), then
+// p = y + h24 (55 f - 59 a + 37 b - 9 c).  The weighted sums of the four derivatives are taken exactly
+// in integers scaled by the largest of them (55 bits and a sign each; 160 times that is below 2^63)
+// and rounded once, so two FP64 operations are left of eight, and the error is that of the last
+// multiply-add instead of four roundings next to y (rms of y's rounding 4.6e-17, 8.8e-17 with the chain
+// of multiply-adds).  With the integer clause counts and without the norm that nobody reads: 64 grid
+// steps at n = 20 8.2 -> 6.8 ms, 12 at n = 26 114 -> 102 ms; the step kernel at n = 26 takes 3.25 ms, of
+// which the FP64 pipe needs 1.6 and memory 1.4: issue slots bind it now.
+__device__ __forceinline__ void pec_fixed(double f, double a, double b, double c, double h24, double& y, double& p) {
+  auto top = [](double v) { return (uint32_t)__double2hiint(v) & 0x7fffffffu; };
+  const int emax = (int)(max(max(top(f), top(a)), max(top(b), top(c))) >> 20);
+  if (emax < 2032 && emax >= 256) {
+    const int64_t qf = to_fixed(f, emax, 2), qa = to_fixed(a, emax, 2), qb = to_fixed(b, emax, 2),
+                  qc = to_fixed(c, emax, 2);
+    const int k = emax - 1077;  // a derivative is its integer times 2^k
+    y = fma(h24, from_fixed(9 * qf + 19 * qa - 5 * qb + qc, k), y);
+    p = fma(h24, from_fixed(55 * qf - 59 * qa + 37 * qb - 9 * qc, k), y);
+  } else {  // infinities, NaN, derivatives beyond 2^1008, below 2^-767 or all zero
+    y += h24 * (9.0 * f + 19.0 * a - 5.0 * b + c);
+    p = y + h24 * (55.0 * f - 59.0 * a + 37.0 * b - 9.0 * c);
+  }
+}
+__device__ __forceinline__ void pec_fixed(float, float, float, float, float, float&, float&) {}
+// exact double of a clause count (0..255) in integer instructions (a conversion runs at the FP64 rate)
+__device__ __forceinline__ double count_value(uint32_t c, double) { return from_fixed((int64_t)c); }
+__device__ __forceinline__ float count_value(uint32_t c, float) { return (float)c; }
 
 template <typename R>
 struct SZ {
@@ -265,6 +292,7 @@ struct TileCtx {
   Layout L;
   uint32_t tsize, tmask;
   int np, npf, nh, ngl, ng, nz, ncls, tcls, stage;
+  bool want_norm;  // STEP: ||y||^2 is read after the step (step-size control, batches)
   int nu;     // all np products are equal-coefficient X strings summed as integers (complex128), or 0
   int up;     // their scale: left shift of the tile's largest exponent
   int hc[3];  // ends of hop classes 0..2 (DevTables::hop_class_end)
@@ -924,7 +952,7 @@ __device__ __forceinline__ void process_tile(const TileCtx<R>& T, uint32_t zb, u
     for (int g = 0; g < G; g++) {
       if (with_diag) {
         R d = T.dconst;
-        if (T.tcls >= 0) d += T.wtab * (R)code[g];
+        if (T.tcls >= 0) d += T.wtab * count_value(code[g], (R)0);
         for (int cc = 0; cc < T.ncls; cc++) {
           if (cc == T.tcls) continue;
           const DevClass cl = T.tab->classes[cc];
@@ -956,12 +984,9 @@ __device__ __forceinline__ void process_tile(const TileCtx<R>& T, uint32_t zb, u
     }
     // 5. epilogue
     const R h = T.h;
-    // corrector and predictor weights h/24 * (9, 19, -5, 1) and h/24 * (55, -59, 37, -9); in
-    // FP64 applied as chains of fused multiply-adds (fewer FP64 instructions)
+    // corrector and predictor: h/24 times the sums weighted (9, 19, -5, 1) and (55, -59, 37, -9)
     const R h24 = kFp64 ? h / (R)24 : T.h24;
     const R h24lo = T.h24lo;
-    const R c9 = (R)9 * h24, c19 = (R)19 * h24, c5 = (R)5 * h24;
-    const R p55 = (R)55 * h24, p59 = (R)59 * h24, p37 = (R)37 * h24, p9 = (R)9 * h24;
     C2 o1[G], o2[G], o3[G];
 #pragma unroll
     for (int g = 0; g < G; g++) {
@@ -979,10 +1004,9 @@ __device__ __forceinline__ void process_tile(const TileCtx<R>& T, uint32_t zb, u
         const C2 fn = C2{ai[g], -ar[g]};
         C2 yn, pn;
         if (kFp64) {
-          yn.x = fma(c9, fn.x, fma(c19, a[g].x, fma(-c5, b[g].x, fma(h24, c[g].x, y0[g].x))));
-          yn.y = fma(c9, fn.y, fma(c19, a[g].y, fma(-c5, b[g].y, fma(h24, c[g].y, y0[g].y))));
-          pn.x = fma(p55, fn.x, fma(-p59, a[g].x, fma(p37, b[g].x, fma(-p9, c[g].x, yn.x))));
-          pn.y = fma(p55, fn.y, fma(-p59, a[g].y, fma(p37, b[g].y, fma(-p9, c[g].y, yn.y))));
+          yn = y0[g];
+          pec_fixed(fn.x, a[g].x, b[g].x, c[g].x, h24, yn.x, pn.x);
+          pec_fixed(fn.y, a[g].y, b[g].y, c[g].y, h24, yn.y, pn.y);
         } else {
           // the weighted sums times (hi + lo): h24 * S + h24lo * S with one rounding of the sum
           const R scx = (R)9 * fn.x + (R)19 * a[g].x - (R)5 * b[g].x + c[g].x;
@@ -1007,7 +1031,7 @@ __device__ __forceinline__ void process_tile(const TileCtx<R>& T, uint32_t zb, u
         o3[g] = pn;
         if (ok[g]) {
           const R dx = yn.x - own[g].x, dy = yn.y - own[g].y;
-          rt0 += yn.x * yn.x + yn.y * yn.y;
+          if (T.want_norm) rt0 += yn.x * yn.x + yn.y * yn.y;
           rt1 += dx * dx + dy * dy;
         }
       } else if (MODE == MODE_RK4) {
@@ -1075,6 +1099,7 @@ __global__ void __launch_bounds__(kThreads, (MODE == MODE_PARTIAL && sizeof(R) =
   const double w0 = P.wdev ? P.wdev[0] : P.w[0], w1 = P.wdev ? P.wdev[1] : P.w[1], w2 = P.wdev ? P.wdev[2] : P.w[2];
   load_coefficients<R>(T, P.tab, P.L, P.layout_index, P.with_diag != 0, P.with_remote != 0, P.dcode, w0, w1, w2, smem);
   T.stage = P.stage;
+  T.want_norm = P.want_norm != 0;
   T.h = (R)P.h;
   set_h24(T, P.h);
   T.step_k = P.step_k;
@@ -1101,6 +1126,7 @@ __global__ void __launch_bounds__(kThreads, (MODE == MODE_PARTIAL && sizeof(R) =
                  v2 = P.wdev ? P.wdev[5] : P.w2[2];
     load_coefficients<R>(T2, P.tab, P.L, P.layout_index, false, false, nullptr, v0, v1, v2, smem, smem + mapA.total);
     T2.stage = 0;
+    T2.want_norm = false;
     T2.h = (R)P.h;
     set_h24(T2, P.h);
     T2.step_k = 0;
@@ -1197,6 +1223,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_slab(const SlabParams S) {
   load_coefficients<R>(TP, B.tab, B.L, B.layout_index, B.with_diag != 0, B.with_remote != 0, B.dcode, B.w[0], B.w[1],
                        B.w[2], smem, smem + mapA.total);
   TS.stage = TP.stage = 0;
+  TS.want_norm = A.want_norm != 0;
+  TP.want_norm = false;
   TS.h = TP.h = (R)A.h;
   set_h24(TS, A.h);
   set_h24(TP, A.h);
@@ -1303,6 +1331,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 2 : 1) k_batch(BatchLaunc
   load_coefficients<R>(T, I->tab, I->layouts[level], level, level == diag_level(nl), first, I->dcode,
                        batch_weight(*I, s, 0), batch_weight(*I, s, 1), batch_weight(*I, s, 2), smem);
   T.stage = 0;
+  T.want_norm = true;
   T.h = (R)I->h;
   set_h24(T, I->h);
   T.step_k = 0;  // clause-by-clause sequences are not batched
