@@ -373,7 +373,8 @@ int aqc_batch_set_shape(aqc_batch *b, int threads, int steps_per_round);
  * clause-by-clause sequence, is refused (AQC_E_UNSUPPORTED); a full batch gives AQC_E_NOMEM. */
 int aqc_batch_add(aqc_batch *b, aqc_ctx *ctx, int *slot_out);
 
-/* Remove the member in `slot` and hand its context back. */
+/* Remove the member in `slot` and hand its context back.  AQC_E_TIMEOUT: a bounded wait inside
+ * one of the member's launches gave up; the context is handed back, its state is invalid. */
 int aqc_batch_remove(aqc_batch *b, int slot);
 
 /* Enqueue `rounds` graph replays: every member advances by up to rounds * steps_per_round

@@ -1765,11 +1765,14 @@ int batch_rebuild(aqc_batch* b) {
   if (!rc) rc = batch_plan_waves(b);
   if (rc) return rc;
   std::vector<BatchItem> items[kMaxLayouts];
+  int64_t need[kMaxLayouts] = {0};  // work items by level, those of the resident members too (the batch's size is a contract)
   int smem[kMaxLayouts] = {0};
   int nlev = 0;
   for (int slot = 0; slot < b->max_members; slot++) {
     aqc_ctx* c = b->members[slot];
-    if (!c || b->res[slot]) continue;
+    if (!c) continue;
+    for (size_t l = 0; l < c->layouts.size(); l++) need[l] += (int64_t)1 << (c->n - c->layouts[l].t);
+    if (b->res[slot]) continue;
     BatchInst& I = b->h_insts[slot];
     const int nl = (int)c->layouts.size();
     nlev = std::max(nlev, nl);
@@ -1786,8 +1789,9 @@ int batch_rebuild(aqc_batch* b) {
     }
     I.ticket = 0;
   }
+  for (int l = 0; l < kMaxLayouts; l++)
+    if (need[l] > b->max_items) BFAIL(b, AQC_E_NOMEM, "batch needs %lld work items > max_items", (long long)need[l]);
   for (int l = 0; l < nlev; l++) {
-    if ((int64_t)items[l].size() > b->max_items) BFAIL(b, AQC_E_NOMEM, "batch needs %zu work items > max_items", items[l].size());
     if (!items[l].empty())
       BCUDA(b, cudaMemcpyAsync(b->d_items[l], items[l].data(), items[l].size() * sizeof(BatchItem),
                                cudaMemcpyHostToDevice, b->stream));

@@ -177,3 +177,31 @@ def test_batch_of_resident_and_other_members(prec):
         assert rel_err(c.state(), want) < tol
         c.close()
     b.close()
+
+
+@pytest.mark.parametrize("max_items,fits", [(15, False), (16, True)])
+def test_batch_work_items_bound_resident_members_too(max_items, fits):
+    """A batch counts 2^(n - tile_bits) work items per member (two of n = 16 on 2^13 tiles: 16)."""
+    import paper_1311_3938_gb300 as P
+    from paper_1311_3938_gb300 import hamiltonians as HB
+    from paper_1311_3938_gb300.engine import Batch, Context
+
+    b = Batch(C64, max_members=2, max_items=max_items, steps_per_round=2)
+    ctxs = []
+    for _ in range(2):
+        ctx = Context(16, C64)
+        HB.load_ec3(ctx, generate_ec3(16, 1))
+        ctx.set_schedule(10.0, HB.linear_schedule())
+        ctx.set_integrator(20, 0.0)
+        ctx.set_initial_state("uniform")
+        b.add(ctx)
+        ctxs.append(ctx)
+    if fits:
+        b.run(1)
+        assert b.poll()[1] == 2
+    else:
+        with pytest.raises(P.AqcError, match="max_items"):
+            b.run(1)
+    b.close()
+    for c in ctxs:
+        c.close()
