@@ -136,54 +136,59 @@ __device__ __forceinline__ void smem_flip(float c, const unsigned char* row, flo
   }
 }
 
-// hops: 2c at output amplitudes whose two flipped bits differ, else 0.  The flip's register
-// bits (RB: local bits 6..8, the pair index r) and its pair bit (SW: local bit 0) fix the
-// parity of every amplitude of the thread relative to its first one: pair r's first amplitude
-// differs by parity(r & RB), its second by that ^ SW.  cA is the coefficient at the parity of
-// the thread's first amplitude, cB at the opposite parity, so no per-amplitude parity is left.
-template <int R_, int RB>
-__device__ __forceinline__ constexpr bool pair_parity() {
-  return (((R_ & RB) ^ ((R_ & RB) >> 1) ^ ((R_ & RB) >> 2)) & 1) != 0;
+// products flipping register positions and the pair bit: acc[r] += c * own[r ^ RB], its amplitudes swapped
+template <int RB>
+__device__ __forceinline__ void reg_flip_swap(float c, const float4 (&own)[8], float4 (&acc)[8]) {
+#pragma unroll
+  for (int r = 0; r < 8; r++) fma4(acc[r], c, swap_pair(own[r ^ RB]));
 }
-template <int RB, bool SW, int R_>
-__device__ __forceinline__ void hop_pair(float cA, float cB, const float4& g, float4& a) {
-  constexpr bool p = pair_parity<R_, RB>();
-  const float c0 = p ? cB : cA, c1 = (p != SW) ? cB : cA;
+
+// Hops: 2c at output amplitudes whose two flipped bits differ, else 0.  Where the bits lie fixes the
+// parity of a thread's amplitudes relative to its first one, and the half whose coefficient is zero
+// is not read: with one register bit (RB) a thread needs four of its eight partner pairs, and which
+// four is an offset of its first address; with no register bit all eight or none; with two of the
+// thread's own bits (two register bits, or one and the pair bit) nothing from shared memory.  Only the
+// pair bit beside a lane's or a warp's bit reads both amplitudes of every pair for one of them (8-byte
+// loads at this stride conflict two ways).  XY path, n = 24, 32 steps and start-up: 24.0 -> 23.6 ms; the
+// step pass then keeps shared memory's pipe 27% busy and issue slots 46% (65% while it forms products).
+// cA is the coefficient at the parity of the thread's first amplitude, cB at the opposite one.
+__device__ __forceinline__ void hop_pair(float c0, float c1, const float4& g, float4& a) {
   a.x = fmaf(c0, g.x, a.x);
   a.y = fmaf(c0, g.y, a.y);
   a.z = fmaf(c1, g.z, a.z);
   a.w = fmaf(c1, g.w, a.w);
 }
-template <int RB, bool SW>
-__device__ __forceinline__ void smem_hop(float cA, float cB, const unsigned char* row, float4 (&acc)[8]) {
-  auto one = [&](auto r_tag) {
-    constexpr int r = decltype(r_tag)::value;
-    const float4 g = *reinterpret_cast<const float4*>(row + ((r ^ RB) << 9));
-    hop_pair<RB, SW, r>(cA, cB, SW ? swap_pair(g) : g, acc[r]);
-  };
-  one(std::integral_constant<int, 0>{});
-  one(std::integral_constant<int, 1>{});
-  one(std::integral_constant<int, 2>{});
-  one(std::integral_constant<int, 3>{});
-  one(std::integral_constant<int, 4>{});
-  one(std::integral_constant<int, 5>{});
-  one(std::integral_constant<int, 6>{});
-  one(std::integral_constant<int, 7>{});
+// one register bit; `needed` = the address of the partner rows with a coefficient, r without bit RB
+template <int RB>
+__device__ __forceinline__ void smem_hop_half(float cA, float cB, const unsigned char* needed, float4 (&acc)[8]) {
+#pragma unroll
+  for (int r = 0; r < 8; r++)
+    if ((r & RB) == 0) {
+      const float4 g = *reinterpret_cast<const float4*>(needed + (r << 9));
+      fma4(acc[r], cA, g);
+      fma4(acc[r | RB], cB, g);
+    }
 }
+// the pair bit and a bit outside the thread
+__device__ __forceinline__ void smem_hop_swap(float cA, float cB, const unsigned char* row, float4 (&acc)[8]) {
+#pragma unroll
+  for (int r = 0; r < 8; r++)
+    hop_pair(cA, cB, swap_pair(*reinterpret_cast<const float4*>(row + (r << 9))), acc[r]);
+}
+// two register bits
 template <int RB>
 __device__ __forceinline__ void reg_hop(float cA, float cB, const float4 (&own)[8], float4 (&acc)[8]) {
-  auto one = [&](auto r_tag) {
-    constexpr int r = decltype(r_tag)::value;
-    hop_pair<RB, false, r>(cA, cB, own[r ^ RB], acc[r]);
-  };
-  one(std::integral_constant<int, 0>{});
-  one(std::integral_constant<int, 1>{});
-  one(std::integral_constant<int, 2>{});
-  one(std::integral_constant<int, 3>{});
-  one(std::integral_constant<int, 4>{});
-  one(std::integral_constant<int, 5>{});
-  one(std::integral_constant<int, 6>{});
-  one(std::integral_constant<int, 7>{});
+#pragma unroll
+  for (int r = 0; r < 8; r++) fma4(acc[r], (((r & RB) & ((r & RB) - 1)) == 0 && (r & RB) != 0) ? cB : cA, own[r ^ RB]);
+}
+// one register bit and the pair bit
+template <int RB>
+__device__ __forceinline__ void reg_hop_swap(float cA, float cB, const float4 (&own)[8], float4 (&acc)[8]) {
+#pragma unroll
+  for (int r = 0; r < 8; r++) {
+    const bool p = (r & RB) != 0;
+    hop_pair(p ? cB : cA, p ? cA : cB, swap_pair(own[r ^ RB]), acc[r]);
+  }
 }
 
 __device__ __forceinline__ double weight_of(const XParams& P, int g) {
@@ -326,8 +331,14 @@ __global__ void __launch_bounds__(kXThreads, 1) k_tile_x(const __grid_constant__
       // while the other half's partners are on their way
       auto far_load = [&](const XFlip& f, int r0, float4 (&g)[4]) {
 #pragma unroll
-        for (int r = 0; r < 4; r++)
-          g[r] = __ldcg(reinterpret_cast<const float4*>(src + ((zb + zoff[r0 + r]) ^ (f.lx & ~1u))));
+        for (int r = 0; r < 4; r++) {
+          const uint32_t z = zb + zoff[r0 + r];
+          // a pair with no coefficient in a hop is not read
+          if (f.par == 0u || (f.lx & 1u) || (__popc(z & f.par) & 1u))
+            g[r] = __ldcg(reinterpret_cast<const float4*>(src + (z ^ (f.lx & ~1u))));
+          else
+            g[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
       };
       auto far_add = [&](const XFlip& f, int r0, const float4 (&g)[4]) {
         const bool sw = (f.lx & 1u) != 0u;
@@ -377,34 +388,27 @@ __global__ void __launch_bounds__(kXThreads, 1) k_tile_x(const __grid_constant__
         const float cA = pb ? f.c : 0.f, cB = pb ? 0.f : f.c;
         if (sx == 0u) {
           switch (rb) {
-            case 1: reg_hop<1>(cA, cB, own, acc); break;
-            case 2: reg_hop<2>(cA, cB, own, acc); break;
             case 3: reg_hop<3>(cA, cB, own, acc); break;
-            case 4: reg_hop<4>(cA, cB, own, acc); break;
             case 5: reg_hop<5>(cA, cB, own, acc); break;
-            case 6: reg_hop<6>(cA, cB, own, acc); break;
-            default: reg_hop<7>(cA, cB, own, acc); break;
+            default: reg_hop<6>(cA, cB, own, acc); break;
+          }
+        } else if (sx == 1u) {
+          switch (rb) {
+            case 1: reg_hop_swap<1>(cA, cB, own, acc); break;
+            case 2: reg_hop_swap<2>(cA, cB, own, acc); break;
+            default: reg_hop_swap<4>(cA, cB, own, acc); break;
           }
         } else {
           const unsigned char* row = t + ((jw ^ (sx & ~1u)) << 3);
-          const bool sw = (sx & 1u) != 0u;
-          switch (rb | (sw ? 8u : 0u)) {
-            case 0: smem_hop<0, false>(cA, cB, row, acc); break;
-            case 1: smem_hop<1, false>(cA, cB, row, acc); break;
-            case 2: smem_hop<2, false>(cA, cB, row, acc); break;
-            case 3: smem_hop<3, false>(cA, cB, row, acc); break;
-            case 4: smem_hop<4, false>(cA, cB, row, acc); break;
-            case 5: smem_hop<5, false>(cA, cB, row, acc); break;
-            case 6: smem_hop<6, false>(cA, cB, row, acc); break;
-            case 7: smem_hop<7, false>(cA, cB, row, acc); break;
-            case 8: smem_hop<0, true>(cA, cB, row, acc); break;
-            case 9: smem_hop<1, true>(cA, cB, row, acc); break;
-            case 10: smem_hop<2, true>(cA, cB, row, acc); break;
-            case 11: smem_hop<3, true>(cA, cB, row, acc); break;
-            case 12: smem_hop<4, true>(cA, cB, row, acc); break;
-            case 13: smem_hop<5, true>(cA, cB, row, acc); break;
-            case 14: smem_hop<6, true>(cA, cB, row, acc); break;
-            default: smem_hop<7, true>(cA, cB, row, acc); break;
+          const unsigned char* needed = row + (pb ? rb << 9 : 0u);
+          switch (rb | ((sx & 1u) ? 8u : 0u)) {
+            case 0:
+              if (pb) smem_flip<0, false>(f.c, row, acc);
+              break;
+            case 1: smem_hop_half<1>(cA, cB, needed, acc); break;
+            case 2: smem_hop_half<2>(cA, cB, needed, acc); break;
+            case 4: smem_hop_half<4>(cA, cB, needed, acc); break;
+            default: smem_hop_swap(cA, cB, row, acc); break;
           }
         }
         continue;
@@ -418,6 +422,17 @@ __global__ void __launch_bounds__(kXThreads, 1) k_tile_x(const __grid_constant__
           case 5: reg_flip<5>(f.c, own, acc); break;
           case 6: reg_flip<6>(f.c, own, acc); break;
           default: reg_flip<7>(f.c, own, acc); break;
+        }
+      } else if (sx == 1u) {
+        switch (rb) {
+          case 0: reg_flip_swap<0>(f.c, own, acc); break;
+          case 1: reg_flip_swap<1>(f.c, own, acc); break;
+          case 2: reg_flip_swap<2>(f.c, own, acc); break;
+          case 3: reg_flip_swap<3>(f.c, own, acc); break;
+          case 4: reg_flip_swap<4>(f.c, own, acc); break;
+          case 5: reg_flip_swap<5>(f.c, own, acc); break;
+          case 6: reg_flip_swap<6>(f.c, own, acc); break;
+          default: reg_flip_swap<7>(f.c, own, acc); break;
         }
       } else {
         const unsigned char* row = t + ((jw ^ (sx & ~1u)) << 3);

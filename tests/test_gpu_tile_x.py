@@ -122,3 +122,32 @@ def test_compensated_and_controlled_steps_agree_with_the_plain_ones():
         assert rel_err(ctx.state(), ref.psi) < 1e-6
         assert st["max_err_est"] < 1e-6
         ctx.close()
+
+
+# every pair of bits as a hop (both, one or none of them held by a thread; two layouts; bits that no
+# layout holds) and X strings over the thread's own bits, coefficients all different.  A sum of m <= 270
+# products in FP32 errs by about sqrt(m) * 2^-24 * 0.5 < 5e-7 relative.
+@pytest.mark.parametrize("n,tile_bits,strings", [(13, 13, False), (13, 13, True), (16, 13, False), (23, 0, True)])
+def test_matvec_with_hops_between_all_bits(n, tile_bits, strings):
+    from paper_1311_3938_gb300 import hamiltonians as HB
+    from paper_1311_3938_gb300.engine import Context
+
+    terms = []
+    for i in range(n):
+        for j in range(i):
+            m, c = (1 << i) | (1 << j), 0.1 + 0.01 * i - 0.013 * j
+            if not (strings and j == 0 and i in (6, 7, 8)):
+                terms += [(0, m, 0, c), (0, m, m, c)]
+    for k in range(8):
+        if strings or k not in (1, 2, 4):
+            terms.append((1, (k << 6) | 1, 0, 0.3 - 0.07 * k))
+    ctx, H = Context(n, C64), O.Hamiltonian(n)
+    if tile_bits:
+        ctx.set_tile_bits(tile_bits)
+    load_both(ctx, H, terms, [(1, c, 0, 1.0) for c in generate_ec3(n, 4).clauses])
+    ctx.set_schedule(1.0, HB.linear_schedule())
+    sched = O.linear_path(1.0)
+    psi = random_state(n, 3).astype(np.complex64)
+    want = O.hpsi(H, sched.weights(0.4), psi.astype(np.complex128), nthreads=16)
+    assert rel_err(ctx.hpsi(0.4, torch.from_numpy(psi).cuda()).cpu().numpy(), want) < 1e-6
+    ctx.close()
