@@ -83,7 +83,7 @@ def alg_bytes(n, amp, pec_steps):
 
 
 def pec_flops_c128(n_flip, n_clause_classes=1):
-    """Algorithmic FP64 flops per amplitude of one PEC step: flip products 4 each (complex
+    """FP64 flops per amplitude of one PEC step done in FP64 throughout: flip products 4 each (complex
     amplitude times real coefficient, accumulated), diagonal 4 + 2 per clause class,
     corrector and predictor 16 each, norm and error reductions 10."""
     return 4 * n_flip + 4 + 2 * n_clause_classes + 32 + 10
@@ -121,10 +121,10 @@ def profiled_traffic(prec_name, n=N_QUBITS):
         d = json.load(open(p))
     except Exception:
         return None
-    e = d.get(prec_name)
-    if not e or e.get("kernel_hash") != kernel_hash() or e.get("n", N_QUBITS) != n:
-        return None
-    return e.get("dram_bytes_per_pec_step")
+    for e in (d.get(prec_name), d.get(prec_name + "_tile_x")):  # complex64: the step with y in memory, and without
+        if e and e.get("kernel_hash") == kernel_hash() and e.get("n", N_QUBITS) == n:
+            return e.get("dram_bytes_per_pec_step")
+    return None
 
 
 # ----------------------------------------------------------------------------- clocks
@@ -890,16 +890,26 @@ def run_ours(a):
             "unit": "GB/s",
             "ms_per_step": r128["ms_per_step"],
             "pec_step_ms": r128["pec_step_ms"],
+            # The flip products and the step's weighted sums of an EC3 X-driver state run as exact
+            # integer sums, so the FP64 pipe does a fraction of the plain algorithm's operations and
+            # memory is the larger floor; `fp64` compares with the plain algorithm at the pipe's rate.
             "roofline": {
-                "bound": "alu",
-                "achieved": flops / (r128["pec_step_ms"] * 1e-3) / 1e12,
-                "peak": fp64_peak,
-                "peak_kind": fp64_kind,
-                "unit": "TFLOP/s",
-                "frac": flops / (r128["pec_step_ms"] * 1e-3) / 1e12 / fp64_peak,
-                "hbm_frac": r128["pec_step_gbs"] / hbm_peak,
+                "bound": "hbm",
+                "achieved": r128["pec_step_gbs"],
+                "peak": hbm_peak,
+                "peak_kind": peak_kind,
+                "unit": "GB/s",
+                "frac": r128["pec_step_gbs"] / hbm_peak,
                 "traffic": profiled_traffic("c128", n),
-                "fp64_fma_measurement": fp64,
+                "alg_bytes_per_launch": 7 * (1 << n) * 16,
+                "fp64": {
+                    "plain_flops_per_step": flops,
+                    "plain_tflops_equivalent": flops / (r128["pec_step_ms"] * 1e-3) / 1e12,
+                    "peak": fp64_peak,
+                    "peak_kind": fp64_kind,
+                    "unit": "TFLOP/s",
+                    "measurement": fp64,
+                },
             },
             "e2e": r128.get("e2e"),
             "gpu_launches": r128["launches"],
