@@ -249,7 +249,8 @@ int aqc_set_graph_steps(aqc_ctx *ctx, int k_steps);
  * (3k + 5) N b for k >= 2 layouts.  Applies on the fixed-step grid with per-CTA tiles, outside
  * batches, the slab order and clause-by-clause sequences, and when the products no layout holds
  * can stay in a partial pass (k >= 3, or none of them).  mode: 0 off (the default: on GB300 the
- * turned step measured slower, 4.71 against 4.37 ms at 28 qubits in complex64), 1 or -1 on where
+ * turned step measured slower, 4.71 against 4.37 ms at 28 qubits in complex64, where the plain
+ * one takes 4.13 since), 1 or -1 on where
  * it applies.  Results equal those of the plain pass order up to the order in which the
  * layouts' sums are added.  AQC_E_INVAL for other modes. */
 int aqc_set_layout_turns(aqc_ctx *ctx, int mode);
