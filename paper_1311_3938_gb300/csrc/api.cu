@@ -1052,7 +1052,7 @@ int launch_resident_on(aqc_ctx* c, const ResParams& p) {
   if (tiles > 1 && tiles <= kResMaxCluster && c->res.slots == 1 && p.evals > 1 && p.npart > 0 &&
       c->grid_limit == 0) {
     ResParams q = p;
-    q.nbuf = 2 * p.npart;
+    q.nbuf = 2 * p.npart + 1;  // the partners' tiles twice, the own one once more
     if (resident_smem_bytes(c->prec, p.t, q.nbuf, p.np, p.ng, c->n_z, c->res.nth, true) <= kResSmem) {
       const cudaError_t e = launch_resident_cluster(c->prec, q, c->res.nth, c->n_z, c->stream);
       if (e == cudaSuccess) {

@@ -384,9 +384,11 @@ size_t resident_smem_bytes(int prec, int t, int nbuf, int np, int ng, int n_z, i
 // slots: 16-byte slots per thread and tile; max_grid: CTAs at most (fewer than tiles: a CTA walks
 // several tiles and the owned vectors stay in global memory)
 cudaError_t launch_resident(int prec, const ResParams& p, int slots, int nth, int max_grid, int n_z, cudaStream_t s);
-// the same as one thread-block cluster (at most kResMaxCluster tiles of one slot per thread, a buffer
-// set of p.npart partner tiles for each parity of the evaluation: p.nbuf = 2 p.npart)
+// the same as one thread-block cluster: at most kResMaxCluster tiles of one slot per thread, two sets of
+// tiles in every CTA's shared memory, each its own tile and its p.npart partners' (p.nbuf = 2 p.npart + 1
+// beside the first); evaluation e works on set cluster_set(e)
 constexpr int kResMaxCluster = 16;
+__host__ __device__ constexpr int cluster_set(int e) { return e & 1; }
 cudaError_t launch_resident_cluster(int prec, const ResParams& p, int nth, int n_z, cudaStream_t s);
 cudaError_t launch_resident_batch(int prec, const ResBatch& b, int slots, int ctas, size_t smem, cudaStream_t s);
 int64_t fma64_count(int blocks, int iters);

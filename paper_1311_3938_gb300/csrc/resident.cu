@@ -24,7 +24,11 @@
 // longer than a small state's step.
 //
 // Up to 16 tiles run as one thread-block cluster and push their tiles into one another's shared
-// memory instead: no flags, no trip through L2.
+// memory instead: no flags, no trip through L2.  A push reports its completion at its destination
+// only, so a CTA cannot tell when its own tile has been read; it keeps two (cluster_set): the tile of
+// evaluation e + 1 is written beside that of e and over that of e - 1.  That one is free by then: a
+// partner sends its tile of e only when it has finished e - 1, for which it needed all of this CTA's
+// tile of e - 1, and no thread writes before it has seen every partner's tile of e.
 //
 // Measured, microseconds per predictor-corrector step (before: one launch per layout pass, replayed
 // from a graph, each on as many CTAs as the state has 64 KiB tiles):
@@ -169,9 +173,6 @@ __device__ __forceinline__ void tile_push(uint32_t dst, uint32_t src, uint32_t b
       "r"(src), "r"(bytes), "r"(b), "r"(rank)
       : "memory");
 }
-__device__ __forceinline__ void push_sources_read() {  // this thread's pushes have read their source
-  asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group.read 0;\n" ::: "memory");
-}
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive;\nbarrier.cluster.wait;\n" ::: "memory");
 }
@@ -308,8 +309,9 @@ __device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 0;\n" ::: "m
 //
 // CLU: the CTAs are one thread-block cluster (at most 16, one slot per thread).  A finished tile goes
 // straight into the partners' shared memory (cp.async.bulk between CTAs, completion on the
-// partner's mbarrier), into one of two sets of buffers by the evaluation's parity: having a
-// partner's data of one evaluation says that it is past the reads of the set written next.
+// partner's mbarrier), into one of two sets of tiles (the own one, then the partners') by the
+// evaluation's parity: having a partner's data of one evaluation says that it is past the reads of
+// the set written next, and that it has all of what this CTA pushed before.
 template <typename R, int S, bool REG, bool PEC, bool COMP, bool CLU>
 __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t cta, const uint32_t G,
                                               BatchInst* const inst) {
@@ -507,6 +509,11 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
       const RGen<R>* const gen = s_gen + par * ng;
       const RScal<R>& sc = s_sc[par];
       RED red0 = (RED)0, red1 = (RED)0;
+      // the set of tiles that this evaluation reads, and where the own tile of the next one goes
+      const uint32_t set = CLU ? (uint32_t)cluster_set(e) * (1u + (uint32_t)nd) : 0u;
+      const unsigned char* const tiles = smem + (size_t)set * tbytes;
+      C2* const xs_e = xs + (size_t)set * tsize;
+      C2* const xs_next = CLU ? xs + (size_t)((uint32_t)cluster_set(e + 1) * (1u + (uint32_t)nd)) * tsize : xs;
       for (uint32_t tile = cta; tile < ntiles; tile += G, visit++) {
         const uint32_t zb = tile << P.t;
         if (e == 0 || multi) {  // the own tile and its clause bytes (then kept up to date in place)
@@ -668,7 +675,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
             }
           }
         };
-        if (act) runs_to(smem, s_part[0].run_end);
+        if (act) runs_to(tiles, s_part[0].run_end);
         // what does not need the partners, while their tiles are on their way (owned vectors in
         // registers): the diagonal and the past's part of the corrector and the predictor
         auto diagonal = [&](uint32_t j, int q) {
@@ -687,10 +694,10 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
           }
         if (nd > 0 && !ring) {  // every partner in one go: the places name the buffers
           if (CLU)
-            arrived((uint32_t)par, (uint32_t)(e >> 1) & 1u);
+            arrived((uint32_t)cluster_set(e), (uint32_t)(e >> 1) & 1u);
           else
             arrived(0, visit & 1u);
-          if (act) runs_to(smem + (CLU && par ? (size_t)nd * tbytes : 0), P.nruns);
+          if (act) runs_to(tiles, P.nruns);
         }
         uint32_t rb = ring ? q0 % (uint32_t)nbuf : 0u, ru = ring ? q0 / (uint32_t)nbuf : 0u;
         auto release = [&]() {  // this warp is done with buffer rb; on to the next ring entry
@@ -708,9 +715,9 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
             release();
           }
         }
-        // every owner is past the products that read the own tile: it can be overwritten
-        // (in a cluster also by the copies that push it)
-        asm volatile("bar.sync 1, %0;\n" ::"r"(CLU ? nth + 32 : nth) : "memory");
+        // every owner is past the products that read the own tile: it can be overwritten (in a cluster
+        // the next one goes elsewhere)
+        if (!CLU) asm volatile("bar.sync 1, %0;\n" ::"r"(nth) : "memory");
         R t0 = (R)0, t1 = (R)0;
         auto fetch_owned = [&](int s, Owned& w) {  // of one slot, from global memory
           const uint32_t z = zb + (uint32_t)(j0 + s * js);
@@ -746,7 +753,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
           if (!act) continue;
           const uint32_t j = (uint32_t)(j0 + s * js), z0 = zb + j;
           C2 own[H], nx[H];
-          load(xs + j, own);
+          load(xs_e + j, own);
 #pragma unroll
           for (int q = 0; q < H; q++) {
             R re = ar[s * H + q], im = ai[s * H + q];
@@ -820,7 +827,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
             }
           }
           if (kind != 7 && (!CLU || last)) store(xout + z0, nx);  // partners of a cluster get it from the tile
-          if (!last && !multi) store(xs + j, nx);
+          if (!last && !multi) store(xs_next + j, nx);
           if (!REG) {
             if (kind == 0 || kind == 5 || kind == 1) store(F(latest + 1) + z0, w.a);
             if (kind == 0 || kind == 4) store((kind == 0 ? YO : Y) + z0, w.y);
@@ -897,14 +904,13 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
           if (e == 0) {
             copy_in(tile, xin, e, latest, q0);
           } else {  // the own tile to the partners
-            if (lane == 0) expect(full0 + 8u * (e & 1), (uint32_t)nd * tbytes);
+            const uint32_t k = (uint32_t)cluster_set(e), bb = full0 + 8u * k;
+            const C2* const set = xs + (size_t)(k * (1u + (uint32_t)nd)) * tsize;
+            if (lane == 0) expect(bb, (uint32_t)nd * tbytes);
             for (int p = lane; p < nd; p += 32)
-              tile_push(saddr(xs + (size_t)(1 + p + ((e & 1) ? nd : 0)) * tsize), saddr(xs), tbytes, full0 + 8u * (e & 1),
-                        cta ^ s_part[p + 1].hi);
-            push_sources_read();
+              tile_push(saddr(set + (size_t)(1 + p) * tsize), saddr(set), tbytes, bb, cta ^ s_part[p + 1].hi);
             __syncwarp();
           }
-          asm volatile("bar.sync 1, %0;\n" ::"r"(nth + 32) : "memory");
         } else if (svc == 3 && nq > 0) {
           copy_in(tile, xin, e, latest, q0);
         }
