@@ -440,6 +440,12 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
     }
     __syncwarp();
   };
+  auto copies_land = [&]() {  // at the end of a launch that gave up (one warp): the copies under way, bounded
+    const int used = CLU ? 2 : (ring ? nbuf : (nbuf > 0 ? 1 : 0));
+    for (int b = lane; b < used; b += 32)
+      for (uint32_t par = 0; par < 2; par++) (void)bar_wait_short(full0 + 8u * b, par);
+    __syncwarp();
+  };
   auto all_sync = [&]() { asm volatile("bar.sync 2, %0;\n" ::"r"((int)blockDim.x) : "memory"); };
   const C2* const src0 = reinterpret_cast<const C2*>(P.src);
   C2* const XA = reinterpret_cast<C2*>(P.xout[0]);
@@ -932,10 +938,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
       if (!CLU && !multi && svc == 3 && lane == 0 && nd > 0) flag_release(P.flags + kResFlagStride * cta, (unsigned)(e + 1));
       xin = e & 1 ? XO : XA;
     }
-    if (s_abort && svc == 3) {  // copies in flight land before the CTA leaves (bounded)
-      for (int b = lane; b < nbuf; b += 32)
-        for (uint32_t par = 0; par < 2; par++) (void)bar_wait_short(full0 + 8u * b, par);
-    }
+    if (s_abort && svc == 3 && !CLU) copies_land();
     if (PEC || P.single == 7) {
       all_sync();
       all_sync();  // the last reductions are there
@@ -946,7 +949,14 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
     }
   }
   const bool reduced = P.n_pec > 0 || P.single == 7;
-  if (CLU) cluster_sync();  // no CTA leaves while others may still write into its shared memory
+  if (CLU) {
+    // No CTA leaves while a push into or out of its shared memory is under way.  At a normal end every push
+    // has been waited for; to a CTA that gave up one may still come, so that CTA waits once none is issued
+    // any more, and all of them for it.
+    cluster_sync();
+    if (s_abort && svc == 3) copies_land();
+    cluster_sync();
+  }
   if (P.single == 6) return;
   __syncthreads();
   if (reduced) {
