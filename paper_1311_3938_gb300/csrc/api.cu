@@ -281,8 +281,6 @@ struct DeviceGuard {
 // n = 19 83 / 74, 169 / 180, 306 / 199.)
 constexpr int kResMaxN[2] = {18, 20};  // by precision
 
-constexpr size_t kResSmem = 222 * 1024;  // dynamic shared memory of a resident CTA (beside 5 KiB static)
-
 uint32_t layout_mask(const Layout& L) {
   uint32_t m = L.c >= 32 ? 0xffffffffu : ((1u << L.c) - 1u);
   if (L.w > 0) m |= ((1u << L.w) - 1u) << L.h;
@@ -517,8 +515,9 @@ int resident_threads(int slots) {
 
 // Products of a resident launch on tiles of 2^R.t by partner tile (the bits they flip above t; the
 // own tile, no such bit, first) into `rt`, and their counts and buffers into R.  False where the
-// tables leave no room for two partner buffers: such products stay on the layout passes.
-bool resident_tables(const aqc_ctx* c, ResPlan& R, ResTable* rt) {
+// tables leave no room for two partner buffers in `limit` bytes of dynamic shared memory: such
+// products stay on the layout passes.
+bool resident_tables(const aqc_ctx* c, ResPlan& R, ResTable* rt, size_t limit) {
   const DevTables* t = c->h_tab;
   const int total = t->flip_begin[t->n_layouts + 1];
   auto plain = [&](const DevFlip& f) { return f.zm == 0 && !f.has2; };
@@ -543,8 +542,8 @@ bool resident_tables(const aqc_ctx* c, ResPlan& R, ResTable* rt) {
   // and four for the owned vectors' quarter tiles where they come through the buffers
   R.nbuf = R.npart ? R.npart + (R.slots >= 4 ? 4 : 0) : 0;
   auto bytes = [&]() { return resident_smem_bytes(c->prec, R.t, R.nbuf, R.np, R.ng, t->n_z, R.nth, false); };
-  while (R.nbuf > 2 && bytes() > kResSmem) R.nbuf--;
-  if (bytes() > kResSmem) return false;
+  while (R.nbuf > 2 && bytes() > limit) R.nbuf--;
+  if (bytes() > limit) return false;
   // runs of one kind, cut between partners where those come one by one (the kernel's ring), between
   // the own tile and the others everywhere
   const bool ring = R.nbuf > 0 && (R.slots >= 4 || R.npart > R.nbuf);
@@ -600,7 +599,7 @@ void plan_resident(aqc_ctx* c) {
   const int slots_all = std::max(1, (1 << R.t) / H);
   R.nth = resident_threads(slots_all);
   R.slots = std::max(1, slots_all / R.nth);
-  R.on = resident_tables(c, R, &c->h_res.alone);
+  R.on = resident_tables(c, R, &c->h_res.alone, kResSmem);
   c->res = R;
 }
 
@@ -1765,7 +1764,7 @@ int batch_plan_waves(aqc_batch* b) {
     for (const Job& j : w) {
       aqc_ctx* c = b->members[j.slot];
       ResPlan R = member_plan(c, best);
-      if (!resident_tables(c, R, &c->h_res.batch)) BFAIL(b, AQC_E_UNSUPPORTED, "member tables too large");
+      if (!resident_tables(c, R, &c->h_res.batch, kResBatchSmem)) BFAIL(b, AQC_E_UNSUPPORTED, "member tables too large");
       if (b->res_t[j.slot] != R.t) {
         c->h_res.member = ResMember{c->n, R.t, R.np, R.ng, R.npart, R.nbuf, R.nruns, R.ncode, c->d_sync + 1, c->d_sync,
                                     c->d_partials, c->d_slots};
@@ -2779,7 +2778,7 @@ static bool batch_holds(const aqc_batch* b, aqc_ctx* c) {
   if ((1 << (c->n - std::min(c->n, hi))) > std::min(b->sms, kResMaxCtas)) return false;
   for (int tb = 9; tb <= hi; tb++) {
     ResPlan R = member_plan(c, tb);
-    if (c->n - R.t <= 7 && !resident_tables(c, R, &c->h_res.batch)) return false;
+    if (c->n - R.t <= 7 && !resident_tables(c, R, &c->h_res.batch, kResBatchSmem)) return false;
   }
   return true;
 }

@@ -258,6 +258,19 @@ struct ResParams {
   double* slots;
 };
 
+// Static shared memory of a resident launch (a batch's also holds the member's ResParams), and what is
+// left for dynamic memory of a multiprocessor's 227 KiB per CTA.
+struct ResStatic {
+  ResPartner part[kResMaxTiles];
+  ResRun run[kResMaxRuns];
+  double err[kResMaxEvals + 2];
+  volatile int abort;
+  int last;
+};
+constexpr size_t res_dynamic(size_t fixed) { return 227 * 1024 - (fixed + 127) / 128 * 128; }
+constexpr size_t kResSmem = res_dynamic(sizeof(ResStatic));
+constexpr size_t kResBatchSmem = res_dynamic(sizeof(ResStatic) + sizeof(ResParams) + alignof(ResParams));
+
 // vectors of a state (workspace order)
 constexpr int kVecY = 0, kVecP = 1, kVecQ = 2, kVecF0 = 3, kVecAcc = 7, kVecCount = 8;
 

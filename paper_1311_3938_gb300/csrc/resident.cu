@@ -323,10 +323,11 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
   constexpr int SC = S / 4 > 0 ? S / 4 : 1;  // slots per streamed quarter tile
   using RED = typename std::conditional<REG, R, double>::type;
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ ResPartner s_part[kResMaxTiles];
-  __shared__ ResRun s_run[kResMaxRuns];
-  __shared__ volatile int s_abort;
-  __shared__ double s_err[kResMaxEvals + 2];
+  __shared__ ResStatic sh;
+  ResPartner* const s_part = sh.part;
+  ResRun* const s_run = sh.run;
+  volatile int& s_abort = sh.abort;
+  double* const s_err = sh.err;
 
   const DevTables* tab = P.tab;
   const int nth = (int)blockDim.x - kService, nwarps = nth >> 5;
@@ -969,7 +970,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
     }
   }
   // the last CTA sums the CTAs' partials in CTA order and clears the flags for the next launch
-  __shared__ int s_last;
+  int& s_last = sh.last;
   __syncthreads();
   if (tid == 0) {
     __threadfence();
