@@ -65,21 +65,46 @@ struct PFlip<double> {
 // the X driver share one coefficient, so their part of H psi is c * (sum of the partners): a tile's
 // amplitudes are converted once to integers scaled by the tile's largest exponent, summed exactly,
 // and the sum is converted back: two FP64 operations per amplitude instead of two per product.
-// Accuracy: the scale leaves the sum of the tile's products just below 2^62, so with up to 16
-// products an amplitude keeps 58 bits below the tile's largest one, and sums of them round once;
-// FP64 rounds every partial sum to 53 bits.
-__device__ __forceinline__ int64_t to_fixed(double v, int emax, int up) {
+// Accuracy: real and imaginary parts have a scale each, which leaves the sum of the tile's products just
+// below 2^62, so a unit is at most 2^-57 (16 products) to 2^-59 (4) of the tile's largest part.  A
+// partner is off by half a unit at most.  FP64 rounds after every product, by up to half an ulp of the
+// sum so far, and where a partner reaches 2^52 units that ulp is a unit or more.  A tile in which the
+// partners of some amplitude all lie below (and lost bits: small amplitudes beside large ones of
+// other places) is summed in FP64 instead: no sum keeps less than FP64's bits.  Random amplitudes
+// pass; late in a run, when the amplitudes of a tile differ by orders of magnitude, most tiles do
+// not.  Microseconds per grid step, linear path from the uniform state, first tenth / second half of a
+// run: n = 20 95 / 146 (FP64 throughout 172), n = 22 394 / 560 (626); integers throughout, tails lost, 93 and 385.
+// `rough` is set where a value below 2^52 units is not zero.
+__device__ __forceinline__ int64_t to_fixed(double v, int emax, int up, bool& rough) {
   const int64_t b = __double_as_longlong(v);
   const int e = (int)((b >> 52) & 0x7ff);
   int64_t m = b & 0xfffffffffffffll;
   if (e) m |= 1ll << 52;
   const int sh = up - (emax - (e ? e : 1));
+  rough = rough || (sh < 0 && m != 0);
   int64_t r;
   if (sh >= 0)
     r = m << sh;
   else
     r = sh < -62 ? 0 : (m + (1ll << (-sh - 1))) >> -sh;
   return b < 0 ? -r : r;
+}
+// the same without branches and flag (emax 256 or more: subnormal values round to zero)
+__device__ __forceinline__ int64_t to_fixed(double v, int emax, int up) {
+  const int64_t b = __double_as_longlong(v);
+  const int d = emax - (int)((b >> 52) & 0x7ff), dc = d < 63 ? d : 63;
+  const uint64_t m = (uint64_t)((b & 0xfffffffffffffll) | (1ll << 52)) << up;  // below 2^62
+  const int64_t r = (int64_t)((m + ((1ull << dc) >> 1)) >> dc);
+  return b < 0 ? -r : r;
+}
+// lanes' bits of the lanes that an XOR by f (below 32) leads to
+__device__ __forceinline__ uint32_t flip_lanes(uint32_t w, uint32_t f) {
+  if (f & 1u) w = ((w & 0x55555555u) << 1) | ((w >> 1) & 0x55555555u);
+  if (f & 2u) w = ((w & 0x33333333u) << 2) | ((w >> 2) & 0x33333333u);
+  if (f & 4u) w = ((w & 0x0f0f0f0fu) << 4) | ((w >> 4) & 0x0f0f0f0fu);
+  if (f & 8u) w = ((w & 0x00ff00ffu) << 8) | ((w >> 8) & 0x00ff00ffu);
+  if (f & 16u) w = (w << 16) | (w >> 16);
+  return w;
 }
 // nearest double of s 2^k (ties upward; s 2^k normal or zero), in integer instructions
 __device__ __forceinline__ double from_fixed(int64_t s, int k = 0) {
@@ -131,7 +156,7 @@ __host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~(size_t
 // dynamic shared memory map of k_apply: [tile][clause bytes][plain flips][general flips][Z strings][reduction]
 template <typename R>
 struct SmemMap {
-  size_t code, pf, gf, zs, red, total;
+  size_t code, pf, gf, zs, red, big, total;
   __host__ __device__ SmemMap(uint32_t tsize, int np, int ng, int nz) {
     using C2 = typename Cplx<R>::T;
     code = align16((size_t)tsize * sizeof(C2));  // the tile's clause bytes
@@ -139,7 +164,8 @@ struct SmemMap {
     gf = align16(pf + (size_t)np * sizeof(PFlip<R>));
     zs = align16(gf + (size_t)ng * sizeof(SFlip<R>));
     red = align16(zs + (size_t)nz * sizeof(SZ<R>));
-    total = red + 8 * 2 * sizeof(double) + 16;
+    big = align16(red + 8 * 2 * sizeof(double) + 16);  // integer sums: two bits per amplitude
+    total = big + (sizeof(R) == 8 ? tsize / 4 : 0);
   }
 };
 
@@ -315,6 +341,7 @@ struct TileCtx {
   SFlip<R>* s_gf;
   SZ<R>* s_z;
   double* s_red;
+  uint32_t* s_big;
   uint64_t pol_keep, pol_drop;  // L2 policies (evict_last / evict_first) of hinted tile passes
 };
 
@@ -365,6 +392,7 @@ __device__ __forceinline__ void load_coefficients(TileCtx<R>& T, const DevTables
   T.s_gf = reinterpret_cast<SFlip<R>*>(tb + map.gf);
   T.s_z = reinterpret_cast<SZ<R>*>(tb + map.zs);
   T.s_red = reinterpret_cast<double*>(tb + map.red);
+  T.s_big = reinterpret_cast<uint32_t*>(tb + map.big);
   for (int k = threadIdx.x; k < T.np; k += blockDim.x) {
     const DevFlip d = tab->flips[fb + k];
     PFlip<R> f;
@@ -572,34 +600,91 @@ __device__ __forceinline__ void process_tile(const TileCtx<R>& T, uint32_t zb, u
   const bool full = tsize >= 2 * HB;  // every state with more than 6 (complex64) / 5 qubits
   // equal-coefficient products as integers: the tile is converted in place
   bool uni = sizeof(R) == 8 && !CL && full && T.nu > 0;
-  double uscale = 0.0;
+  double us[2] = {0.0, 0.0};  // coefficient times the value of a unit, real and imaginary parts
   if constexpr (sizeof(R) == 8 && !CL) {
     if (uni) {
-      uint32_t m = 0;
+      uint32_t* const s_max = reinterpret_cast<uint32_t*>(T.s_red);
+      const uint32_t nw = blockDim.x >> 5, rows = tsize >> 5;
+      uint32_t m[2] = {0u, 0u};
+      const bool any = threadIdx.x < tsize;
+      const C2 mine = any ? s_p[threadIdx.x] : zero2;
+#pragma unroll 8
       for (uint32_t j = threadIdx.x; j < tsize; j += blockDim.x) {
         const C2 v = s_p[j];
-        m = max(m, max((uint32_t)__double2hiint(v.x) & 0x7fffffffu, (uint32_t)__double2hiint(v.y) & 0x7fffffffu));
+        m[0] = max(m[0], (uint32_t)__double2hiint(v.x) & 0x7fffffffu);
+        m[1] = max(m[1], (uint32_t)__double2hiint(v.y) & 0x7fffffffu);
       }
-      m = __reduce_max_sync(0xffffffffu, m);
-      uint32_t* const s_max = reinterpret_cast<uint32_t*>(T.s_red);
-      if ((threadIdx.x & 31u) == 0u) s_max[threadIdx.x >> 5] = m;
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+        m[k] = __reduce_max_sync(0xffffffffu, m[k]);
+        if ((threadIdx.x & 31u) == 0u) s_max[2u * (threadIdx.x >> 5) + k] = m[k];
+      }
       __syncthreads();
-      m = 0;
-      for (uint32_t w = 0; w < (blockDim.x >> 5); w++) m = max(m, s_max[w]);
-      const int emax = (int)(m >> 20);
-      // tiles with infinities or NaN, and tiles so small that the scale would be subnormal, keep
-      // the FP64 products
-      uni = emax < 0x7ff && emax >= 256;
+      int emax[2];
+#pragma unroll
+      for (int k = 0; k < 2; k++) {
+        m[k] = 0;
+        for (uint32_t w = 0; w < nw; w++) m[k] = max(m[k], s_max[2u * w + k]);
+        // tiles with infinities or NaN, and tiles so small that the scale would be subnormal, keep
+        // the FP64 products; a part that is zero throughout takes any scale
+        emax[k] = max((int)(m[k] >> 20), 256);
+        uni = uni && emax[k] < 0x7ff && (m[k] == 0u || (m[k] >> 20) >= 256u);
+      }
       if (uni) {
+        // Too many of a sample small: some sum would lack a big partner, not worth the conversion.  With a
+        // share q of small parts a tile's 8192 sums of k products lack one with 8192 q^k: q = 1/2 at 12
+        // products, 1/3 at 8; the sample counts places whose two parts are big.
+        auto big = [&](double v, int k) {
+          return m[k] == 0u || (int)(((uint32_t)__double2hiint(v) & 0x7fffffffu) >> 20) >= emax[k] - T.up;
+        };
+        const int n = __syncthreads_count(any && big(mine.x, 0) && big(mine.y, 1));
+        uni = 4u * (uint32_t)n >= (T.nu > 8 ? 2u : 3u) * min(tsize, blockDim.x);
+      }
+      if (uni) {
+        bool rough = false;
+#pragma unroll 4
         for (uint32_t j = threadIdx.x; j < tsize; j += blockDim.x) {
           const C2 v = s_p[j];
           longlong2 q;
-          q.x = to_fixed(v.x, emax, T.up);
-          q.y = to_fixed(v.y, emax, T.up);
+          q.x = to_fixed(v.x, emax[0], T.up, rough);
+          q.y = to_fixed(v.y, emax[1], T.up, rough);
           reinterpret_cast<longlong2*>(s_p)[j] = q;
         }
-        uscale = T.s_pf[0].c * __longlong_as_double((long long)(emax - 1075 - T.up + 1023) << 52);
-        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 2; k++)
+          us[k] = T.s_pf[0].c * __longlong_as_double((long long)(emax[k] - 1075 - T.up + 1023) << 52);
+        if (__syncthreads_or(rough)) {
+#pragma unroll 4
+          for (uint32_t j = threadIdx.x; j < tsize; j += blockDim.x) {  // (whole warps)
+            const longlong2 q = reinterpret_cast<const longlong2*>(s_p)[j];
+            const int hx = (int)(q.x >> 32), hy = (int)(q.y >> 32);
+            const uint32_t wx = __ballot_sync(0xffffffffu, hx >= (1 << 20) || hx < -(1 << 20));
+            const uint32_t wy = __ballot_sync(0xffffffffu, hy >= (1 << 20) || hy < -(1 << 20));
+            if ((threadIdx.x & 31u) == 0u) {
+              T.s_big[j >> 5] = wx;
+              T.s_big[rows + (j >> 5)] = wy;
+            }
+          }
+          __syncthreads();
+          bool good = true;  // every sum has a big partner
+          for (uint32_t i = threadIdx.x; i < 2u * rows; i += blockDim.x) {
+            if ((i >= rows ? m[1] : m[0]) == 0u) continue;  // all zero
+            const uint32_t* const w = T.s_big + (i >= rows ? rows : 0u);
+            const uint32_t r = i >= rows ? i - rows : i;
+            uint32_t any = 0u;
+            for (int kk = 0; kk < T.nu; kk++) {
+              const uint32_t lx = T.s_pf[kk].lx;
+              any |= flip_lanes(w[r ^ (lx >> 5)], lx & 31u);
+            }
+            good = good && any == 0xffffffffu;
+          }
+          uni = __syncthreads_and(good) != 0;
+          if (!uni) {  // the amplitudes again
+            for (uint32_t j = threadIdx.x; j < tsize; j += blockDim.x) cp_async16(s_p + j, src + tile_z(L, j, zb));
+            cp_async_wait_all();
+            __syncthreads();
+          }
+        }
       }
     }
   }
@@ -822,8 +907,8 @@ __device__ __forceinline__ void process_tile(const TileCtx<R>& T, uint32_t zb, u
         }
 #pragma unroll
         for (int g = 0; g < 2; g++) {
-          ar[g] = fma((double)uscale, from_fixed(sr[g]), (double)ar[g]);
-          ai[g] = fma((double)uscale, from_fixed(si[g]), (double)ai[g]);
+          ar[g] = fma(us[0], from_fixed(sr[g]), (double)ar[g]);
+          ai[g] = fma(us[1], from_fixed(si[g]), (double)ai[g]);
         }
       }
     }
