@@ -183,6 +183,7 @@ struct aqc_ctx {
   int sms = 0;        // multiprocessors of the device
   SlabParams slab;    // slab-ordered last passes of a PEC step (slab.n_slabs == 0: off)
   bool in_batch = false;  // batch members use per-CTA tiles only
+  bool batch_declined = false;  // a member on layout passes whose size would run resident
 
   // staged host transfers (aqc_transfer_attach): caller-owned staging vectors, library-owned
   // copy streams; in_free / out_free mark when the context stream has consumed / the output
@@ -370,13 +371,26 @@ int to_qubit_order(aqc_ctx* c, void* dst, const void* src) { return permute_gath
 // own gets them).
 bool resident_size(const aqc_ctx* c) { return c->tile_bits == 0 && c->n <= kResMaxN[c->prec]; }
 
+// A context of such a size whose evaluations run resident: no option that selects another pass order
+// (slabs need three layouts, more than these sizes have), no clause-by-clause sequence (its
+// coefficients change shape with s), tables that fit.
+bool resident_wanted(const aqc_ctx* c) {
+  if (!resident_size(c) || c->res_declined || c->batch_declined || c->turn_req != 0) return false;
+  for (const ClauseH& k : c->clauses)
+    if (k.stepwise) return false;
+  return true;
+}
+
 // Order that minimises the products (weighted by how many share a flip mask) that no layout
 // holds: deterministic local search over transpositions, kept only if strictly better than the
 // identity.
 std::vector<int> choose_order(const aqc_ctx* c) {
   std::vector<int> id(c->n);
   for (int q = 0; q < c->n; q++) id[q] = q;
-  if (!c->relabel || c->layouts.size() < 2 || (resident_size(c) && !c->res_declined)) return id;
+  // (resident launches exchange whole tiles in any order; everything else gains: clause-by-clause XY path,
+  // complex128, microseconds per step in the identity's order / the chosen one: n = 16 301 / 226,
+  // n = 18 420 / 248; complex64 n = 20 92 / 85)
+  if (!c->relabel || c->layouts.size() < 2 || resident_wanted(c)) return id;
   std::vector<std::pair<uint32_t, int>> masks;  // distinct multi-bit flip masks with counts
   for (const TermH& th : c->terms) {
     if (__builtin_popcount(th.x) < 2) continue;
@@ -603,11 +617,7 @@ void plan_resident(aqc_ctx* c) {
   c->res = R;
 }
 
-// The launches run resident: no option that selects another pass order, no clause-by-clause
-// sequence (its coefficients change shape with s).
-bool resident_on(const aqc_ctx* c) {
-  return c->res.on && !c->slab.n_slabs && c->turn_req == 0 && c->step_class < 0;
-}
+bool resident_on(const aqc_ctx* c) { return c->res.on && resident_wanted(c); }
 
 int build_tables(aqc_ctx* c) {
   c->tables_version++;
@@ -2805,13 +2815,14 @@ int aqc_batch_add(aqc_batch* b, aqc_ctx* c, int* slot_out) {
   const bool res = rc == 0 && resident_on(c) && batch_holds(b, c);
   if (!rc && !res && !c->in_batch) {
     c->in_batch = true;  // per-CTA tiles for the batched kernel
+    c->batch_declined = true;
     c->dirty = true;
     rc = ensure_ready(c);
   }
   if (!rc) rc = plan_first_segment(c);
   if (rc) {
     if (c->in_batch) c->dirty = true;
-    c->in_batch = false;
+    c->in_batch = c->batch_declined = false;
     BFAIL(b, rc, "member: %s", c->err.c_str());
   }
   c->in_batch = true;
@@ -2889,7 +2900,7 @@ int aqc_batch_remove(aqc_batch* b, int slot) {
     c->dirty = true;
   }
   b->members[slot] = nullptr;
-  c->in_batch = false;
+  c->in_batch = c->batch_declined = false;
   memset(&b->h_insts[slot], 0, sizeof(BatchInst));
   BCUDA(b, cudaMemcpyAsync(b->d_insts + slot, &b->h_insts[slot], sizeof(BatchInst), cudaMemcpyHostToDevice, b->stream));
   BCUDA(b, cudaStreamSynchronize(b->stream));
