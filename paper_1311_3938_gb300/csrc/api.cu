@@ -1007,6 +1007,7 @@ bool tile_x_pass(const aqc_ctx* c, const ApplyParams& p, XParams* x) {
   x->stage = p.stage;
   x->with_diag = p.with_diag;
   x->with_remote = remote;
+  x->others = p.with_diag && (c->n_z > 0 || c->h_tab->n_classes > (p.dcode ? 1 : 0));
   x->top_bits = remote ? c->n - p.L.h - p.L.w : 0;
   for (int g = 0; g < 3; g++) x->w[g] = p.w[g];
   x->wdev = p.wdev;

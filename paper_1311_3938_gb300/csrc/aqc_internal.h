@@ -201,6 +201,7 @@ struct XParams {
   int layout_index;
   int mode, stage;       // as in ApplyParams
   int with_diag, with_remote;
+  int others;            // with_diag: clause classes beside the byte table's, or Z strings
   int top_bits;          // > 0: visit tiles that differ in this many top index bits side by side
   double w[3];
   const double* wdev;    // nullable: weights from device memory (as ApplyParams::wdev)

@@ -208,30 +208,51 @@ struct XSmem {  // [pad to 1 KiB][tile 0][tile 1][clause bytes 0, 1][flips][Z st
   }
 };
 
-// clause classes other than the byte table's and Z strings at index z (rare)
-__device__ __noinline__ float x_other_diagonal(const XParams& P, const float2* s_z, int code, uint32_t z) {
+// Clause classes other than the byte table's and Z strings (XY path: the catalyst; Ising couplings), for
+// a thread's 16 amplitudes: index zj, its pair bit and bits 6..8.  Each class, clause and string is taken
+// once for all of them, a string by one parity and the signs of those four bits.  (One amplitude at a time
+// 120 strings made a step at n = 24 take 1.59 ms; three layout passes with this part in the one of k_apply
+// took 1.26.)
+__device__ __forceinline__ void x_other_diagonal(const XParams& P, const float2* s_z, int nz, const int (&code)[16],
+                                                 uint32_t zj, float (&d)[16]) {
   const DevTables* tab = P.tab;
   const int tcls = P.dcode ? tab->table_class : -1;
-  float d = 0.f;
+#pragma unroll
+  for (int i = 0; i < 16; i++) d[i] = 0.f;
   for (int cc = 0; cc < tab->n_classes; cc++) {
     if (cc == tcls) continue;
     const DevClass cl = tab->classes[cc];
     const bool derived = cl.derived && tcls >= 0;
     const int b = derived ? cl.dbegin : cl.begin, e = derived ? cl.dend : cl.end;
-    int cnt = 0;
+    int cnt[16];
+#pragma unroll
+    for (int i = 0; i < 16; i++) cnt[i] = 0;
     for (int k = b; k < e; k++) {
-      const int o = 1 - __popc(tab->clause_mask[k] & z);
-      cnt += cl.pen == 0 ? (o != 0) : o * o;
+      const uint32_t m = tab->clause_mask[k];
+#pragma unroll
+      for (int i = 0; i < 16; i++) {
+        const int o = 1 - __popc(m & (zj | (uint32_t)((i >> 1) << 6) | (uint32_t)(i & 1)));
+        cnt[i] += cl.pen == 0 ? (o != 0) : o * o;
+      }
     }
-    d = fmaf((float)(cl.scale * weight_of(P, cl.group)), (float)(derived ? code - cnt : cnt), d);
+    const float w = (float)(cl.scale * weight_of(P, cl.group));
+#pragma unroll
+    for (int i = 0; i < 16; i++) d[i] = fmaf(w, (float)(derived ? code[i] - cnt[i] : cnt[i]), d[i]);
   }
-  for (int m = 0; m < tab->n_z; m++) d += (__popc(__float_as_uint(s_z[m].x) & z) & 1) ? -s_z[m].y : s_z[m].y;
-  return d;
+  for (int m = 0; m < nz; m++) {
+    const uint32_t zm = __float_as_uint(s_z[m].x);
+    const uint32_t c = __float_as_uint(s_z[m].y) ^ ((uint32_t)__popc(zm & zj) << 31);
+    const uint32_t s0 = zm << 31, s6 = (zm >> 6) << 31, s7 = (zm >> 7) << 31, s8 = (zm >> 8) << 31;
+#pragma unroll
+    for (int i = 0; i < 16; i++)
+      d[i] += __uint_as_float(c ^ (i & 1 ? s0 : 0u) ^ (i & 2 ? s6 : 0u) ^ (i & 4 ? s7 : 0u) ^ (i & 8 ? s8 : 0u));
+  }
 }
 
 // MODE as in ApplyParams.  DIAG: this pass adds the diagonal (the contiguous layout).  FAR: it reads
-// the partners of products that no layout holds.
-template <int MODE, bool DIAG, bool FAR>
+// the partners of products that no layout holds.  OTHERS: the diagonal has more than the byte table's
+// class (kernels of their own: the part's registers would cost the others 3%).
+template <int MODE, bool DIAG, bool FAR, bool OTHERS>
 __global__ void __launch_bounds__(kXThreads, 1) k_tile_x(const __grid_constant__ XParams P) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   unsigned char* base = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
@@ -242,7 +263,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_tile_x(const __grid_constant__
   const int npl = tab->plain_count[P.layout_index];
   const int np = npl + tab->hop_count[P.layout_index];  // X strings, then hops
   const int nf = np + (FAR ? tab->n_remote : 0);
-  const int nz = DIAG ? tab->n_z : 0, ncls = DIAG ? tab->n_classes : 0;
+  const int nz = DIAG && OTHERS ? tab->n_z : 0;
   const XSmem M(nf, nz, DIAG && P.dcode);
   XFlip* s_f = reinterpret_cast<XFlip*>(base + M.flips);
   float2* s_z = reinterpret_cast<float2*>(base + M.z);
@@ -258,11 +279,9 @@ __global__ void __launch_bounds__(kXThreads, 1) k_tile_x(const __grid_constant__
   for (int k = tid; k < nz; k += blockDim.x)
     s_z[k] = make_float2(__uint_as_float(tab->z[k].zm), (float)(tab->z[k].coef * weight_of(P, tab->z[k].group)));
   float dconst = 0.f, wtab = 0.f;
-  bool others = false;
   if (DIAG) {
     dconst = (float)(tab->ident[0] * weight_of(P, 0) + tab->ident[1] * weight_of(P, 1) + tab->ident[2] * weight_of(P, 2));
     if (P.dcode) wtab = (float)(tab->classes[tab->table_class].scale * weight_of(P, tab->classes[tab->table_class].group));
-    others = nz > 0 || ncls > (P.dcode ? 1 : 0);
   }
   if (tid == 0) {
     mbar_init(bar0, 1);
@@ -470,35 +489,44 @@ __global__ void __launch_bounds__(kXThreads, 1) k_tile_x(const __grid_constant__
         if (P.stage > 1) v[1] = *reinterpret_cast<const float4*>(reinterpret_cast<const float2*>(P.acc) + z);
       }
     };
-    if (NV > 0) fetch(0, in[0]);
     const uint8_t* const code = base + M.code + ((size_t)b << kXTileBits);
+    auto counts = [&](int r, int& k0, int& k1) {  // cached clause counts of a pair
+      k0 = k1 = 0;
+      if (P.dcode) {
+        const uint32_t two = *reinterpret_cast<const uint16_t*>(code + (jw | ((uint32_t)r << 6)));
+        k0 = (int)(two & 0xffu);
+        k1 = (int)(two >> 8);
+      }
+    };
+    // (selects: a branch lets the warp's stores come apart, 1% of a step at 28 qubits)
+    auto add_diagonal = [&](float d0, float d1, const float4& w, float4& a) {
+      const bool n0 = d0 != 0.f, n1 = d1 != 0.f;
+      const float4 t = make_float4(fmaf(d0, w.x, a.x), fmaf(d0, w.y, a.y), fmaf(d1, w.z, a.z), fmaf(d1, w.w, a.w));
+      a = make_float4(n0 ? t.x : a.x, n0 ? t.y : a.y, n1 ? t.z : a.z, n1 ? t.w : a.w);
+    };
+    if constexpr (DIAG && OTHERS) {
+      int k16[16];
+      float od[16];
+#pragma unroll
+      for (int r = 0; r < 8; r++) counts(r, k16[2 * r], k16[2 * r + 1]);
+      x_other_diagonal(P, s_z, nz, k16, zj, od);
+#pragma unroll
+      for (int r = 0; r < 8; r++)
+        add_diagonal(fmaf(wtab, (float)k16[2 * r], dconst) + od[2 * r],
+                     fmaf(wtab, (float)k16[2 * r + 1], dconst) + od[2 * r + 1], own[r], acc[r]);
+    }
+    if (NV > 0) fetch(0, in[0]);
     float t0 = 0.f, t1 = 0.f;
 #pragma unroll
     for (int r = 0; r < 8; r++) {
       if (NV > 0 && r < 7) fetch(r + 1, in[(r + 1) & 1]);
-      const uint32_t z = zb + zoff[r], j = jw | ((uint32_t)r << 6);
+      const uint32_t z = zb + zoff[r];
       float4 a = acc[r];
       const float4 w = own[r];
-      if (DIAG) {
-        int k0 = 0, k1 = 0;
-        if (P.dcode) {
-          const uint32_t two = *reinterpret_cast<const uint16_t*>(code + j);
-          k0 = (int)(two & 0xffu);
-          k1 = (int)(two >> 8);
-        }
-        float d0 = fmaf(wtab, (float)k0, dconst), d1 = fmaf(wtab, (float)k1, dconst);
-        if (others) {
-          d0 += x_other_diagonal(P, s_z, k0, z);
-          d1 += x_other_diagonal(P, s_z, k1, z + 1u);
-        }
-        if (d0 != 0.f) {
-          a.x = fmaf(d0, w.x, a.x);
-          a.y = fmaf(d0, w.y, a.y);
-        }
-        if (d1 != 0.f) {
-          a.z = fmaf(d1, w.z, a.z);
-          a.w = fmaf(d1, w.w, a.w);
-        }
+      if constexpr (DIAG && !OTHERS) {
+        int k0, k1;
+        counts(r, k0, k1);
+        add_diagonal(fmaf(wtab, (float)k0, dconst), fmaf(wtab, (float)k1, dconst), w, a);
       }
       auto put = [&](void* v, const float4& x) { *reinterpret_cast<float4*>(reinterpret_cast<float2*>(v) + z) = x; };
       const float4 fn = make_float4(a.y, -a.x, a.w, -a.z);  // -i r
@@ -511,6 +539,7 @@ __global__ void __launch_bounds__(kXThreads, 1) k_tile_x(const __grid_constant__
         t1 += (w.x * a.y - w.y * a.x) + (w.z * a.w - w.w * a.z);
       } else if constexpr (MODE == MODE_STEP) {
         const float4(&v)[NV] = in[r & 1];  // f_n, f_{n-1}, f_{n-2}, f_{n-3}
+        put(P.fout, fn);
         float4 pn, yn;
         auto one = [&](float p, float f, float f0, float f1, float f2, float f3, float& po, float& yo) {
           const float d1 = f - f0, d2 = f0 - f1, d3 = f1 - f2, d4 = f2 - f3;
@@ -525,7 +554,6 @@ __global__ void __launch_bounds__(kXThreads, 1) k_tile_x(const __grid_constant__
         one(w.y, fn.y, v[0].y, v[1].y, v[2].y, v[3].y, pn.y, yn.y);
         one(w.z, fn.z, v[0].z, v[1].z, v[2].z, v[3].z, pn.z, yn.z);
         one(w.w, fn.w, v[0].w, v[1].w, v[2].w, v[3].w, pn.w, yn.w);
-        put(P.fout, fn);
         put(P.pout, pn);
         if (P.yout) put(P.yout, yn);
       } else if constexpr (MODE == MODE_RK4) {
@@ -601,10 +629,10 @@ __global__ void __launch_bounds__(kXThreads, 1) k_tile_x(const __grid_constant__
   }
 }
 
-template <int MODE, bool DIAG, bool FAR = false>
+template <int MODE, bool DIAG, bool FAR = false, bool OTHERS = false>
 cudaError_t launch_x(const XParams& p, int n_flips, int n_z, cudaStream_t s) {
   const size_t smem = XSmem(n_flips, n_z, DIAG && p.dcode).total;
-  auto kern = k_tile_x<MODE, DIAG, FAR>;
+  auto kern = k_tile_x<MODE, DIAG, FAR, OTHERS>;
   static int configured = 0, cached_dev = -1, cached_g = 0;
   if ((int)smem > configured) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -628,6 +656,11 @@ cudaError_t launch_x(const XParams& p, int n_flips, int n_z, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+template <int MODE>
+cudaError_t launch_diag(const XParams& p, int n_flips, int n_z, cudaStream_t s) {
+  return p.others ? launch_x<MODE, true, false, true>(p, n_flips, n_z, s) : launch_x<MODE, true>(p, n_flips, n_z, s);
+}
+
 }  // namespace
 
 bool tile_x_layout_ok(const Layout& L) {
@@ -641,14 +674,17 @@ size_t tile_x_smem_bytes(int n_flips, int n_z, bool codes) { return XSmem(n_flip
 
 cudaError_t launch_tile_x(const XParams& p, int n_flips, int n_z, cudaStream_t s) {
   if (p.with_remote && (p.mode != MODE_PARTIAL || p.with_diag)) return cudaErrorInvalidValue;
+  if (!p.with_diag) {
+    if (p.mode != MODE_PARTIAL) return cudaErrorInvalidValue;
+    return p.with_remote ? launch_x<MODE_PARTIAL, false, true>(p, n_flips, 0, s)
+                         : launch_x<MODE_PARTIAL, false>(p, n_flips, 0, s);
+  }
   switch (p.mode) {
-    case MODE_PARTIAL: return p.with_diag ? launch_x<MODE_PARTIAL, true>(p, n_flips, n_z, s)
-                             : p.with_remote ? launch_x<MODE_PARTIAL, false, true>(p, n_flips, 0, s)
-                                             : launch_x<MODE_PARTIAL, false>(p, n_flips, 0, s);
-    case MODE_STEP: return launch_x<MODE_STEP, true>(p, n_flips, n_z, s);
-    case MODE_RK4: return launch_x<MODE_RK4, true>(p, n_flips, n_z, s);
-    case MODE_DERIV: return launch_x<MODE_DERIV, true>(p, n_flips, n_z, s);
-    case MODE_ENERGY: return launch_x<MODE_ENERGY, true>(p, n_flips, n_z, s);
+    case MODE_PARTIAL: return launch_diag<MODE_PARTIAL>(p, n_flips, n_z, s);
+    case MODE_STEP: return launch_diag<MODE_STEP>(p, n_flips, n_z, s);
+    case MODE_RK4: return launch_diag<MODE_RK4>(p, n_flips, n_z, s);
+    case MODE_DERIV: return launch_diag<MODE_DERIV>(p, n_flips, n_z, s);
+    case MODE_ENERGY: return launch_diag<MODE_ENERGY>(p, n_flips, n_z, s);
   }
   return cudaErrorInvalidValue;
 }
