@@ -94,10 +94,10 @@ __host__ __device__ constexpr int owners(int slots) { return slots >= 8 ? kResMa
 __host__ __device__ inline size_t up16(size_t v) { return (v + 15) & ~(size_t)15; }
 
 // shared memory: [own tile][nbuf partner tiles][clause bytes][weights][bases][plain x2][general x2]
-// [Z x2][scalars x2][reductions x2][lane sums][mbarriers]
+// [Z x2][Z masks][scalars x2][reductions x2][lane sums][mbarriers]
 template <typename R>
 struct ResSmem {
-  size_t code, w, base, pl, gen, z, scal, red, lane, bar, total;
+  size_t code, w, base, pl, gen, z, zm, scal, red, lane, bar, total;
   __host__ __device__ ResSmem(uint32_t tsize, int nbuf, int np, int ng, int nz, int nth, bool dred) {
     code = up16((size_t)tsize * (1 + nbuf) * 2 * sizeof(R));
     w = up16(code + tsize);
@@ -105,7 +105,8 @@ struct ResSmem {
     pl = up16(base + (size_t)np * sizeof(RBase));
     gen = up16(pl + 2 * (size_t)np * sizeof(RPlain<R>));
     z = up16(gen + 2 * (size_t)ng * sizeof(RGen<R>));
-    scal = up16(z + 2 * (size_t)nz * sizeof(R));
+    zm = up16(z + 2 * (size_t)nz * sizeof(R));
+    scal = up16(zm + (size_t)nz * sizeof(uint32_t));
     red = up16(scal + 2 * sizeof(RScal<R>));
     lane = up16(red + 2 * (size_t)nth * (dred ? sizeof(double) : sizeof(R)));
     bar = lane + 8 * (kResMaxEvals + 1) * sizeof(double);
@@ -276,20 +277,45 @@ __device__ __forceinline__ int count_clauses(const DevTables* __restrict__ tab, 
   return cnt;
 }
 
-// Diagonal parts beside the table lookup: other clause classes and Z strings (rare).
+// -v where bit 0 of `odd` is set
+__device__ __forceinline__ float negate_if(float v, uint32_t odd) { return __uint_as_float(__float_as_uint(v) ^ (odd << 31)); }
+__device__ __forceinline__ double negate_if(double v, uint32_t odd) {
+  return __hiloint2double((int)((uint32_t)__double2hiint(v) ^ (odd << 31)), __double2loint(v));
+}
+// Diagonal parts beside the table lookup, for the consecutive indices of a slot: other clause classes and
+// Z strings, each taken once for both.  (One amplitude at a time, masks read from memory, 120 strings made a step
+// at n = 20 take 265 us; two layout passes took 100.)
 template <typename R>
-__device__ __noinline__ R other_diagonal(const DevTables* tab, const RScal<R>& sc, const R* zc, int tcls, int code,
-                                         uint32_t z) {
-  R d = (R)0;
+struct RSlot {
+  R d[RT<R>::H];
+};
+template <typename R>
+__device__ __noinline__ RSlot<R> other_diagonal(const DevTables* tab, const RScal<R>& sc, const R* zc, const uint32_t* zm,
+                                                int tcls, int code0, int code1, uint32_t z) {
+  constexpr int H = RT<R>::H;
+  RSlot<R> r;
+#pragma unroll
+  for (int q = 0; q < H; q++) r.d[q] = (R)0;
   for (int cc = 0; cc < tab->n_classes; cc++) {
     if (cc == tcls) continue;
     const DevClass cl = tab->classes[cc];
-    const int cnt = (cl.derived && tcls >= 0) ? code - count_clauses(tab, cl.pen, cl.dbegin, cl.dend, z)
-                                              : count_clauses(tab, cl.pen, cl.begin, cl.end, z);
-    d = fma_(sc.cw[cc], (R)cnt, d);
+    const bool derived = cl.derived && tcls >= 0;
+    const int b = derived ? cl.dbegin : cl.begin, e = derived ? cl.dend : cl.end;
+#pragma unroll
+    for (int q = 0; q < H; q++) {
+      const int cnt = count_clauses(tab, cl.pen, b, e, z + (uint32_t)q);
+      r.d[q] = fma_(sc.cw[cc], (R)(derived ? (q ? code1 : code0) - cnt : cnt), r.d[q]);
+    }
   }
-  for (int m = 0; m < tab->n_z; m++) d += (__popc(tab->z[m].zm & z) & 1) ? -zc[m] : zc[m];
-  return d;
+  const int nz = tab->n_z;
+#pragma unroll 4
+  for (int m = 0; m < nz; m++) {
+    const uint32_t x = zm[m];
+    const R c = negate_if(zc[m], (uint32_t)__popc(x & z));
+    r.d[0] += c;
+    if (H == 2) r.d[H - 1] += negate_if(c, x);
+  }
+  return r;
 }
 
 // All threads of the CTA, from the loop of any role.
@@ -351,6 +377,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
   RPlain<R>* const s_pl = reinterpret_cast<RPlain<R>*>(smem + M.pl);
   RGen<R>* const s_gen = reinterpret_cast<RGen<R>*>(smem + M.gen);
   R* const s_z = reinterpret_cast<R*>(smem + M.z);
+  uint32_t* const s_zm = reinterpret_cast<uint32_t*>(smem + M.zm);
   RScal<R>* const s_sc = reinterpret_cast<RScal<R>*>(smem + M.scal);
   RED* const s_red = reinterpret_cast<RED*>(smem + M.red);           // [parity][nth]
   double* const s_lane = reinterpret_cast<double*>(smem + M.lane);  // [E + 1][8]
@@ -366,6 +393,7 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
   }
   for (int k = tid; k <= nd; k += blockDim.x) s_part[k] = P.rt->part[k];
   for (int k = tid; k < P.nruns; k += blockDim.x) s_run[k] = P.rt->run[k];
+  for (int k = tid; k < nz; k += blockDim.x) s_zm[k] = tab->z[k].zm;
   for (int k = tid; k < 3 * E; k += blockDim.x)
     s_w[k] = P.wdev ? P.wdev[(size_t)P.wstride * (k / 3) + k % 3] : P.w[k];
   __syncthreads();
@@ -685,18 +713,30 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
         if (act) runs_to(tiles, s_part[0].run_end);
         // what does not need the partners, while their tiles are on their way (owned vectors in
         // registers): the diagonal and the past's part of the corrector and the predictor
-        auto diagonal = [&](uint32_t j, int q) {
-          const int code = tcls >= 0 ? s_code[j + q] : 0;
-          R d = sc.dt[code];
-          if (others) d += other_diagonal<R>(tab, sc, s_z + par * nz, tcls, code, zb + j + q);
-          return d;
+        auto diagonal = [&](uint32_t j, R (&d)[H]) {  // of one slot
+          int code[2] = {0, 0};
+#pragma unroll
+          for (int q = 0; q < H; q++) {
+            if (tcls >= 0) code[q] = s_code[j + q];
+            d[q] = sc.dt[code[q]];
+          }
+          if (others) {
+            const RSlot<R> o = other_diagonal<R>(tab, sc, s_z + par * nz, s_zm, tcls, code[0], code[1], zb + j);
+#pragma unroll
+            for (int q = 0; q < H; q++) d[q] += o.d[q];
+          }
         };
         C2 cb[REG ? A : 1], pb[REG ? A : 1];
         R dg[REG ? A : 1];
         if (REG && act)
 #pragma unroll
           for (int g = 0; g < A; g++) {
-            dg[REG ? g : 0] = diagonal((uint32_t)(j0 + (g / H) * js), g % H);
+            if (g % H == 0) {
+              R d[H];
+              diagonal((uint32_t)(j0 + (g / H) * js), d);
+#pragma unroll
+              for (int q = 0; q < H; q++) dg[REG ? g + q : 0] = d[q];
+            }
             if (kind == 0 || kind == 5) past(o[REG ? g / H : 0], g % H, kind, cb[REG ? g : 0], pb[REG ? g : 0]);
           }
         if (nd > 0 && !ring) {  // every partner in one go: the places name the buffers
@@ -760,11 +800,13 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
           if (!act) continue;
           const uint32_t j = (uint32_t)(j0 + s * js), z0 = zb + j;
           C2 own[H], nx[H];
+          R ds[H];
           load(xs_e + j, own);
+          if (!REG) diagonal(j, ds);
 #pragma unroll
           for (int q = 0; q < H; q++) {
             R re = ar[s * H + q], im = ai[s * H + q];
-            const R d = REG ? dg[REG ? s * H + q : 0] : diagonal(j, q);
+            const R d = REG ? dg[REG ? s * H + q : 0] : ds[q];
             if (d != (R)0) {  // an infinite amplitude must not make NaN of an H without diagonal
               re = fma_(d, own[q].x, re);
               im = fma_(d, own[q].y, im);
