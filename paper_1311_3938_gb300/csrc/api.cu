@@ -2894,6 +2894,7 @@ int aqc_batch_remove(aqc_batch* b, int slot) {
     BCUDA(b, cudaMemcpyAsync(&fault, c->d_slots + kSlotFault, sizeof(double), cudaMemcpyDeviceToHost, b->stream));
     BCUDA(b, cudaStreamSynchronize(b->stream));
     timed_out = fault != 0.0;
+    c->short_ring = true;  // owned vectors in registers: f_{n-3} was not written
     // the exchange vectors may have traded places
     c->vec[V_P] = I.vec[kVecP];
     c->vec[V_Q] = I.vec[kVecQ];
