@@ -340,7 +340,8 @@ int aqc_energy(aqc_ctx *ctx, int group_mask, double t, double *out);
 int aqc_norm2(aqc_ctx *ctx, double *out);
 
 /* out = H(t) psi for caller-owned device vectors psi, out (state precision, 2^n amplitudes,
- * distinct, not inside the workspace).  Uses the workspace vector q as scratch, so it
+ * distinct, 16-byte aligned (AQC_E_INVAL otherwise; AQC_C64 states of at most 6 qubits take any out),
+ * not inside the workspace).  Uses the workspace vector q as scratch, so it
  * must not overlap a propagation of the same context (same stream ordering suffices).
  * This is the stand-alone SQH matvec of Sec. I.A. */
 int aqc_hpsi(aqc_ctx *ctx, double t, const void *psi, void *out);

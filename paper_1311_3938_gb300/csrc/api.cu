@@ -1133,6 +1133,8 @@ int resident_steps(aqc_ctx* c, int n_rk, bool hist, int n_pec) {
   return AQC_OK;
 }
 
+bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
+
 // One evaluation of H(t) src over all layouts.  The strided layouts run first as partial sums
 // (the first one also adds the products no layout holds); the contiguous layout 0 runs last
 // with the mode epilogue, so the kernel touching the most vectors has the smallest page
@@ -1140,7 +1142,7 @@ int resident_steps(aqc_ctx* c, int n_rk, bool hist, int n_pec) {
 // With top >= 0, only the partial passes of layouts top .. 1 run (the first of them adds the
 // products no layout holds); the caller finishes the evaluation.
 int evaluate(aqc_ctx* c, const double w[3], const void* src, ApplyParams fin, void* partial_out, int top = -1) {
-  if (top < 0 && resident_on(c) && (fin.mode == MODE_PARTIAL || fin.mode == MODE_ENERGY))
+  if (top < 0 && resident_on(c) && (fin.mode == MODE_ENERGY || (fin.mode == MODE_PARTIAL && aligned16(partial_out))))
     return resident_single(c, w, src, fin.mode == MODE_PARTIAL ? partial_out : nullptr);
   c->q_ready = -1;  // the passes below overwrite q
   const int nl = (int)c->layouts.size();
@@ -2684,6 +2686,9 @@ int aqc_hpsi(aqc_ctx* ctx, double t, const void* psi, void* out) {
     int rc = build_tables(ctx);
     if (rc) return rc;
   }
+  // vectors are read and written 16 bytes at a time (complex64 up to 6 qubits: out one amplitude)
+  if ((!ctx->permuted && !aligned16(psi)) || (!aligned16(out) && !(ctx->prec == AQC_C64 && ctx->n <= 6)))
+    FAIL(ctx, AQC_E_INVAL, "psi and out must be 16-byte aligned");
   double w[3];
   sched_weights(ctx, t, w);
   ApplyParams fin = base_params(ctx);
