@@ -11,7 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libaqc.so")
 SOURCES = ["api.cu", "kernels.cu", "xpartial.cu", "resident.cu", "lanczos.cu", "noalloc.cu"]
-HEADERS = ["aqc_internal.h", os.path.join("..", "..", "include", "aqc.h")]
+HEADERS = ["aqc_internal.h", "kernel_shape.h", os.path.join("..", "..", "include", "aqc.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # host code without contracted multiply-adds: its FP64 arithmetic (step times, schedule
 # weights, segment plans) rounds the same on x86 and Arm, each operation rounded on its own

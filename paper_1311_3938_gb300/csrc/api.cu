@@ -129,6 +129,7 @@ struct ResPlan {
   int t = 0, nth = 0, slots = 0;         // tile bits, threads that own amplitudes, slots per thread
   int np = 0, ng = 0, npart = 0, nbuf = 0, nruns = 0;  // as in ResParams
   int ncode = 0;
+  int cluster[3] = {-1, -1, -1};         // launch_resident_cluster's answers
 };
 
 struct aqc_ctx {
@@ -909,16 +910,14 @@ int64_t rule_steps(const aqc_ctx* c) {
 
 // The driver's tensor-map encoder, looked up once through the runtime (no link to libcuda).
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
+  static const PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-  }
+      return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+    return nullptr;
+  }();
   return fn;
 }
 
@@ -1011,7 +1010,8 @@ bool tile_x_pass(const aqc_ctx* c, const ApplyParams& p, XParams* x) {
   x->top_bits = remote ? c->n - p.L.h - p.L.w : 0;
   for (int g = 0; g < 3; g++) x->w[g] = p.w[g];
   x->wdev = p.wdev;
-  x->max_grid = c->grid_limit;
+  // one CTA per multiprocessor (two tiles fill its shared memory)
+  x->max_grid = c->grid_limit > 0 ? std::min(c->grid_limit, c->sms) : c->sms;
   x->h = p.h;
   x->dcode = p.with_diag ? p.dcode : nullptr;
   x->src = p.src;
@@ -1064,7 +1064,7 @@ int launch_resident_on(aqc_ctx* c, const ResParams& p) {
     ResParams q = p;
     q.nbuf = 2 * p.npart + 1;  // the partners' tiles twice, the own one once more
     if (resident_smem_bytes(c->prec, p.t, q.nbuf, p.np, p.ng, c->n_z, c->res.nth, true) <= kResSmem) {
-      const cudaError_t e = launch_resident_cluster(c->prec, q, c->res.nth, c->n_z, c->stream);
+      const cudaError_t e = launch_resident_cluster(c->prec, q, c->res.nth, c->n_z, c->res.cluster, c->stream);
       if (e == cudaSuccess) {
         c->launches++;
         return AQC_OK;

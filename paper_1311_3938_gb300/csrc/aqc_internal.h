@@ -205,7 +205,7 @@ struct XParams {
   int top_bits;          // > 0: visit tiles that differ in this many top index bits side by side
   double w[3];
   const double* wdev;    // nullable: weights from device memory (as ApplyParams::wdev)
-  int max_grid;          // > 0: at most this many CTAs
+  int max_grid;          // at most this many CTAs (the multiprocessors, or fewer)
   double h;
   const uint8_t* dcode;  // nullable
   const void* src;
@@ -403,7 +403,9 @@ cudaError_t launch_resident(int prec, const ResParams& p, int slots, int nth, in
 // beside the first); evaluation e works on set cluster_set(e)
 constexpr int kResMaxCluster = 16;
 __host__ __device__ constexpr int cluster_set(int e) { return e & 1; }
-cudaError_t launch_resident_cluster(int prec, const ResParams& p, int nth, int n_z, cudaStream_t s);
+// fits: whether the device holds such a cluster, by kernel (start-up, steps, compensated steps); -1 not
+// asked yet, filled in; cudaErrorNotSupported where it does not
+cudaError_t launch_resident_cluster(int prec, const ResParams& p, int nth, int n_z, int (&fits)[3], cudaStream_t s);
 cudaError_t launch_resident_batch(int prec, const ResBatch& b, int slots, int ctas, size_t smem, cudaStream_t s);
 int64_t fma64_count(int blocks, int iters);
 int reduce_grid(uint64_t N);

@@ -21,6 +21,7 @@
 #include <type_traits>
 
 #include "aqc_internal.h"
+#include "kernel_shape.h"
 
 namespace cg = cooperative_groups;
 
@@ -1478,18 +1479,11 @@ size_t apply_smem_bytes(int prec, int t, int n_plain, int n_general, int n_z) {
 // for cluster layouts, the number of clusters that can be resident at once (x cluster size).
 template <typename R, int MODE, bool CL, bool COMP, bool TURN>
 static cudaError_t grid_for(uint32_t ntiles, int smem, cudaStream_t s, int* grid) {
-  static int configured = 0, cached_smem = -1, cached_dev = -1, cached_g = 0;
+  static KernelShape shape;
   auto kern = k_apply<R, MODE, CL, COMP, TURN>;
-  if (smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    configured = smem;
-  }
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (!(dev == cached_dev && smem == cached_smem)) {
-    int g = 0;
+  int full = 0;
+  cudaError_t e = shape.grid(kern, smem, [&](int dev, int* g) {
+    cudaError_t e = cudaSuccess;
     if (CL) {
       cudaLaunchConfig_t cfg = {};
       cudaLaunchAttribute attr[1];
@@ -1505,20 +1499,17 @@ static cudaError_t grid_for(uint32_t ntiles, int smem, cudaStream_t s, int* grid
       cfg.numAttrs = 1;
       int nclusters = 0;
       e = cudaOccupancyMaxActiveClusters(&nclusters, kern, &cfg);
-      if (e != cudaSuccess) return e;
-      g = (nclusters < 1 ? 1 : nclusters) << kClusterBits;
+      *g = (nclusters < 1 ? 1 : nclusters) << kClusterBits;
     } else {
       int sms = 0, per = 0;
       e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
       if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kThreads, smem);
-      if (e != cudaSuccess) return e;
-      g = sms * (per < 1 ? 1 : per);
+      *g = sms * (per < 1 ? 1 : per);
     }
-    cached_dev = dev;
-    cached_smem = smem;
-    cached_g = g;
-  }
-  uint64_t g = (uint64_t)cached_g;
+    return e;
+  }, &full);
+  if (e != cudaSuccess) return e;
+  uint64_t g = (uint64_t)full;
   if (g > (uint64_t)kMaxApplyGrid) g = kMaxApplyGrid;
   if (CL) {
     const uint64_t tiles_ctas = (uint64_t)ntiles << kClusterBits;
@@ -1608,26 +1599,18 @@ size_t table_smem_bytes(int prec, int t, int n_plain, int n_general, int n_z) {
 
 template <typename R>
 static cudaError_t launch_slab_t(const SlabParams& p, int smem, cudaStream_t s) {
-  static int configured = 0, cached_smem = -1, cached_dev = -1, cached_g = 0;
+  static KernelShape shape;
   auto kern = k_slab<R>;
-  if (smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    configured = smem;
-  }
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (!(dev == cached_dev && smem == cached_smem)) {
+  int g = 0;
+  const cudaError_t e = shape.grid(kern, smem, [&](int dev, int* full) {
     int sms = 0, per = 0;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kThreads, smem);
-    if (e != cudaSuccess) return e;
-    cached_dev = dev;
-    cached_smem = smem;
-    cached_g = sms * (per < 1 ? 1 : per);
-  }
-  int g = cached_g > kMaxApplyGrid ? kMaxApplyGrid : cached_g;
+    *full = sms * (per < 1 ? 1 : per);
+    return e;
+  }, &g);
+  if (e != cudaSuccess) return e;
+  if (g > kMaxApplyGrid) g = kMaxApplyGrid;
   if ((uint32_t)g > p.n_items) g = (int)p.n_items;
   kern<<<g, kThreads, smem, s>>>(p);
   return cudaGetLastError();
@@ -1642,12 +1625,9 @@ cudaError_t launch_slab(int prec, const SlabParams& p, int smem, cudaStream_t s)
 
 template <typename R, int NT>
 static cudaError_t launch_batch_t(const BatchLaunch& b, int nitems, int smem, cudaStream_t s) {
-  static int configured = 0;
-  if (smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_batch<R, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    configured = smem;
-  }
+  static KernelShape shape;
+  const cudaError_t e = shape.allow(k_batch<R, NT>, smem);
+  if (e != cudaSuccess) return e;
   k_batch<R, NT><<<nitems, NT, smem, s>>>(b);
   return cudaGetLastError();
 }

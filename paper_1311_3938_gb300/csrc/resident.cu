@@ -45,6 +45,7 @@
 #include <type_traits>
 
 #include "aqc_internal.h"
+#include "kernel_shape.h"
 
 namespace aqc {
 
@@ -713,11 +714,12 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
         if (act) runs_to(tiles, s_part[0].run_end);
         // what does not need the partners, while their tiles are on their way (owned vectors in
         // registers): the diagonal and the past's part of the corrector and the predictor
-        auto diagonal = [&](uint32_t j, R (&d)[H]) {  // of one slot
+        auto code_at = [&](uint32_t j) { return tcls >= 0 ? (int)s_code[j] : 0; };
+        auto diagonal = [&](uint32_t j, R (&d)[H]) {  // of the slot at j
           int code[2] = {0, 0};
 #pragma unroll
           for (int q = 0; q < H; q++) {
-            if (tcls >= 0) code[q] = s_code[j + q];
+            code[q] = code_at(j + q);
             d[q] = sc.dt[code[q]];
           }
           if (others) {
@@ -1124,12 +1126,9 @@ template <typename R, int S, bool REG, bool PEC, bool COMP>
 cudaError_t launch_t(const ResParams& p, int nth, int max_grid, int n_z, cudaStream_t s) {
   const size_t smem = ResSmem<R>(1u << p.t, p.nbuf, p.np, p.ng, n_z, nth, !REG).total;
   auto kern = k_resident<R, S, REG, PEC, COMP>;
-  static int configured = 0;
-  if ((int)smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = (int)smem;
-  }
+  static KernelShape shape;
+  cudaError_t e = shape.allow(kern, smem);
+  if (e != cudaSuccess) return e;
   int grid = 1 << (p.n - p.t);
   if (grid > max_grid) grid = max_grid;
   cudaLaunchConfig_t cfg = {};
@@ -1142,7 +1141,7 @@ cudaError_t launch_t(const ResParams& p, int nth, int max_grid, int n_z, cudaStr
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = p.evals > 1 && grid > 1 ? 1 : 0;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, p);
+  e = cudaLaunchKernelEx(&cfg, kern, p);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -1155,16 +1154,12 @@ cudaError_t launch_c(const ResParams& p, int nth, int max_grid, int n_z, cudaStr
 
 // One cluster of 2^(n - t) CTAs.  p.nbuf: two sets of partner buffers.
 template <typename R, bool PEC, bool COMP>
-cudaError_t launch_cluster_t(const ResParams& p, int nth, int n_z, cudaStream_t s) {
+cudaError_t launch_cluster_t(const ResParams& p, int nth, int n_z, int* fits, cudaStream_t s) {
   const size_t smem = ResSmem<R>(1u << p.t, p.nbuf, p.np, p.ng, n_z, nth, false).total;
   auto kern = k_resident_cluster<R, PEC, COMP>;
-  static int configured = 0;
-  if ((int)smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    configured = (int)smem;
-  }
+  static KernelShape shape;
+  cudaError_t e = shape.allow(kern, smem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1176,22 +1171,23 @@ cudaError_t launch_cluster_t(const ResParams& p, int nth, int n_z, cudaStream_t 
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  static int known[3] = {-1, -1, -1}, fits = 0;  // whether the device holds such a cluster
-  const int shape[3] = {(int)cfg.gridDim.x, nth, (int)smem};
-  if (shape[0] != known[0] || shape[1] != known[1] || shape[2] != known[2]) {
-    cudaError_t q = cudaOccupancyMaxActiveClusters(&fits, kern, &cfg);
-    if (q != cudaSuccess) return q;
-    for (int i = 0; i < 3; i++) known[i] = shape[i];
+  if (*fits < 0) {
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    int clusters = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
+    if (e != cudaSuccess) return e;
+    *fits = clusters > 0 ? 1 : 0;
   }
-  if (fits < 1) return cudaErrorNotSupported;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, p);
+  if (*fits == 0) return cudaErrorNotSupported;
+  e = cudaLaunchKernelEx(&cfg, kern, p);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <typename R>
-cudaError_t launch_cluster_r(const ResParams& p, int nth, int n_z, cudaStream_t s) {
-  if (p.n_pec == 0) return launch_cluster_t<R, false, false>(p, nth, n_z, s);
-  return p.ylo ? launch_cluster_t<R, true, sizeof(R) == 4>(p, nth, n_z, s) : launch_cluster_t<R, true, false>(p, nth, n_z, s);
+cudaError_t launch_cluster_r(const ResParams& p, int nth, int n_z, int* fits, cudaStream_t s) {
+  if (p.n_pec == 0) return launch_cluster_t<R, false, false>(p, nth, n_z, fits, s);
+  return p.ylo ? launch_cluster_t<R, true, sizeof(R) == 4>(p, nth, n_z, fits + 2, s)
+               : launch_cluster_t<R, true, false>(p, nth, n_z, fits + 1, s);
 }
 
 template <typename R>
@@ -1217,12 +1213,9 @@ size_t resident_smem_bytes(int prec, int t, int nbuf, int np, int ng, int n_z, i
 template <typename R, int S>
 static cudaError_t launch_batch_s(const ResBatch& b, int ctas, size_t smem, cudaStream_t s) {
   auto kern = k_resident_batch<R, S>;
-  static int configured = 0;
-  if ((int)smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = (int)smem;
-  }
+  static KernelShape shape;
+  cudaError_t e = shape.allow(kern, smem);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -1233,7 +1226,7 @@ static cudaError_t launch_batch_s(const ResBatch& b, int ctas, size_t smem, cuda
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, kern, b);
+  e = cudaLaunchKernelEx(&cfg, kern, b);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -1256,8 +1249,8 @@ cudaError_t launch_resident(int prec, const ResParams& p, int slots, int nth, in
   return prec == 0 ? launch_r<double>(p, slots, nth, max_grid, n_z, s) : launch_r<float>(p, slots, nth, max_grid, n_z, s);
 }
 
-cudaError_t launch_resident_cluster(int prec, const ResParams& p, int nth, int n_z, cudaStream_t s) {
-  return prec == 0 ? launch_cluster_r<double>(p, nth, n_z, s) : launch_cluster_r<float>(p, nth, n_z, s);
+cudaError_t launch_resident_cluster(int prec, const ResParams& p, int nth, int n_z, int (&fits)[3], cudaStream_t s) {
+  return prec == 0 ? launch_cluster_r<double>(p, nth, n_z, fits, s) : launch_cluster_r<float>(p, nth, n_z, fits, s);
 }
 
 }  // namespace aqc

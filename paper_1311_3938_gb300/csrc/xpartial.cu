@@ -35,6 +35,7 @@
 #include <type_traits>
 
 #include "aqc_internal.h"
+#include "kernel_shape.h"
 
 namespace aqc {
 
@@ -633,25 +634,10 @@ template <int MODE, bool DIAG, bool FAR = false, bool OTHERS = false>
 cudaError_t launch_x(const XParams& p, int n_flips, int n_z, cudaStream_t s) {
   const size_t smem = XSmem(n_flips, n_z, DIAG && p.dcode).total;
   auto kern = k_tile_x<MODE, DIAG, FAR, OTHERS>;
-  static int configured = 0, cached_dev = -1, cached_g = 0;
-  if ((int)smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = (int)smem;
-  }
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static KernelShape shape;
+  const cudaError_t e = shape.allow(kern, smem);
   if (e != cudaSuccess) return e;
-  if (dev != cached_dev) {  // one CTA per multiprocessor (two tiles fill its shared memory)
-    int sms = 0;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-    cached_dev = dev;
-    cached_g = sms;
-  }
-  int g = cached_g;
-  if (p.max_grid > 0 && g > p.max_grid) g = p.max_grid;
-  if ((uint32_t)g > p.ntiles) g = (int)p.ntiles;
+  const int g = (uint32_t)p.max_grid > p.ntiles ? (int)p.ntiles : p.max_grid;
   kern<<<g, kXThreads, smem, s>>>(p);
   return cudaGetLastError();
 }
