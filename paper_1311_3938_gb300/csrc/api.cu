@@ -611,10 +611,23 @@ void plan_resident(aqc_ctx* c) {
     R.t = c->n <= 10 ? 6 : std::max(7, c->n - 7);
   else
     R.t = c->n <= 13 ? std::max(8, c->n - 4) : std::max(8, c->n - 7);
-  const int slots_all = std::max(1, (1 << R.t) / H);
-  R.nth = resident_threads(slots_all);
-  R.slots = std::max(1, slots_all / R.nth);
-  R.on = resident_tables(c, R, &c->h_res.alone, kResSmem);
+  auto fit = [&](int t) {
+    R.t = t;
+    const int slots_all = std::max(1, (1 << t) / H);
+    R.nth = resident_threads(slots_all);
+    R.slots = std::max(1, slots_all / R.nth);
+    return resident_tables(c, R, &c->h_res.alone, kResSmem);
+  };
+  const int t0 = R.t, most = std::min(c->n, c128 ? std::max(t0, 9) : 13);
+  // A limit on the CTAs: tiles so large that each is one CTA's again, or the largest ones (complex128, bound by
+  // FP64 whatever the tile: 2^9), since a visit of a tile costs an exchange.  Nonlinear path, microseconds
+  // per step with the tiles above / with these: complex64 n = 12 on 2 CTAs 32 / 7.5, n = 16 on 4 150 / 62, on 16
+  // 40 / 18, n = 19 on 32 107 / 79; complex128 n = 14 on 2 496 / 313, on 8 125 / 80.
+  int tb = t0;
+  if (c->grid_limit > 0)
+    while (tb < most && (1 << (c->n - tb)) > c->grid_limit) tb++;
+  R.on = fit(tb);
+  if (!R.on && tb != t0) R.on = fit(t0);
   c->res = R;
 }
 
@@ -2183,6 +2196,7 @@ int aqc_set_layout_turns(aqc_ctx* ctx, int mode) {
 int aqc_set_grid_limit(aqc_ctx* ctx, int max_ctas) {
   if (!ctx) return AQC_E_INVAL;
   if (max_ctas < 0) FAIL(ctx, AQC_E_INVAL, "max_ctas must be >= 0");
+  if (max_ctas != ctx->grid_limit && resident_size(ctx)) ctx->dirty = true;  // other tiles (plan_resident)
   ctx->grid_limit = max_ctas;
   DeviceGuard dg(ctx->device);
   drop_step_graph(ctx);  // captured launches carry the grid size

@@ -554,12 +554,29 @@ __device__ __forceinline__ void resident_body(const ResParams& P, const uint32_t
         const uint32_t zb = tile << P.t;
         if (e == 0 || multi) {  // the own tile and its clause bytes (then kept up to date in place)
           if (multi) cta_sync();  // readers of the previous tile are done
-          for (uint32_t j = j0; j < tsize; j += js)
-            *reinterpret_cast<float4*>(xs + j) = __ldcg(reinterpret_cast<const float4*>(xin + zb + j));
-          if (tcls >= 0)
+          if (REG) {
             for (uint32_t j = j0; j < tsize; j += js)
+              *reinterpret_cast<float4*>(xs + j) = __ldcg(reinterpret_cast<const float4*>(xin + zb + j));
+            if (tcls >= 0)
+              for (uint32_t j = j0; j < tsize; j += js)
 #pragma unroll
-              for (int q = 0; q < H; q++) s_code[j + q] = P.dcode[zb + j + q];
+                for (int q = 0; q < H; q++) s_code[j + q] = P.dcode[zb + j + q];
+          } else if (act) {  // on every visit: all loads at once
+            float4 v[REG ? 1 : S];
+#pragma unroll
+            for (int s = 0; s < S; s++) v[REG ? 0 : s] = __ldcg(reinterpret_cast<const float4*>(xin + zb + (uint32_t)(j0 + s * js)));
+            if (tcls >= 0) {
+              if (tsize >= 16u) {
+                for (uint32_t j = 16u * tid; j < tsize; j += 16u * nth)
+                  *reinterpret_cast<float4*>(s_code + j) = __ldg(reinterpret_cast<const float4*>(P.dcode + zb + j));
+              } else {
+#pragma unroll
+                for (int q = 0; q < H; q++) s_code[j0 + q] = P.dcode[zb + (uint32_t)j0 + q];
+              }
+            }
+#pragma unroll
+            for (int s = 0; s < S; s++) *reinterpret_cast<float4*>(xs + (j0 + s * js)) = v[REG ? 0 : s];
+          }
           cta_sync();
         }
         R ar[A], ai[A];
