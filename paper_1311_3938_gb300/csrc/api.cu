@@ -759,8 +759,9 @@ int build_tables(aqc_ctx* c) {
     } else {
       for (const DevFlip& f : per[l]) t->flips[pos + k++] = f;
     }
-    // 4: below that the conversion costs more than the products; 16: the bits left for the sum
-    if (l < nl && c->prec == AQC_C128 && np >= 4 && np <= 16 && (int)per[l].size() == np) {
+    // 4: below that the conversion costs more than the products, as it does up to 8 qubits (matvec 8.4
+    // against 6.5 us); 16: the bits left for the sum
+    if (l < nl && c->prec == AQC_C128 && c->n > 8 && np >= 4 && np <= 16 && (int)per[l].size() == np) {
       bool same = true;
       for (int i = 1; i < np; i++)
         same = same && t->flips[pos + i].coef == t->flips[pos].coef && t->flips[pos + i].group == t->flips[pos].group;
@@ -1148,6 +1149,17 @@ int resident_steps(aqc_ctx* c, int n_rk, bool hist, int n_pec) {
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 
+// Whether one evaluation alone (a matvec, an energy) runs as a resident launch: not where its prologue
+// (tables and tile into every CTA) outweighs the exchange that it saves.  Microseconds per call, resident /
+// layout passes, linear and nonlinear path: matvec complex64 n = 9 6.6 / 6.5, 8.4 / 7.1, n = 10 7.3 / 6.5, 8.4 / 8.5,
+// n = 11 8.5 / 8.5, 8.4 / 10.6; complex128 n = 4 6.5 / 6.4, 8.5 / 6.6, n = 8 8.4 / 6.6, 10.5 / 10.1, n = 9 8.5 / 8.4,
+// 10.5 / 12.6; energy (with its read back) complex64 n = 19 39 / 41, 44 / 54, n = 20 53 / 42, 77 / 54.
+bool single_resident(const aqc_ctx* c, const ApplyParams& fin, const void* out) {
+  if (!resident_on(c)) return false;
+  const bool by_size = c->prec == AQC_C128 ? c->n > 8 : c->n < 20 && c->n != 9 && c->n != 10;
+  return by_size && (fin.mode == MODE_ENERGY || (fin.mode == MODE_PARTIAL && aligned16(out)));
+}
+
 // One evaluation of H(t) src over all layouts.  The strided layouts run first as partial sums
 // (the first one also adds the products no layout holds); the contiguous layout 0 runs last
 // with the mode epilogue, so the kernel touching the most vectors has the smallest page
@@ -1155,7 +1167,7 @@ bool aligned16(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 // With top >= 0, only the partial passes of layouts top .. 1 run (the first of them adds the
 // products no layout holds); the caller finishes the evaluation.
 int evaluate(aqc_ctx* c, const double w[3], const void* src, ApplyParams fin, void* partial_out, int top = -1) {
-  if (top < 0 && resident_on(c) && (fin.mode == MODE_ENERGY || (fin.mode == MODE_PARTIAL && aligned16(partial_out))))
+  if (top < 0 && single_resident(c, fin, partial_out))
     return resident_single(c, w, src, fin.mode == MODE_PARTIAL ? partial_out : nullptr);
   c->q_ready = -1;  // the passes below overwrite q
   const int nl = (int)c->layouts.size();
