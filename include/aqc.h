@@ -237,7 +237,8 @@ int aqc_set_slab_bits(aqc_ctx *ctx, int slab_bits);
  * pass order), or a multiple of 4 in [4, 64].  The graph is
  * recaptured when the tables, the step size or the vectors change, and is not used under
  * step-size control, the slab order or a clause-by-clause sequence (those steps run one by
- * one).  Grid steps that remain after the last whole replay run one by one.  AQC_E_INVAL for
+ * one).  Grid steps that remain after the last whole replay run one by one, or in one launch
+ * where the state stays on the GPU.  AQC_E_INVAL for
  * other k_steps; a failed capture returns AQC_E_CUDA from aqc_propagate. */
 int aqc_set_graph_steps(aqc_ctx *ctx, int k_steps);
 

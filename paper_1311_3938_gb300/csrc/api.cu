@@ -86,9 +86,11 @@ std::vector<Layout> layouts_for(int n, int prec, int tile_bits, bool allow_clust
 }
 
 
-// partials of the reductions: two per k_apply CTA, one per k_norm2 CTA, (64 + 1) x 128 of a resident
-// launch; the ResArea lies behind them
+// Partials of the reductions in use at a time, at most: (64 + 1) x 128 of a resident launch (128 tiles),
+// up to three per CTA of a layout pass (its grid: the CTAs that the GPU holds), one per k_norm2 CTA (1216), the
+// coefficients of 4096 Lanczos steps.  The ResArea lies behind them.
 constexpr size_t kResPartials = (kResMaxEvals + 1) * 152;
+static_assert(kResPartials >= (kResMaxEvals + 1) * 128 && kResPartials >= 2 * 4096 && kResPartials >= 3 * 8 * 152, "partials");
 
 struct WsPlan {
   size_t off_tab, off_slots, off_counter, off_sync, off_perm, off_wdev, off_partials, off_dcode, off_vec, vec_bytes, total;
@@ -1748,7 +1750,7 @@ int batch_plan_waves(aqc_batch* b) {
   };
   auto pack = [&](int tb, std::vector<std::vector<Job>>* out) {  // estimated time, or infinity
     double total = 0.0;
-    for (int S = 1; S <= 16; S *= 2) {
+    for (int S : {1, 2, 8, 16}) {  // (resident_threads gives no other)
       std::vector<Job> jobs;
       for (int slot : who) {
         const aqc_ctx* c = b->members[slot];
@@ -2682,7 +2684,7 @@ void tridiag_eigvec(const double* a, const double* b, int k, double lam, double*
 }
 
 struct LzPlan {
-  size_t ld_bytes, off_partials, off_coef, off_h, off_scal, total;
+  size_t ld_bytes, off_partials, off_coef, off_scal, total;
   uint32_t G;
 };
 
@@ -2695,8 +2697,7 @@ LzPlan lanczos_plan(int n, int prec, int max_iter) {
   p.G = lanczos_dot_blocks(N);
   p.off_partials = m * p.ld_bytes;
   p.off_coef = align_up(p.off_partials + m * p.G * 2 * sizeof(double), 256);
-  p.off_h = align_up(p.off_coef + m * 2 * sizeof(double), 256);
-  p.off_scal = align_up(p.off_h + m * 2 * sizeof(double), 256);
+  p.off_scal = align_up(p.off_coef + m * 2 * sizeof(double), 256);
   p.total = p.off_scal + 256;
   return p;
 }

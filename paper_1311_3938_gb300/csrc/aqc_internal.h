@@ -226,7 +226,7 @@ struct XParams {
 // A resident launch (kernel k_resident): a sequence of evaluations of one state whose tiles, one
 // per CTA, are all on the GPU at once.  n_rk Runge-Kutta steps, then (hist) the start of the
 // derivative history, or n_pec predictor-corrector steps; or one evaluation alone (single).
-constexpr int kResMaxThreads = 512;  // threads that own amplitudes (one more warp does scalar work)
+constexpr int kResMaxThreads = 512;  // threads that own amplitudes (four service warps beside them)
 constexpr int kResMaxEvals = 64;
 constexpr int kResFlagStride = 8;   // 32 bytes between tile flags: polls of one do not slow another
 struct ResParams {

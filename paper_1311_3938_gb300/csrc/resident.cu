@@ -32,12 +32,14 @@
 //
 // Measured, microseconds per predictor-corrector step (before: one launch per layout pass, replayed
 // from a graph, each on as many CTAs as the state has 64 KiB tiles):
-//   complex64, nonlinear path: n = 8 11 -> 1.8, n = 12 31 -> 2.4, n = 16 43 -> 4.3, n = 18 46 -> 8.8, n = 20 50 -> 36
+//   complex64, nonlinear path: n = 8 11 -> 1.8, n = 12 31 -> 2.4, n = 16 43 -> 4.2, n = 18 46 -> 8.5, n = 20 50 -> 35
 //   complex128, linear path:   n = 10 20 -> 3.6, n = 14 68 -> 4.9, n = 16 71 -> 11, n = 18 72 -> 42
 // An exchange takes about 0.8 us in a cluster and 1.5 us through memory (from the last store to the
 // first partner read); the rest of a small state's step is dependent shared-memory reads and, in
-// complex128, FP64 latency.  Above n = 14 complex64 is bound by the shared-memory reads of the
-// partners (16 bytes per product and slot), complex128 by the FP64 pipe.
+// complex128, FP64 latency.  Counters: n = 12 complex64 waits (issue slots 25% busy on 16 multiprocessors,
+// barriers the first stall); n = 20 keeps shared memory's pipe 46% busy with the partners' reads (16
+// bytes per product and slot) and issue slots 42%, the rest is barriers between its phases, with one CTA
+// per multiprocessor; complex128 n = 16 keeps the FP64 pipe 81% busy.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>

@@ -25,8 +25,9 @@
 //
 // Measured (GB300): every pass of 28 qubits runs at the copy rate of 6.7 TB/s: partial passes 0.65 and
 // 0.90 ms, the step 2.59 ms (17.4 GB; as k_apply with y in memory 2.83 ms); at 23 qubits the step
-// 112 -> 96 us, the XY step of 24 qubits (78 hops) 486 -> 389 us, the last pass of H psi at 26 qubits
-// 403 -> 289 us, the XY pass with products that no layout holds 178 -> 98 us.
+// 112 -> 96 us, the XY step of 24 qubits (78 hops, the catalyst's class) 486 -> 281 us, the last pass of
+// H psi at 26 qubits 403 -> 289 us, the XY pass with products that no layout holds 178 -> 98 us (three
+// layouts; 260 us where it stands for two of them).
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -150,8 +151,9 @@ __device__ __forceinline__ void reg_flip_swap(float c, const float4 (&own)[8], f
 // four is an offset of its first address; with no register bit all eight or none; with two of the
 // thread's own bits (two register bits, or one and the pair bit) nothing from shared memory.  Only the
 // pair bit beside a lane's or a warp's bit reads both amplitudes of every pair for one of them (8-byte
-// loads at this stride conflict two ways).  XY path, n = 24, 32 steps and start-up: 24.0 -> 23.6 ms; the
-// step pass then keeps shared memory's pipe 27% busy and issue slots 46% (65% while it forms products).
+// loads at this stride conflict two ways).  XY path, n = 24, 32 steps and start-up: 24.0 -> 23.6 ms (22
+// since the diagonal takes classes once per thread); the step pass keeps shared memory's pipe 46% busy
+// and issue slots 42%, the one before it issue slots 51%.
 // cA is the coefficient at the parity of the thread's first amplitude, cB at the opposite one.
 __device__ __forceinline__ void hop_pair(float c0, float c1, const float4& g, float4& a) {
   a.x = fmaf(c0, g.x, a.x);
