@@ -604,28 +604,27 @@ __device__ __forceinline__ void process_tile(const TileCtx<R>& T, uint32_t zb, u
   double us[2] = {0.0, 0.0};  // coefficient times the value of a unit, real and imaginary parts
   if constexpr (sizeof(R) == 8 && !CL) {
     if (uni) {
-      uint32_t* const s_max = reinterpret_cast<uint32_t*>(T.s_red);
+      uint2* const s_max = reinterpret_cast<uint2*>(T.s_red);
       const uint32_t nw = blockDim.x >> 5, rows = tsize >> 5;
-      uint32_t m[2] = {0u, 0u};
       const bool any = threadIdx.x < tsize;
       const C2 mine = any ? s_p[threadIdx.x] : zero2;
+      uint32_t m[2] = {(uint32_t)__double2hiint(mine.x) & 0x7fffffffu, (uint32_t)__double2hiint(mine.y) & 0x7fffffffu};
 #pragma unroll 8
-      for (uint32_t j = threadIdx.x; j < tsize; j += blockDim.x) {
+      for (uint32_t j = threadIdx.x + blockDim.x; j < tsize; j += blockDim.x) {
         const C2 v = s_p[j];
         m[0] = max(m[0], (uint32_t)__double2hiint(v.x) & 0x7fffffffu);
         m[1] = max(m[1], (uint32_t)__double2hiint(v.y) & 0x7fffffffu);
       }
-#pragma unroll
-      for (int k = 0; k < 2; k++) {
-        m[k] = __reduce_max_sync(0xffffffffu, m[k]);
-        if ((threadIdx.x & 31u) == 0u) s_max[2u * (threadIdx.x >> 5) + k] = m[k];
-      }
+      for (int k = 0; k < 2; k++) m[k] = __reduce_max_sync(0xffffffffu, m[k]);
+      if ((threadIdx.x & 31u) == 0u) s_max[threadIdx.x >> 5] = make_uint2(m[0], m[1]);
       __syncthreads();
+      const uint2 other = s_max[min(threadIdx.x & 31u, nw - 1u)];  // of one warp per lane
+      m[0] = other.x;
+      m[1] = other.y;
       int emax[2];
 #pragma unroll
       for (int k = 0; k < 2; k++) {
-        m[k] = 0;
-        for (uint32_t w = 0; w < nw; w++) m[k] = max(m[k], s_max[2u * w + k]);
+        m[k] = __reduce_max_sync(0xffffffffu, m[k]);
         // tiles with infinities or NaN, and tiles so small that the scale would be subnormal, keep
         // the FP64 products; a part that is zero throughout takes any scale
         emax[k] = max((int)(m[k] >> 20), 256);
