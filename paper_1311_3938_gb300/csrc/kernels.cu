@@ -124,8 +124,8 @@ __device__ __forceinline__ double from_fixed(int64_t s, int k = 0) {
 // and rounded once, so two FP64 operations are left of eight, and the error is that of the last
 // multiply-add instead of four roundings next to y (rms of y's rounding 4.6e-17, 8.8e-17 with the chain
 // of multiply-adds).  With the integer clause counts and without the norm that nobody reads: 64 grid
-// steps at n = 20 8.2 -> 6.8 ms, 12 at n = 26 114 -> 102 ms (6.9 and 108 with the check of the products'
-// sums above).  The step kernel at n = 22 keeps the FP64 pipe 59% busy, issue slots 39%, memory 29%.
+// steps at n = 20 8.2 -> 6.8 ms, 12 at n = 26 114 -> 102 ms (6.8 and 107 with the check of the products'
+// sums above).  The step kernel at n = 22 keeps the FP64 pipe 58% busy, issue slots 39%, memory 29%.
 __device__ __forceinline__ void pec_fixed(double f, double a, double b, double c, double h24, double& y, double& p) {
   auto top = [](double v) { return (uint32_t)__double2hiint(v) & 0x7fffffffu; };
   const int emax = (int)(max(max(top(f), top(a)), max(top(b), top(c))) >> 20);
